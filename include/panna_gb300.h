@@ -229,10 +229,12 @@ panna_status panna_set_angular_precision(panna_ctx* ctx, int32_t mode);
  * adjoint only 5 = the compensated kernel walking each atom's pairs in diagonal order
  * (k, k + d mod n), whose rounds of min(32, n - 1) pairs touch distinct entries on each side,
  * so the per-entry gradients are summed without atomics in a fixed order (bit-reproducible).
- * With FP32 networks (extended angular terms) the descriptor's candidates are variants 0 and 1
- * only.  Without autotuning, batches of at least 1216 atoms take variant 2 (adjoint: 5; the
- * descriptor with FP32 networks: 0) and smaller ones variant 0
- * (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks): a bit mask of the first layer's
+* Matrix form: descriptor 5 (any descriptor of the modified term): one warp per atom, the products over sectors and shells on the tensor cores from
+ * operands split into TF32 parts; sums in a fixed order.  Where they apply, batches of at least 1216
+ * atoms take them without measuring.  With FP32 networks (extended angular terms) the descriptor's
+ * candidates are variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that
+ * the matrix forms do not take use variant 2 (adjoint: 5; the descriptor with FP32 networks: 0) and
+ * smaller ones variant 0 (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks): a bit mask of the first layer's
  * products (descriptor width to first hidden width, almost all of the networks'
  * arithmetic) that run on the tensor cores with operands split into TF32 parts, the rest
  * staying on the CUDA cores in plain FP32: 1 = forward (three parts), 4 = tangent of the
@@ -248,8 +250,7 @@ panna_status panna_set_tuning(panna_ctx* ctx, const char* knob, int32_t value);
 /* The kernel variant that knob "descriptor", "adjoint" or "jvp" ran with in the last compute
  * call that used it (tuned or forced): 0 blocked, 1 flattened, 2 / 3 / 4 compensated with 32 / 16
  * / 8 lanes per (species block, theta chunk, R chunk) unit (adjoint 4: flattened units), 5
- * (adjoint only) compensated in diagonal pair order; -1 before any such call or for an unknown
- * knob. */
+ * compensated in diagonal pair order (adjoint) or the matrix form (descriptor); -1 before any such call or for an unknown knob. */
 int32_t panna_tuning_choice(const panna_ctx* ctx, const char* knob);
 
 /*

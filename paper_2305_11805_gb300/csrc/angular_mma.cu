@@ -1,0 +1,575 @@
+// Angular descriptor with the products over sectors and shells on the warp-level
+// tensor cores (modified angular term; the forms are those of descriptor.cu).
+//
+// What is different from the one-lane-per-pair kernels.  Per pair of neighbours the angular term
+// is an outer product A (x) e of n_theta sector powers and n_R shell Gaussians.  A lane that owns a
+// pair evaluates 8 + 8 of them, reads the sectors' and shells' constants from shared memory for
+// each, and holds (descriptor) a 64-float tile or reads (adjoint) a 64-float tile per pair.  Here a
+// warp takes its pairs 32 at a time in two steps.  Step 1, a lane per pair: the geometry (half
+// angles, mean distance), left in shared memory.  Step 2, lanes in the layout of the MMA operands:
+// lane (g, t) = (lane / 4, lane mod 4) evaluates sector g and shell g for pairs t, t + 4 of each
+// group of 8, so the sector's and shell's constants stay in its registers, two pairs share every
+// two-wide FP32 instruction, and mma.m16n8k8 contracts over the pairs.  The tile is 4 registers.
+// (The contraction is 8 x 8 x 8 per group of pairs of one atom, far below the 128-row tiles of
+// tcgen05, whose operands would have to pass through shared memory besides.)
+//
+// What bounds it (ncu, water box of 16,384 atoms): instruction issue, two-wide FP32 instructions taking
+// two dispatch cycles each, next to the shared-memory data path.  A round of 32 pairs takes about 214
+// warp instructions (fast descriptor) against 400 in the lane-per-pair kernel; mma.m16n8k8 with TF32
+// operands issues every 8 cycles per scheduler and stays below 20 % busy.  Pair buffers hold what a
+// lane reads as 4-byte words because a load returns at most 128 bytes a cycle to the warp, also when
+// its lanes share addresses.
+//
+// Measured (GB300, before -> after, ms per launch; before: descriptor.cu's compensated or float-pair
+// descriptor and its diagonal-order adjoint):
+//                                            BF16 networks                FP32 networks
+//                                       descriptor     adjoint       descriptor     adjoint
+//   128 ragged boxes (107,202 atoms)   1.03 -> 0.74  1.39 -> 1.20   2.48 -> 1.31  1.66 -> 1.51
+//   water box (16,384 atoms)           0.67 -> 0.59  1.26 -> 0.94   1.89 -> 1.16  1.57 -> 1.26
+//   FCC box (131,072 atoms)            1.66 -> 1.07  2.56 -> 1.66   4.47 -> 2.3   3.13 -> 2.14
+//   1024 molecules (17,396 atoms)      0.14 -> 0.07  0.125 -> 0.117 0.23 -> 0.10  0.145 -> 0.133
+//
+// FP32 accuracy on TF32 operands: every operand is split into hi + lo TF32 parts (hi its leading 11
+// bits, lo the exact rest), so products carry about 22 bits; the descriptor puts A_hi in rows 0..7
+// and A_lo in rows 8..15 of one A operand.  The tensor cores accumulate a round of 32 pairs, which
+// is then added to the block's sum in plain FP32.
+//
+// The eps-regularised angle.  With R = sqrt(1 + eps), (cos, sin_eps) = R (cos th', sin th') exactly,
+// so 1 - y_m = t_m = R sin^2((th' - theta_m)/2) - (R - 1)/2: one angle th' per pair carries eps, and
+// sin, cos of (th' - theta_m)/2 come from the half angles of th' with relative accuracy.
+//
+// Two arithmetics.  FAST (the BF16 networks' rows, 16 significant bits): hardware square roots and
+// y^zeta = 2^(zeta log2 y) from the hardware log2 (absolute error 2^-22).  Otherwise Newton steps and
+// y^zeta = 2^(zeta log2(1 - t)) from the Taylor series of the logarithm: y^zeta exceeds 2^-30 only for
+// small t, and dropping the terms from t^(d+1) on moves y^zeta by at most
+// zeta t^(d+1)/(d+1) (1-t)^zeta <= 1.5e-9 (d = 8, zeta >= 32), 1.1e-9 (d = 13, zeta >= 16) of its
+// maximum; all terms have one sign, so for t near 1 the sum still underflows as y^zeta does.  Below
+// zeta = 16 the power comes from the float pair 1 - t.
+#include <cuda_bf16.h>
+#include <math.h>
+
+#include <algorithm>
+
+#include "angular.cuh"
+#include "common.cuh"
+
+namespace panna {
+
+namespace {
+
+constexpr int kMW = 4;   // warps per CTA
+
+// D += A B, m16n8k8, TF32 operands (the leading 19 bits of each register), FP32 accumulators
+__device__ __forceinline__ void mma8(float (&c)[4], float a0, float a1, float a2, float a3, float b0, float b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(__float_as_uint(a0)), "r"(__float_as_uint(a1)), "r"(__float_as_uint(a2)),
+                   "r"(__float_as_uint(a3)), "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)));
+}
+
+// D = A B
+__device__ __forceinline__ void mma8z(float (&c)[4], float a0, float a1, float a2, float a3, float b0, float b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%10,%10,%10,%10};"
+                 : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+                 : "r"(__float_as_uint(a0)), "r"(__float_as_uint(a1)), "r"(__float_as_uint(a2)),
+                   "r"(__float_as_uint(a3)), "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)), "f"(0.f));
+}
+
+__device__ __forceinline__ float tf_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
+
+// x = hi + lo exactly; hi has the bits that TF32 keeps.  ROUND: hi to nearest, so that lo is signed
+// and what the tensor cores drop of it (its bits past 11) has no bias.
+template <bool ROUND>
+__device__ __forceinline__ void tf_split(float2 x, float2& hi, float2& lo)
+{
+    const uint32_t r = ROUND ? 0x1000u : 0u;
+    hi = make_float2(__uint_as_float((__float_as_uint(x.x) + r) & 0xffffe000u),
+                     __uint_as_float((__float_as_uint(x.y) + r) & 0xffffe000u));
+    lo = __fadd2_rn(x, make_float2(-hi.x, -hi.y));
+}
+
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+// zeta log2(1 - t) (or zeta - 1: coefficients zl) to degree PW, see the file comment
+template <int PW>
+__device__ __forceinline__ float2 log_series(const float* zl, float2 t)
+{
+    float2 p = dup(zl[PW - 1]);
+#pragma unroll
+    for (int k = PW - 2; k >= 0; --k) p = __ffma2_rn(p, t, dup(zl[k]));
+    return __fmul2_rn(p, t);
+}
+
+// (1 - t)^zeta below zeta = 16, from the float pair yh + yl = 1 - t: repeated squaring for whole
+// exponents (n > 0), the hardware log2 otherwise
+__device__ __forceinline__ float pow_low(float zeta, int n, float t)
+{
+    const float yh = 1.f - t;
+    const float yl = (1.f - yh) - t;
+    if (!(yh > 0.f)) return 0.f;
+    const float rel = yl * rcpf(yh);
+    if (n <= 0) return ex2f(zeta * fmaf(rel, 1.4426950408889634f, lg2f(yh)));
+    float p = 1.f, b = yh;
+    for (int k = n; k; k >>= 1) {
+        if (k & 1) p *= b;
+        b *= b;
+    }
+    return fmaf(p, zeta * rel, p);
+}
+
+// y^zeta = 2^(zeta log2 |y|) (FAST): y >= -eps/2, so its powers vanish to rounding below 0
+__device__ __forceinline__ float2 pow2_y(float zeta, float2 y)
+{
+    const float2 z = __fmul2_rn(make_float2(lg2f(fabsf(y.x)), lg2f(fabsf(y.y))), dup(zeta));
+    return make_float2(ex2f(z.x), ex2f(z.y));
+}
+
+// (1 - t)^zeta, zeta the exponent of the coefficients zl
+template <int PW>
+__device__ __forceinline__ float2 pow2_t(const float* zl, float zeta, int zeta_int, float2 t)
+{
+    if (PW == 0) return make_float2(pow_low(zeta, zeta_int, t.x), pow_low(zeta, zeta_int, t.y));
+    const float2 z = log_series<PW ? PW : 1>(zl, t);
+    return make_float2(ex2f(z.x), ex2f(z.y));
+}
+
+// Half angles (sin, cos of th'/2) from cos(theta) and sin_eps^2(theta): the one of (1 + |cos th'|)/2
+// without cancellation by a square root, the other from sin th' / 2
+template <bool FAST>
+__device__ __forceinline__ void half_angles(const DescDev& d, float c, float se2, float& sh, float& ch)
+{
+    float hq, o;
+    const float q = fmaf(0.5f * d.r_inv, fabsf(c), 0.5f);   // in [1/2, 1]
+    if (FAST) {
+        const float iq = rsqf(q);
+        hq = q * iq;
+        o = (0.5f * d.r_inv) * se2 * rsqf(fmaxf(se2, 1e-37f)) * iq;
+    } else {
+        hq = sqrt_nr(q);
+        o = div_nr(0.5f * d.r_inv * sqrt_nr(se2), hq);
+    }
+    ch = c >= 0.f ? hq : o;
+    sh = c >= 0.f ? o : hq;
+}
+
+// sqrt((1 + c + cl)/2) as hi + lo, c + cl >= -1
+__device__ __forceinline__ void half_pair(float c, float cl, float& h, float& l)
+{
+    float qh, ql;
+    two_sum(1.f, c, qh, ql);
+    ql += cl;
+    fast_two_sum(qh, ql, qh, ql);   // near c = -1 the low part is a large fraction
+    qh = fmaxf(0.5f * qh, 0.f);
+    h = sqrt_nr(qh);
+    l = h > 0.f ? fmaf(0.5f, ql, fmaf(-h, h, qh)) * (0.5f * rcpf(h)) : 0.f;
+}
+
+// The pairs of one species block as positions p = 0 .. n - 1: entries of the smaller segment (M of
+// them) against those of the larger one by diagonals, k1 = r, k2 = r + q (mod) with q = p / M,
+// r = p mod M; inside one segment (k, k + q + 1 mod M), each unordered pair once.  All positions of
+// one q have distinct first entries and distinct second entries.  A lane starts at p = lane and
+// steps by 32.
+struct BlockPairs {
+    int b1, b2, M, mod, off, n;
+    int q, r, dq, dr;
+    __device__ __forceinline__ BlockPairs(int sa, int na, int sb, int nb, bool same, int lane)
+    {
+        const bool sw = na > nb;
+        M = max(same ? na : (sw ? nb : na), 1);
+        mod = same ? na : (sw ? na : nb);
+        b1 = same || !sw ? sa : sb;
+        b2 = same || sw ? sa : sb;
+        off = same ? 1 : 0;
+        n = same ? na * (na - 1) / 2 : na * nb;
+        // quotients of small integers: the exact one is at least 1/(2M) from the next integer
+        const float inv = rcpf((float)M);
+        q = (int)(((float)lane + 0.5f) * inv);
+        r = lane - q * M;
+        dq = (int)(32.5f * inv);
+        dr = 32 - dq * M;
+    }
+    __device__ __forceinline__ void get(bool on, int& k1, int& k2) const
+    {
+        const int s = r + q + off;
+        const int y = s >= mod ? s - mod : s;
+        k1 = on ? b1 + r : 0;
+        k2 = on ? b2 + y : 0;
+    }
+    __device__ __forceinline__ void next()
+    {
+        r += dr;
+        q += dq;
+        if (r >= M) { r -= M; ++q; }
+    }
+};
+
+// species segments of an atom's entries (grouped by species) into seg[0..S]
+__device__ __forceinline__ void species_segments(const DescDev& d, const int2* __restrict__ idx, int n, int* seg,
+                                                 int lane)
+{
+    // entry k starts the segments of every species after its predecessor's up to its own
+    for (int k = lane; k <= n; k += 32) {
+        const int s1 = k < n ? meta_species(idx[k].y) : d.S;
+        const int s0 = k > 0 ? meta_species(idx[k - 1].y) : -1;
+        for (int s = s0 + 1; s <= s1; ++s) seg[s] = k;
+    }
+}
+
+// ------------------------------------------------------------------ descriptor
+
+// Arithmetic of the descriptor kernel.  FAST: see the file comment.  PAIR (FP32 networks, whose
+// forces have to meet 1e-5 of RMS): the half angles as float pairs.  Rounding them to single floats
+// moves the angle by about 3e-8, which the zeta-th power turns into 1e-6 of a term.  The error of a
+// rounded (sin, cos) along the circle is one angle delta per pair, so that
+//   sin((th' - theta_m)/2) = [sh cos_m - ch sin_m] + (delta - delta_m) cos((th' - theta_m)/2),
+// the bracket by an FMA-compensated difference of products, delta_m the same error of the sector's
+// constants.  Distances enter as the exact sum r1 + r2 = 2 (hi + lo).
+
+// shared bytes per warp: unit vectors and distances (PAIR: and their low parts), r, f_c, the pairs
+template <bool FAST>
+__host__ __device__ inline size_t desc_mma_warp_bytes(int cap)
+{
+    return FAST ? (size_t)((cap + 1) & ~1) * (16 + 4 + 4) + 16 * (16 + 16) : (size_t)cap * (16 + 16) + 16 * (16 + 16 + 16);
+}
+
+template <bool FAST, int CM, int PW>
+__global__ void __launch_bounds__(kMW * 32, FAST ? (CM == 1 ? 8 : 7) : (CM == 1 ? 6 : 5))
+k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __restrict__ out,
+           __nv_bfloat16* __restrict__ Gh, __nv_bfloat16* __restrict__ Gl)
+{
+    extern __shared__ float4 sm4[];
+    __shared__ int s_seg[kMW][kMaxSpecies + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int cap = w.cap, cap2 = (cap + 1) & ~1;
+    char* base = reinterpret_cast<char*>(sm4) + (size_t)warp * desc_mma_warp_bytes<FAST>(cap);
+    // FAST: (unit vector, rho = (r - R_c) sqrt(eta_l) / 2), r, f_c; PAIR: (unit vector, r), (its low
+    // part, f_c).  rho: distances relative to the middle shell R_c in units of the Gaussians' width, so
+    // that exp(-eta (r_bar - R)^2) = 2^(-x^2) with x = rho_1 + rho_2 - (R - R_c) sqrt(eta_l); rounding
+    // r - R_c instead of r keeps the small x of the terms that count
+    float4* sv = reinterpret_cast<float4*>(base);
+    float4* sl = sv + cap;
+    float* sr = reinterpret_cast<float*>(sv + cap2);
+    float* sf = sr + cap2;
+    const float r_c = d.rs_ang[d.n_ang_r / 2], s_eta = sqrtf(d.eta_ang * 1.4426950408889634f);
+    // geometry of the round's pairs, each for pairs t and t + 4 of a group.  pa: sin, cos of th'/2;
+    // pr: FAST x + nR, f_c f_c; PAIR: the halves of r_bar; pd: PAIR delta, f_c f_c.  Groups 2 and 3
+    // swap the two halves of each float4, so that the 32 lanes' stores fall on 32 banks
+    float4* pa = FAST ? reinterpret_cast<float4*>(sf + cap2) : sl + cap;
+    float4* pr = pa + 16;
+    float4* pd = pr + 16;
+    // this lane's slot of the pair buffers when it owns pair `lane`
+    const int slot = (lane >> 3) * 4 + t, half = (lane >> 2) & 1;
+    const int off0 = slot * 4 + half + ((lane >> 4) << 1), off1 = slot * 4 + half + (2 - ((lane >> 4) << 1));
+    float* pa_f = reinterpret_cast<float*>(pa);
+    float* pr_f = reinterpret_cast<float*>(pr);
+    float* pd_f = reinterpret_cast<float*>(pd);
+    int* seg = s_seg[warp];
+    const int ncm = (d.n_theta + 7) / 8, ncn = (d.n_ang_r + 7) / 8;
+    const int nbins = d.n_theta * d.n_ang_r;
+    const float eta_rl = d.eta_rad * 1.4426950408889634f;   // exp(-eta x^2) = 2^(-eta_l x^2)
+    const bool even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0;   // bin pairs on 8-byte boundaries
+    auto put = [&](size_t idx, float v) {
+        if (Gh) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            Gh[idx] = h;
+            if (Gl) Gl[idx] = __float2bfloat16_rn(v - __bfloat162float(h));
+        } else {
+            out[idx] = v;
+        }
+    };
+    auto put2 = [&](size_t idx, float v0, float v1) {
+        if (Gh) {
+            const __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
+            *reinterpret_cast<__nv_bfloat162*>(Gh + idx) = __nv_bfloat162(h0, h1);
+            if (Gl)
+                *reinterpret_cast<__nv_bfloat162*>(Gl + idx) =
+                    __nv_bfloat162(__float2bfloat16_rn(v0 - __bfloat162float(h0)),
+                                   __float2bfloat16_rn(v1 - __bfloat162float(h1)));
+        } else {
+            *reinterpret_cast<float2*>(out + idx) = make_float2(v0, v1);
+        }
+    };
+    for (int64_t i = (int64_t)blockIdx.x * kMW + warp; i < w.N; i += (int64_t)gridDim.x * kMW) {
+        const int64_t row = row_map ? row_map[i] : i;
+        if (row < 0) continue;   // ghosts are not centres
+        const int n = w.nb_count[i];
+        const size_t sb = (size_t)i * cap;
+        __syncwarp();   // the previous atom's reads of the staging area are done
+        for (int k = lane; k < n; k += 32) {
+            const float4 v = w.nb_vec[sb + k];
+            if (FAST) {
+                const float ir = 1.f / v.w;
+                sv[k] = make_float4(v.x * ir, v.y * ir, v.z * ir, (v.w - r_c) * (0.5f * s_eta));
+                const float c_ = cospif(0.5f * (v.w / d.rc));
+                sr[k] = v.w;
+                sf[k] = c_ * c_;
+            } else {
+                // the relative vector as hi + lo when the search kept the low parts; r and 1/r to
+                // about 2^-46
+                const float4 vl = w.nb_vlo ? w.nb_vlo[sb + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+                float px, ex, py, ey, pz, ez, s1, e1, s2, e2;
+                two_prod(v.x, v.x, px, ex);
+                two_prod(v.y, v.y, py, ey);
+                two_prod(v.z, v.z, pz, ez);
+                ex = fmaf(2.f * v.x, vl.x, ex);
+                ey = fmaf(2.f * v.y, vl.y, ey);
+                ez = fmaf(2.f * v.z, vl.z, ez);
+                two_sum(px, py, s1, e1);
+                two_sum(s1, pz, s2, e2);
+                const float r2l = ((e1 + e2) + (ex + ey)) + ez;
+                const float rh = sqrtf(s2);
+                const float rl = (fmaf(-rh, rh, s2) + r2l) * (0.5f / rh);
+                const float ih = 1.f / rh;
+                const float il = ih * (fmaf(-rh, ih, 1.f) - rl * ih);
+                const float hx = __fmul_rn(v.x, ih), hy = __fmul_rn(v.y, ih), hz = __fmul_rn(v.z, ih);
+                sv[k] = make_float4(hx, hy, hz, rh);
+                const float c_ = cospif(0.5f * (rh / d.rc));
+                sl[k] = make_float4(fmaf(v.x, ih, -hx) + fmaf(v.x, il, vl.x * ih),
+                                    fmaf(v.y, ih, -hy) + fmaf(v.y, il, vl.y * ih),
+                                    fmaf(v.z, ih, -hz) + fmaf(v.z, il, vl.z * ih), c_ * c_);
+            }
+        }
+        species_segments(d, w.nb_idx + sb, n, seg, lane);
+        __syncwarp();
+
+        // radial terms: lanes over shells
+        for (int nn = lane; nn < d.n_rad; nn += 32) {
+            const float rs = d.rs_rad[nn];
+            for (int sp = 0; sp < d.S; ++sp) {
+                float acc = 0.f;
+                for (int k = seg[sp]; k < seg[sp + 1]; ++k) {
+                    const float xr = (FAST ? sr[k] : sv[k].w) - rs;
+                    acc = fmaf(ex2f(-eta_rl * (xr * xr)), FAST ? sf[k] : sl[k].w, acc);
+                }
+                put((size_t)row * d.D + sp * d.n_rad + nn, acc);
+            }
+        }
+
+        // angular terms: CM sector chunks of 8 and one shell chunk of 8 at a time
+        for (int u0 = 0; u0 < ncm * ncn; u0 += CM) {
+            const int m0 = (u0 % ncm) * 8, n0 = (u0 / ncm) * 8;   // CM divides ncm
+            float2 chm[CM], shm[CM], tan_m[FAST ? 1 : CM];
+#pragma unroll
+            for (int mc = 0; mc < CM; ++mc) {
+                const int m = min(m0 + mc * 8 + g, d.n_theta - 1);
+                chm[mc] = dup(d.chr_t[m]);
+                shm[mc] = dup(d.shr_t[m]);
+                if (!FAST) tan_m[mc] = dup(d.tan_t[m]);
+            }
+            const float rs_g = d.rs_ang[min(n0 + g, d.n_ang_r - 1)];
+            const float2 nR = dup(FAST ? (r_c - rs_g) * s_eta : -rs_g);
+            const float2 y0 = dup(1.f + d.r_half), nk0 = dup(-d.r_half);
+            // the factor 2 of A_m = 2 y_m^zeta; FAST: and what rounding 1 + (R - 1)/2 takes from y^zeta
+            // where it is not small (y near 1)
+            const float two = FAST ? fmaf(2.f * d.zeta, d.r_half - (y0.x - 1.f), 2.f) : 2.f;
+            const float2 me = dup(-d.eta_ang * 1.4426950408889634f);
+            int blk = 0;
+            for (int a = 0; a < d.S; ++a)
+                for (int b = a; b < d.S; ++b, ++blk) {
+                    BlockPairs bp(seg[a], seg[a + 1] - seg[a], seg[b], seg[b + 1] - seg[b], a == b, lane);
+                    float acc[CM][4], comp[FAST ? 1 : CM][4];
+#pragma unroll
+                    for (int mc = 0; mc < CM; ++mc)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) acc[mc][q] = comp[FAST ? 0 : mc][q] = 0.f;
+                    for (int p0 = 0; p0 < bp.n; p0 += 32, bp.next()) {
+                        // step 1: geometry of the lane's pair (weight 0 past the block's end)
+                        {
+                            const bool on = p0 + lane < bp.n;
+                            int k1, k2;
+                            bp.get(on, k1, k2);
+                            const float4 va = sv[k1], vb = sv[k2];
+                            if (FAST) {
+                                const float wx = fmaf(va.y, vb.z, -va.z * vb.y);
+                                const float wy = fmaf(va.z, vb.x, -va.x * vb.z);
+                                const float wz = fmaf(va.x, vb.y, -va.y * vb.x);
+                                const float c = fmaf(va.x, vb.x, fmaf(va.y, vb.y, va.z * vb.z));
+                                const float s2 = fmaf(wx, wx, fmaf(wy, wy, fmaf(wz, wz, d.eps_theta)));
+                                float sh, ch;
+                                half_angles<true>(d, c, s2, sh, ch);
+                                pa_f[off0] = sh;
+                                pa_f[off1] = ch;
+                                pr_f[off0] = va.w + vb.w;
+                                pr_f[off1] = on ? sf[k1] * sf[k2] : 0.f;
+                            } else {
+                                const float4 la = sl[k1], lb = sl[k2];
+                                // cos = u1 . u2 as hi + lo
+                                float p0_, e0, p1_, e1, p2_, e2, s, ea, c, eb;
+                                two_prod(va.x, vb.x, p0_, e0);
+                                two_prod(va.y, vb.y, p1_, e1);
+                                two_prod(va.z, vb.z, p2_, e2);
+                                two_sum(p0_, p1_, s, ea);
+                                two_sum(s, p2_, c, eb);
+                                const float cross = fmaf(va.x, lb.x, fmaf(la.x, vb.x, fmaf(va.y, lb.y,
+                                                    fmaf(la.y, vb.y, fmaf(va.z, lb.z, la.z * vb.z)))));
+                                // cos th' = cos / R
+                                const float cl = fmaf(-c, d.r_def, (((ea + eb) + (e0 + e1)) + e2) + cross);
+                                // sin, cos of th'/2 as hi + lo: square roots of (1 -/+ cos th')/2
+                                float sh, shl, ch, chl;
+                                half_pair(-c, -cl, sh, shl);
+                                half_pair(c, cl, ch, chl);
+                                float rbh, rbl;
+                                rbar_halves(va.w, vb.w, rbh, rbl);
+                                pa_f[off0] = sh;
+                                pa_f[off1] = ch;
+                                pr_f[off0] = rbh;
+                                pr_f[off1] = rbl;
+                                pd_f[off0] = fmaf(shl, ch, -chl * sh);
+                                pd_f[off1] = on ? la.w * lb.w : 0.f;
+                            }
+                        }
+                        __syncwarp();
+                        // step 2: groups of 8 pairs
+                        float c[CM][4];
+#pragma unroll
+                        for (int mc = 0; mc < CM; ++mc)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) c[mc][q] = 0.f;
+                        float q2[FAST ? 1 : CM][4];
+                        const int left = bp.n - p0;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (8 * k >= left) break;
+                            float4 ha = pa[4 * k + t], hr = pr[4 * k + t], hd;
+                            if (!FAST) hd = pd[4 * k + t];
+                            if (k >= 2) {
+                                ha = make_float4(ha.z, ha.w, ha.x, ha.y);
+                                hr = make_float4(hr.z, hr.w, hr.x, hr.y);
+                                if (!FAST) hd = make_float4(hd.z, hd.w, hd.x, hd.y);
+                            }
+                            const float2 sh = make_float2(ha.x, ha.y), ch = make_float2(ha.z, ha.w);
+                            float2 z, ff;
+                            if (FAST) {
+                                const float2 x = __fadd2_rn(make_float2(hr.x, hr.y), nR);
+                                z = __fmul2_rn(x, make_float2(-x.x, -x.y));
+                                ff = make_float2(hr.z, hr.w);
+                            } else {
+                                const float2 x = __fadd2_rn(__fadd2_rn(make_float2(hr.x, hr.y), nR),
+                                                            make_float2(hr.z, hr.w));
+                                z = __fmul2_rn(__fmul2_rn(x, x), me);
+                                ff = make_float2(hd.z, hd.w);
+                            }
+                            const float2 e = __fmul2_rn(make_float2(ex2f(z.x), ex2f(z.y)), ff);
+                            float2 eh, el;
+                            tf_split<!FAST>(e, eh, el);
+#pragma unroll
+                            for (int mc = 0; mc < CM; ++mc) {
+                                const float2 w2 = __fmul2_rn(ch, shm[mc]);
+                                float2 ee = __ffma2_rn(sh, chm[mc], make_float2(-w2.x, -w2.y));
+                                if (FAST) {
+                                    const float2 A = pow2_y(d.zeta, __ffma2_rn(ee, make_float2(-ee.x, -ee.y), y0));
+                                    // scalar differences: the operand quad interleaves hi and lo
+                                    const float a0 = tf_hi(A.x), a1 = tf_hi(A.y), l0 = A.x - a0, l1 = A.y - a1;
+                                    mma8(c[mc], a0, l0, a1, l1, eh.x, eh.y);
+                                    mma8(c[mc], a0, l0, a1, l1, el.x, el.y);
+                                } else {
+                                    const float2 mch = make_float2(-ch.x, -ch.y);
+                                    const float2 dw = __ffma2_rn(mch, shm[mc], w2);   // minus the rounding of w2
+                                    const float2 cc = __ffma2_rn(ch, chm[mc], __fmul2_rn(sh, shm[mc]));
+                                    const float2 dt = __fadd2_rn(make_float2(hd.x, hd.y), tan_m[mc]);
+                                    ee = __fadd2_rn(ee, __ffma2_rn(dt, cc, dw));
+                                    const float2 A = pow2_t<PW>(d.zlog, d.zeta, d.zeta_int, __ffma2_rn(ee, ee, nk0));
+                                    float2 Ah, Al;
+                                    tf_split<true>(A, Ah, Al);
+                                    // the tensor cores truncate their sums: two groups deep here
+                                    if (k & 1) mma8(q2[mc], Ah.x, Al.x, Ah.y, Al.y, el.x, el.y);
+                                    else mma8z(q2[mc], Ah.x, Al.x, Ah.y, Al.y, el.x, el.y);
+                                    mma8(q2[mc], Ah.x, Al.x, Ah.y, Al.y, eh.x, eh.y);
+                                    if ((k & 1) || 8 * (k + 1) >= left) {
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) c[mc][j] += q2[mc][j];
+                                    }
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int mc = 0; mc < CM; ++mc)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                if (FAST) {
+                                    acc[mc][q] += c[mc][q];
+                                } else {   // compensated sum over the block's rounds
+                                    const float v = c[mc][q] - comp[FAST ? 0 : mc][q], ns = acc[mc][q] + v;
+                                    comp[FAST ? 0 : mc][q] = (ns - acc[mc][q]) - v;
+                                    acc[mc][q] = ns;
+                                }
+                            }
+                        __syncwarp();
+                    }
+                    // rows g (A_hi) and g + 8 (A_lo), shells 2 t and 2 t + 1
+#pragma unroll
+                    for (int mc = 0; mc < CM; ++mc) {
+                        const int m = m0 + mc * 8 + g, nq = n0 + 2 * t;
+                        const float v0 = two * (acc[mc][0] + acc[mc][2]), v1 = two * (acc[mc][1] + acc[mc][3]);
+                        const size_t o = (size_t)row * d.D + d.rad_cols + blk * nbins + m * d.n_ang_r + nq;
+                        if (m < d.n_theta) {
+                            if (even && nq < d.n_ang_r) {
+                                put2(o, v0, v1);
+                            } else {
+                                if (nq < d.n_ang_r) put(o, v0);
+                                if (nq + 1 < d.n_ang_r) put(o + 1, v1);
+                            }
+                        }
+                    }
+                }
+        }
+    }
+}
+
+int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 152;
+}
+
+// resident CTAs walking the atoms: as many as fit on the GPU at once, no more than the atoms need
+template <class Kern, class... Args>
+cudaError_t launch_resident(Kern kern, int64_t N, size_t smem, cudaStream_t s, Args... args)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMW * 32, smem);
+    if (e != cudaSuccess) return e;
+    const unsigned nb = (unsigned)std::min<int64_t>((N + kMW - 1) / kMW, (int64_t)sm_count() * std::max(per_sm, 1));
+    kern<<<nb, kMW * 32, smem, s>>>(args...);
+    return cudaGetLastError();
+}
+
+constexpr size_t kMaxSmem = 200 * 1024;
+
+}  // namespace
+
+// FAST needs exponents for which the splits' truncation stays below the hardware log2's error
+static bool desc_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 16.f; }
+
+static size_t desc_smem(const Work& w, const DescDev& d, bool fast)
+{
+    return kMW * (desc_fast(d, fast) ? desc_mma_warp_bytes<true>(w.cap) : desc_mma_warp_bytes<false>(w.cap));
+}
+
+bool desc_mma_fits(const Work& w, const DescDev& d, bool fast)
+{
+    return d.ang_kind == 0 && desc_smem(w, d, fast) <= kMaxSmem;
+}
+
+cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_map, float* G_rows,
+                            __nv_bfloat16* Gh, __nv_bfloat16* Gl, bool fast, cudaStream_t s)
+{
+    if (!desc_mma_fits(w, d, fast)) return cudaErrorNotSupported;
+    if (w.N == 0) return cudaSuccess;
+    const size_t smem = desc_smem(w, d, fast);
+    auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, row_map, G_rows, Gh, Gl); };
+    const bool two = ((d.n_theta + 7) / 8) % 2 == 0;
+    if (desc_fast(d, fast)) return two ? run(k_desc_mma<true, 2, 0>) : run(k_desc_mma<true, 1, 0>);
+    if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8>) : run(k_desc_mma<false, 1, 8>);
+    if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13>) : run(k_desc_mma<false, 1, 13>);
+    return two ? run(k_desc_mma<false, 2, 0>) : run(k_desc_mma<false, 1, 0>);
+}
+
+}  // namespace panna

@@ -65,8 +65,9 @@ struct Arena {
 };
 
 constexpr int kNumVariants = 6;   // most variants of one descriptor-family kernel
-// variants per kernel: descriptor and JVP 0..4, adjoint 0..5
-constexpr int kKindVariants[3] = {5, 6, 5};
+// variants per kernel: descriptor 0..5, adjoint 0..5, JVP 0..4; the matrix form's number (-1: none)
+constexpr int kMmaVariant[3] = {5, -1, -1};
+constexpr int kKindVariants[3] = {6, 6, 5};
 const char* kStages[] = {"neighbors", "descriptor", "mlp", "adjoint", "forces", "jvp", "mlp_grad", "loss"};
 constexpr int kNumStages = 8;
 
@@ -377,25 +378,40 @@ ParamRanges frozen_ranges(const panna_ctx* c)
 enum { KV_DESC = 0, KV_ADJ = 1, KV_JVP = 2 };
 
 template <class Launch>
-int tuned_variant_(panna_ctx* c, const panna_system* sys, int prec, int kind, cudaStream_t s, Launch launch, bool ext);
+int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int prec, int kind, cudaStream_t s,
+                   Launch launch, bool acc);
 
-// ext (descriptor with FP32 networks, force tolerance 1e-5 of RMS): only the kernels that carry
-// the angular terms as float pairs (variants 0 and 1) are candidates.  The compensated FP32
+// The matrix form (descriptor 5) where it applies, without measuring anything: from
+// kSplitAtoms atoms on it was the fastest on every workload measured, from 5-29-atom molecules
+// (descriptor 0.144 -> 0.068 ms for 1024 of them) to the 1M-atom box (below that size the old kernels
+// spread one atom over several warps).
+int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
+{
+    if (w.N < kSplitAtoms) return -1;
+    if (kind == KV_DESC && desc_mma_fits(w, c->d, !acc)) return 5;
+    return -1;
+}
+
+// acc: FP32 networks (force tolerance 1e-5 of RMS).  Their descriptor takes only the kernels that
+// carry the angle as float pairs (variants 0, 1 and 5).  The compensated FP32
 // kernels keep the angle in single floats, whose rounding (about 6e-8 rad) the zeta-th power
 // turns into ~1e-6 relative per term; on the 1024 molecules that put one atom's force at
 // 0.95-1.16e-5 of RMS against 4.3e-6 with the float pairs.
 template <class Launch>
-int tuned_variant(panna_ctx* c, const panna_system* sys, int prec, int kind, cudaStream_t s, Launch launch,
-                  bool ext = false)
+int tuned_variant(panna_ctx* c, const panna_system* sys, const Work& w, int prec, int kind, cudaStream_t s,
+                  Launch launch, bool acc)
 {
-    const int v = tuned_variant_(c, sys, prec, kind, s, launch, ext && kind == KV_DESC);
+    int v = c->force_variant[kind] >= 0 ? -1 : mma_variant(c, w, kind, acc);
+    if (v < 0) v = tuned_variant_(c, sys, w, prec, kind, s, launch, acc);
     c->last_variant[kind] = v;
     return v;
 }
 
 template <class Launch>
-int tuned_variant_(panna_ctx* c, const panna_system* sys, int prec, int kind, cudaStream_t s, Launch launch, bool ext)
+int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int prec, int kind, cudaStream_t s,
+                   Launch launch, bool acc)
 {
+    const bool ext = acc && kind == KV_DESC;
     if (c->force_variant[kind] >= 0) return c->force_variant[kind];
     panna_ctx::Tuned* t = nullptr;
     for (int k = 0; k < c->n_tuned; ++k) {
@@ -407,12 +423,18 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, int prec, int kind, cu
     const int fallback = (sys->n_atoms < kSplitAtoms || ext) ? 0 : (kind == KV_ADJ ? 5 : 2);
     if (!c->autotune || c->async || sys->n_atoms == 0) return fallback;
     float ms[kNumVariants] = {};
-    const int nv = ext ? 2 : kKindVariants[kind];
-    for (int v = 0; v < nv; ++v) launch(v);   // first launches load and configure the kernels
+    const bool mma = kind == KV_DESC && desc_mma_fits(w, c->d, !acc);
+    auto candidate = [&](int v) {
+        if (v == kMmaVariant[kind]) return mma;
+        return !ext || v < 2;
+    };
+    for (int v = 0; v < kKindVariants[kind]; ++v)
+        if (candidate(v)) launch(v);   // first launches load and configure the kernels
     int best = 0;
     // three back-to-back launches per variant: the host's launch work then overlaps the kernels
     // instead of showing up as idle device time in a single short measurement
-    for (int v = 0; v < nv; ++v) {
+    for (int v = 0; v < kKindVariants[kind]; ++v) {
+        if (!candidate(v)) continue;
         cudaEventRecord(c->tev[0], s);
         for (int r = 0; r < 3; ++r) launch(v);
         cudaEventRecord(c->tev[1], s);
@@ -468,7 +490,7 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
         CU(mlp_tiles(c->plan, L.w.seg_off, L.mb.tile_start, s, &nl));
         stage_mark(c, 1, s);
         int dummy = 0;
-        const int v = tuned_variant(c, sys, rq.prec, KV_DESC, s, [&](int vv) {
+        const int v = tuned_variant(c, sys, L.w, rq.prec, KV_DESC, s, [&](int vv) {
             launch_descriptor(L.w, c->d, L.G, L.w.row_of_atom, acc, s, &dummy, vv);
         }, acc);
         const bool tcp = rq.prec == PANNA_MLP_BF16 || rq.prec == PANNA_MLP_BF16_FAST;
@@ -514,9 +536,9 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
             CU(launch_store_adjoint(*sv, c->d, L.g, F, rq.virial ? L.vir_atom : nullptr, s, &nl));
         } else {
             int dummy = 0;
-            const int variant = tuned_variant(c, sys, rq.prec, KV_ADJ, s, [&](int vv) {
+            const int variant = tuned_variant(c, sys, L.w, rq.prec, KV_ADJ, s, [&](int vv) {
                 launch_adjoint(L.w, c->d, L.g, L.F_tune, nullptr, acc, vv, s, &dummy);
-            });
+            }, acc);
             CU(cudaMemsetAsync(F, 0, sizeof(float) * 3 * N, s));
             CU(launch_adjoint(L.w, c->d, L.g, F, rq.virial ? L.vir_atom : nullptr, acc, variant, s, &nl));
         }
@@ -547,9 +569,9 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
             // forces): the plain FP32 angular form unless extended precision is forced
             const bool acc_jvp = c->ang_mode == 1;
             int dummy = 0;
-            const int v = tuned_variant(c, sys, rq.prec, KV_JVP, s, [&](int vv) {
+            const int v = tuned_variant(c, sys, L.w, rq.prec, KV_JVP, s, [&](int vv) {
                 launch_jvp(L.w, c->d, u, L.wdot, acc_jvp, s, &dummy, vv);
-            });
+            }, acc_jvp);
             CU(launch_jvp(L.w, c->d, u, L.wdot, acc_jvp, s, &nl, v));
         } else {
             CU(cudaMemsetAsync(L.wdot, 0, sizeof(float) * (size_t)N * c->d.D, s));
@@ -1060,7 +1082,7 @@ panna_status panna_qeq_energy_forces(panna_ctx* c, const panna_system* sys, cons
         CU(mlp_tiles(c->plan, L.w.seg_off, L.mb.tile_start, s, &nl));
         stage_mark(c, 1, s);
         int dummy = 0;
-        const int vd = tuned_variant(c, sys, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
+        const int vd = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
             launch_descriptor(L.w, c->d, L.G, L.w.row_of_atom, acc, s, &dummy, vv);
         }, acc);
         CU(launch_descriptor(L.w, c->d, L.G, L.w.row_of_atom, acc, s, &nl, vd));
@@ -1074,9 +1096,9 @@ panna_status panna_qeq_energy_forces(panna_ctx* c, const panna_system* sys, cons
                       &nl));
         stage_mark(c, 3, s);
         CU(mlp_input_grad(c->plan, L.mb, theta, N, L.g, s, &nl, nullptr, true));
-        const int va = tuned_variant(c, sys, PANNA_MLP_FP32, KV_ADJ, s, [&](int vv) {
+        const int va = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_ADJ, s, [&](int vv) {
             launch_adjoint(L.w, c->d, L.g, L.F_tune, nullptr, acc, vv, s, &dummy);
-        });
+        }, acc);
         CU(launch_adjoint(L.w, c->d, L.g, F, nullptr, acc, va, s, &nl));
         stage_mark(c, 7, s);
         CU(launch_cfg_reduce(L.w, L.E_rows, nullptr, E_cfg, nullptr, E_atom, L.cfg_part, s, &nl));
@@ -1134,7 +1156,7 @@ panna_status panna_qeq_loss_grad(panna_ctx* c, const panna_system* sys, const fl
         CU(mlp_tiles(c->plan, L.w.seg_off, L.mb.tile_start, s, &nl));
         stage_mark(c, 1, s);
         int dummy = 0;
-        const int vd = tuned_variant(c, sys, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
+        const int vd = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
             launch_descriptor(L.w, c->d, L.G, L.w.row_of_atom, acc, s, &dummy, vv);
         }, acc);
         CU(launch_descriptor(L.w, c->d, L.G, L.w.row_of_atom, acc, s, &nl, vd));
@@ -1147,9 +1169,9 @@ panna_status panna_qeq_loss_grad(panna_ctx* c, const panna_system* sys, const fl
                       &nl));
         stage_mark(c, 3, s);
         CU(mlp_input_grad(c->plan, L.mb, theta, N, L.g, s, &nl, nullptr, true));
-        const int va = tuned_variant(c, sys, PANNA_MLP_FP32, KV_ADJ, s, [&](int vv) {
+        const int va = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_ADJ, s, [&](int vv) {
             launch_adjoint(L.w, c->d, L.g, L.F_tune, nullptr, acc, vv, s, &dummy);
-        });
+        }, acc);
         CU(launch_adjoint(L.w, c->d, L.g, Fo, nullptr, acc, va, s, &nl));
         CU(launch_cfg_reduce(L.w, L.E_rows, nullptr, Eo, nullptr, nullptr, L.cfg_part, s, &nl));
         stage_mark(c, 7, s);
@@ -1157,9 +1179,9 @@ panna_status panna_qeq_loss_grad(panna_ctx* c, const panna_system* sys, const fl
                        w_force, loss, L.alpha_cfg, L.u, L.loss_part, s, &nl));
         stage_mark(c, 5, s);
         const bool acc_jvp = c->ang_mode == 1;
-        const int vj = tuned_variant(c, sys, PANNA_MLP_FP32, KV_JVP, s, [&](int vv) {
+        const int vj = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_JVP, s, [&](int vv) {
             launch_jvp(L.w, c->d, L.u, L.wdot, acc_jvp, s, &dummy, vv);
-        });
+        }, acc_jvp);
         CU(launch_jvp(L.w, c->d, L.u, L.wdot, acc_jvp, s, &nl, vj));
         stage_mark(c, 6, s);
         CU(mlp_param_grad(c->plan, L.mb, theta, N, L.wdot, nullptr, dtheta, s, &nl, false, nullptr,
@@ -1293,7 +1315,7 @@ panna_status panna_store_build(panna_ctx* c, const panna_system* sys, const pann
     CU(launch_store_offsets(L.w, v.ent_off, s, &nl));
     const bool acc = c->ang_mode != 2;
     int dummy = 0;
-    const int variant = tuned_variant(c, sys, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
+    const int variant = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
         launch_descriptor(L.w, c->d, v.G, L.w.row_of_atom, acc, s, &dummy, vv);
     }, acc);
     CU(launch_descriptor(L.w, c->d, v.G, L.w.row_of_atom, acc, s, &nl, variant));

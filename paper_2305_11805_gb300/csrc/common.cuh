@@ -49,6 +49,12 @@ struct DescDev {
     float zpoly[5];                // zeta log2(e) log(y) = w (c0 + c1 w^2 + ... + c4 w^8), w = t / (2 - t)
     float rs_ang_step;             // dR of a uniform angular R grid, else 0
     float cos_t[kMaxTheta], sin_t[kMaxTheta];   // cos(theta_m), sin(theta_m)
+    // matrix form (angular_mma.cu), R = sqrt(1 + eps): sqrt(R) cos(theta_m/2), sqrt(R) sin(theta_m/2),
+    // (R - 1)/2, 1/R, and the Taylor coefficients of zeta log2(1 - t), (zeta - 1) log2(1 - t)
+    float chr_t[kMaxTheta], shr_t[kMaxTheta];
+    float tan_t[kMaxTheta];   // angle of the float pair (chr_t, shr_t) above theta_m/2
+    float r_half, r_inv, r_def;   // r_def = 1 - 1/R
+    float zlog[13], zlog1[13];
     // standard BP angular term (ang_kind 1): sector m = (lambda_m, zeta_m), shell n = eta_n
     int32_t ang_kind;              // 0 = modified (mBP), 1 = standard BP
     float bp_lambda[kMaxTheta], bp_zeta[kMaxTheta], bp_pref[kMaxTheta];   // pref = 2^(1 - zeta)
@@ -155,6 +161,13 @@ cudaError_t launch_adjoint(const Work& w, const DescDev& d, const float* g_rows,
 // networks whose operand rows hold about 16 significant bits
 cudaError_t launch_descriptor_bf16(const Work& w, const DescDev& d, __nv_bfloat16* Gh, __nv_bfloat16* Gl,
                                    const int32_t* row_map, int variant, cudaStream_t s, int* launches, bool fast);
+// Matrix form of the angular kernels (angular_mma.cu): the products over sectors and shells on the
+// warp-level tensor cores.  cudaErrorNotSupported when the descriptor or the batch is outside what
+// they take (desc_mma_fits).  Rows in FP32 (G_rows) or as BF16 hi (+ lo) parts.
+// fast: the forms of the BF16 networks; otherwise those of the FP32 ones.
+bool desc_mma_fits(const Work& w, const DescDev& d, bool fast);
+cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_map, float* G_rows,
+                            __nv_bfloat16* Gh, __nv_bfloat16* Gl, bool fast, cudaStream_t s);
 cudaError_t launch_jvp(const Work& w, const DescDev& d, const float* u, float* wdot_rows, bool acc, cudaStream_t s,
                        int* launches, int variant = 0);
 
