@@ -229,7 +229,8 @@ panna_status panna_set_angular_precision(panna_ctx* ctx, int32_t mode);
  * adjoint only 5 = the compensated kernel walking each atom's pairs in diagonal order
  * (k, k + d mod n), whose rounds of min(32, n - 1) pairs touch distinct entries on each side,
  * so the per-entry gradients are summed without atomics in a fixed order (bit-reproducible).
-* Matrix form: descriptor 5 (any descriptor of the modified term): one warp per atom, the products over sectors and shells on the tensor cores from
+ * Matrix forms: descriptor 5 (any descriptor of the modified term) and adjoint 6 (at most 16 sectors
+ * and 8 shells): one warp per atom, the products over sectors and shells on the tensor cores from
  * operands split into TF32 parts; sums in a fixed order.  Where they apply, batches of at least 1216
  * atoms take them without measuring.  With FP32 networks (extended angular terms) the descriptor's
  * candidates are variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that
@@ -250,7 +251,8 @@ panna_status panna_set_tuning(panna_ctx* ctx, const char* knob, int32_t value);
 /* The kernel variant that knob "descriptor", "adjoint" or "jvp" ran with in the last compute
  * call that used it (tuned or forced): 0 blocked, 1 flattened, 2 / 3 / 4 compensated with 32 / 16
  * / 8 lanes per (species block, theta chunk, R chunk) unit (adjoint 4: flattened units), 5
- * compensated in diagonal pair order (adjoint) or the matrix form (descriptor); -1 before any such call or for an unknown knob. */
+ * compensated in diagonal pair order (adjoint) or the matrix form (descriptor), 6 the adjoint's
+ * matrix form; -1 before any such call or for an unknown knob. */
 int32_t panna_tuning_choice(const panna_ctx* ctx, const char* knob);
 
 /*

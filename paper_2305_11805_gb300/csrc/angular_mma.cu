@@ -1,4 +1,4 @@
-// Angular descriptor with the products over sectors and shells on the warp-level
+// Angular descriptor and its adjoint with the products over sectors and shells on the warp-level
 // tensor cores (modified angular term; the forms are those of descriptor.cu).
 //
 // What is different from the one-lane-per-pair kernels.  Per pair of neighbours the angular term
@@ -520,6 +520,397 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
     }
 }
 
+// ------------------------------------------------------------------ adjoint
+
+// Gradient of sum_i g_i . G_i with respect to the neighbour vectors, as k_adj_cd of descriptor.cu,
+// with the products T e and T (x e) of a species block's gradient tile T (sectors x shells) on the
+// tensor cores: 16 pairs are the rows of one A operand (their Gaussians, evaluated by lane (g, t) for
+// pairs g, g + 8 and shells t, t + 4), T^T the B operand, held in registers for the whole block.
+// The result leaves sectors 2t, 2t + 1 of pairs g, g + 8 in lane (g, t), which evaluates those
+// sectors' powers and multiplies; the four lanes of a pair leave their sums in shared memory for
+// the pair's own lane, which applies the chain rule (step 3).
+//
+// Per-entry sums.  dc/dv1 = (W x v1)/(r1^3 r2), dc/dv2 = -(W x v2)/(r1 r2^3) with W = v1 x v2, so one
+// vector X = (dT/dc) W/(r1 r2) serves both entries of a pair: q_k = (sum X) x v_k / r_k^2 (minus for
+// second entries) plus the distance terms along v_k.  Each pair adds one float4 (X, dT/dr) to each of
+// its entries; the positions of one diagonal of the block touch distinct entries, and the few
+// diagonals within a round of 32 pairs go to different copies of the sums (nc of them), so nothing
+// needs atomics and every sum has a fixed order.
+
+// Shared-memory traffic bounds the kernel next to instruction issue (a warp's load of 4 bytes per lane
+// takes the SM's data path for a cycle, also when lanes share addresses), so the pair buffers carry
+// single floats, f_c and f_c' stay in registers from step 1 to step 3, and FAST stages unit vectors.
+
+struct AdjSmem {
+    int sv, sx, sr, sq, g, pa, pr, pts, pt1, total;   // byte offsets within a warp's area
+};
+__host__ __device__ inline AdjSmem adj_mma_smem(const DescDev& d, int cap, int nc, bool fast)
+{
+    const int c2 = (cap + 1) & ~1, c4 = (cap + 3) & ~3;
+    AdjSmem a;
+    a.sv = 0;
+    a.sx = a.sv + cap * 16;
+    a.sr = a.sx + c2 * (fast ? 8 : 16);
+    a.sq = a.sr + (fast ? c4 * 4 : 0);
+    a.g = a.sq + nc * cap * 16;
+    a.pa = a.g + ((d.D + 3) & ~3) * 4;
+    a.pr = a.pa + 16 * 16;
+    a.pts = a.pr + 16 * (fast ? 8 : 16);
+    a.pt1 = a.pts + 128 * 8;
+    a.total = a.pt1 + 128 * 4;
+    return a;
+}
+
+template <bool FAST, int CM, int PW>
+__global__ void __launch_bounds__(kMW * 32, CM == 1 ? 5 : 4)
+k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict__ F, float* __restrict__ vir_atom,
+          int nc)
+{
+    extern __shared__ float4 sm4[];
+    __shared__ int s_seg[kMW][kMaxSpecies + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int cap = w.cap;
+    const AdjSmem lay = adj_mma_smem(d, cap, nc, FAST);
+    char* base = reinterpret_cast<char*>(sm4) + (size_t)warp * lay.total;
+    float4* sv = reinterpret_cast<float4*>(base + lay.sv);   // FAST: (unit vector, rho), else (v, r)
+    float2* sx2 = reinterpret_cast<float2*>(base + lay.sx);  // FAST: (f_c, f_c')
+    float4* sx4 = reinterpret_cast<float4*>(base + lay.sx);  // else (f_c, f_c', 1/r, -)
+    float* sr = reinterpret_cast<float*>(base + lay.sr);     // FAST: r
+    float4* sq = reinterpret_cast<float4*>(base + lay.sq);   // nc copies of (sum X, sum dT/dr)
+    float* sg = reinterpret_cast<float*>(base + lay.g);      // the atom's gradient row
+    float4* pa = reinterpret_cast<float4*>(base + lay.pa);   // pairs p, p + 8: sin, cos of th'/2 (FAST: cos, sin_eps)
+    float2* pr2 = reinterpret_cast<float2*>(base + lay.pr);  // pairs p, p + 8: FAST distance,
+    float4* pr4 = reinterpret_cast<float4*>(base + lay.pr);  // else its hi and lo parts
+    float2* pts = reinterpret_cast<float2*>(base + lay.pts); // the four lanes' parts of a pair's sums
+    float* pt1 = reinterpret_cast<float*>(base + lay.pt1);
+    const int my = (lane >> 4) * 8 + (lane & 7), half = (lane >> 3) & 1;
+    float* pa_my = reinterpret_cast<float*>(pa) + my * 4 + half;
+    float* pr_my = reinterpret_cast<float*>(pr2) + my * (FAST ? 2 : 4) + half;
+    int* seg = s_seg[warp];
+    const int nbins = d.n_theta * d.n_ang_r;
+    const float eta_l = d.eta_ang * 1.4426950408889634f;
+    const float r_c = d.rs_ang[d.n_ang_r / 2], s_eta = sqrtf(eta_l);
+    // this lane's shells (t, t + 4) and sectors (2t, 2t + 1 of each chunk)
+    float2 nR0, nR1, chm[CM], shm[CM];
+    {
+        const float ra = d.rs_ang[min(t, d.n_ang_r - 1)], rb = d.rs_ang[min(t + 4, d.n_ang_r - 1)];
+        nR0 = dup(FAST ? (r_c - ra) * s_eta : -ra);
+        nR1 = dup(FAST ? (r_c - rb) * s_eta : -rb);
+#pragma unroll
+        for (int mc = 0; mc < CM; ++mc) {
+            const int ma = min(mc * 8 + 2 * t, d.n_theta - 1), mb = min(mc * 8 + 2 * t + 1, d.n_theta - 1);
+            chm[mc] = FAST ? make_float2(d.half_cos_t[ma], d.half_cos_t[mb]) : make_float2(d.chr_t[ma], d.chr_t[mb]);
+            shm[mc] = FAST ? make_float2(d.half_sin_t[ma], d.half_sin_t[mb]) : make_float2(d.shr_t[ma], d.shr_t[mb]);
+        }
+    }
+    // dT/dr = s1 Fp S1 + ...: x e in the units of nR0
+    const float s1 = FAST ? -2.f * d.eta_ang / s_eta : -2.f * d.eta_ang;
+    const bool gvec = (d.D & 3) == 0 && (reinterpret_cast<uintptr_t>(g_rows) & 15) == 0;
+
+    for (int64_t i = (int64_t)blockIdx.x * kMW + warp; i < w.N; i += (int64_t)gridDim.x * kMW) {
+        const int64_t row = w.row_of_atom[i];
+        if (row < 0) continue;   // ghosts are not centres
+        const int n = w.nb_count[i];
+        const size_t sb = (size_t)i * cap;
+        __syncwarp();   // the previous atom's reads of the staging area are done
+        {
+            const float* gi = g_rows + (size_t)row * d.D;
+            if (gvec) {
+                for (int c = lane; c < d.D / 4; c += 32)
+                    reinterpret_cast<float4*>(sg)[c] = reinterpret_cast<const float4*>(gi)[c];
+            } else {
+                for (int c = lane; c < d.D; c += 32) sg[c] = gi[c];
+            }
+        }
+        for (int k = lane; k < n; k += 32) {
+            const float4 v = w.nb_vec[sb + k];
+            const float ir = 1.f / v.w;
+            float s_, c_;
+            sincospif(0.5f * (v.w / d.rc), &s_, &c_);
+            const float fc = c_ * c_, dfc = -d.pi_rc * s_ * c_;
+            if (FAST) {
+                sv[k] = make_float4(v.x * ir, v.y * ir, v.z * ir, (v.w - r_c) * (0.5f * s_eta));
+                sx2[k] = make_float2(fc, dfc);
+                sr[k] = v.w;
+            } else {
+                sv[k] = v;
+                sx4[k] = make_float4(fc, dfc, ir, 0.f);
+            }
+            for (int c = 0; c < nc; ++c) sq[c * cap + k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        species_segments(d, w.nb_idx + sb, n, seg, lane);
+        __syncwarp();
+
+        // radial terms: four lanes per entry, each every fourth shell
+        for (int k0 = 0; k0 < n; k0 += 8) {
+            const int k = k0 + g;
+            float T0 = 0.f, T1 = 0.f;
+            if (k < n) {
+                int sp = 0;
+                while (k >= seg[sp + 1]) ++sp;
+                const float* gr = sg + sp * d.n_rad;
+                const float r = FAST ? sr[k] : sv[k].w, me = -d.eta_rad * 1.4426950408889634f;
+                for (int nn = t; nn < d.n_rad; nn += 4) {
+                    const float xr = r - d.rs_rad[nn];
+                    const float ge = gr[nn] * ex2f(me * (xr * xr));
+                    T0 += ge;
+                    T1 = fmaf(ge, xr, T1);
+                }
+            }
+            T0 += __shfl_xor_sync(0xffffffffu, T0, 1);
+            T1 += __shfl_xor_sync(0xffffffffu, T1, 1);
+            T0 += __shfl_xor_sync(0xffffffffu, T0, 2);
+            T1 += __shfl_xor_sync(0xffffffffu, T1, 2);
+            if (k < n && t == 0) {
+                const float fc = FAST ? sx2[k].x : sx4[k].x, dfc = FAST ? sx2[k].y : sx4[k].y;
+                sq[k].w = fmaf(dfc, T0, -2.f * d.eta_rad * fc * T1);
+            }
+        }
+        __syncwarp();
+
+        int blk = 0;
+        for (int a = 0; a < d.S; ++a)
+            for (int b = a; b < d.S; ++b, ++blk) {
+                BlockPairs bp(seg[a], seg[a + 1] - seg[a], seg[b], seg[b + 1] - seg[b], a == b, lane);
+                if (bp.n == 0) continue;
+                // T^T as B operands (sector g, shells t and t + 4), hi and lo
+                // FAST: and of T^T with its columns scaled by R - R_c (in the units of x)
+                float2 th[CM], tl[CM], uh[FAST ? CM : 1], ul[FAST ? CM : 1];
+#pragma unroll
+                for (int mc = 0; mc < CM; ++mc) {
+                    const int m = mc * 8 + g;
+                    const float* gt = sg + d.rad_cols + blk * nbins + m * d.n_ang_r;
+                    const bool in = m < d.n_theta;
+                    const float2 T = make_float2(in && t < d.n_ang_r ? gt[t] : 0.f,
+                                                 in && t + 4 < d.n_ang_r ? gt[t + 4] : 0.f);
+                    tf_split<true>(T, th[mc], tl[mc]);
+                    if (FAST) tf_split<true>(__fmul2_rn(T, make_float2(nR0.x, nR1.x)), uh[mc], ul[mc]);
+                }
+                for (int p0 = 0; p0 < bp.n; p0 += 32, bp.next()) {
+                    // step 1: geometry of the lane's pair
+                    const bool on = p0 + lane < bp.n;
+                    int k1, k2;
+                    bp.get(on, k1, k2);
+                    float wx, wy, wz, ise;   // W/(r1 r2), 1/sin_eps
+                    float2 f1, f2;           // (f_c, f_c') of the two entries
+                    float rho = 0.f;
+                    {
+                        const float4 va = sv[k1], vb = sv[k2];
+                        float sh, ch;
+                        if (FAST) {
+                            f1 = sx2[k1]; f2 = sx2[k2];
+                            wx = fmaf(va.y, vb.z, -va.z * vb.y);
+                            wy = fmaf(va.z, vb.x, -va.x * vb.z);
+                            wz = fmaf(va.x, vb.y, -va.y * vb.x);
+                            const float s2 = fmaf(wx, wx, fmaf(wy, wy, fmaf(wz, wz, d.eps_theta)));
+                            ise = rsqf(fmaxf(s2, 1e-37f));
+                            sh = fmaf(va.x, vb.x, fmaf(va.y, vb.y, va.z * vb.z));   // cos, sin_eps themselves
+                            ch = s2 * ise;
+                            rho = va.w + vb.w;
+                            pr_my[0] = rho;
+                        } else {
+                            const float4 xa = sx4[k1], xb = sx4[k2];
+                            f1 = make_float2(xa.x, xa.y);
+                            f2 = make_float2(xb.x, xb.y);
+                            const float ir12 = xa.z * xb.z;
+                            wx = dop(va.y, vb.z, va.z, vb.y) * ir12;
+                            wy = dop(va.z, vb.x, va.x, vb.z) * ir12;
+                            wz = dop(va.x, vb.y, va.y, vb.x) * ir12;
+                            const float s2 = fmaf(wx, wx, fmaf(wy, wy, fmaf(wz, wz, d.eps_theta)));
+                            const float c = fmaf(va.x, vb.x, fmaf(va.y, vb.y, va.z * vb.z)) * ir12;
+                            half_angles<false>(d, fminf(fmaxf(c, -1.f), 1.f), s2, sh, ch);
+                            const float se = sqrt_nr(s2);
+                            ise = se > 0.f ? div_nr(1.f, se) : 0.f;
+                            float rbh, rbl;
+                            rbar_halves(va.w, vb.w, rbh, rbl);
+                            pr_my[0] = rbh;
+                            pr_my[2] = rbl;
+                        }
+                        pa_my[0] = sh;
+                        pa_my[2] = ch;
+                    }
+                    __syncwarp();
+                    // step 2: groups of 16 pairs
+                    const int left = bp.n - p0;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (16 * h >= left) break;
+                        float2 x0, x1, z0, z1;
+                        if (FAST) {
+                            const float2 hr = pr2[8 * h + g];
+                            x0 = __fadd2_rn(hr, nR0);
+                            x1 = __fadd2_rn(hr, nR1);
+                            z0 = __fmul2_rn(x0, make_float2(-x0.x, -x0.y));
+                            z1 = __fmul2_rn(x1, make_float2(-x1.x, -x1.y));
+                        } else {
+                            const float4 hr = pr4[8 * h + g];
+                            const float2 hi = make_float2(hr.x, hr.y), lo = make_float2(hr.z, hr.w);
+                            x0 = __fadd2_rn(__fadd2_rn(hi, nR0), lo);
+                            x1 = __fadd2_rn(__fadd2_rn(hi, nR1), lo);
+                            z0 = __fmul2_rn(__fmul2_rn(x0, x0), dup(-eta_l));
+                            z1 = __fmul2_rn(__fmul2_rn(x1, x1), dup(-eta_l));
+                        }
+                        const float2 e0 = make_float2(ex2f(z0.x), ex2f(z0.y)), e1 = make_float2(ex2f(z1.x), ex2f(z1.y));
+                        float2 e0h, e0l, e1h, e1l, f0h, f0l, f1h, f1l;
+                        tf_split<!FAST>(e0, e0h, e0l);
+                        tf_split<!FAST>(e1, e1h, e1l);
+                        if (!FAST) {
+                            tf_split<true>(__fmul2_rn(x0, e0), f0h, f0l);
+                            tf_split<true>(__fmul2_rn(x1, e1), f1h, f1l);
+                        }
+                        const float4 sc = pa[8 * h + g];   // sin of the two pairs, cos of the two pairs
+                        float2 Tc[2], S0[2], S1[2];
+#pragma unroll
+                        for (int mc = 0; mc < CM; ++mc) {
+                            float C[4], X[4];
+                            mma8z(C, e0h.x, e0h.y, e1h.x, e1h.y, tl[mc].x, tl[mc].y);
+                            mma8(C, e0l.x, e0l.y, e1l.x, e1l.y, th[mc].x, th[mc].y);
+                            mma8(C, e0h.x, e0h.y, e1h.x, e1h.y, th[mc].x, th[mc].y);
+                            if (FAST) {
+                                // sum x T e = rho sum T e + sum (R_c - R) T e: rho enters in step 3
+                                mma8z(X, e0h.x, e0h.y, e1h.x, e1h.y, ul[mc].x, ul[mc].y);
+                                mma8(X, e0l.x, e0l.y, e1l.x, e1l.y, uh[mc].x, uh[mc].y);
+                                mma8(X, e0h.x, e0h.y, e1h.x, e1h.y, uh[mc].x, uh[mc].y);
+                            } else {
+                                mma8z(X, f0h.x, f0h.y, f1h.x, f1h.y, tl[mc].x, tl[mc].y);
+                                mma8(X, f0l.x, f0l.y, f1l.x, f1l.y, th[mc].x, th[mc].y);
+                                mma8(X, f0h.x, f0h.y, f1h.x, f1h.y, th[mc].x, th[mc].y);
+                            }
+#pragma unroll
+                            for (int P = 0; P < 2; ++P) {
+                                const float2 sh2 = dup(P ? sc.y : sc.x), ch2 = dup(P ? sc.w : sc.z);
+                                float2 y, p1, ef;   // y_m, y_m^(zeta - 1), sin_eps dy_m/dcos
+                                if (FAST) {
+                                    y = __ffma2_rn(sh2, chm[mc], __ffma2_rn(ch2, shm[mc], dup(0.5f)));
+                                    ef = __ffma2_rn(ch2, chm[mc], __fmul2_rn(make_float2(-sh2.x, -sh2.y), shm[mc]));
+                                    p1 = pow2_y(d.zeta - 1.f, y);
+                                } else {
+                                    const float2 ee = __ffma2_rn(sh2, chm[mc],
+                                                                 __fmul2_rn(make_float2(-ch2.x, -ch2.y), shm[mc]));
+                                    const float2 tt = __ffma2_rn(ee, ee, dup(-d.r_half));
+                                    y = __fadd2_rn(dup(1.f), make_float2(-tt.x, -tt.y));
+                                    ef = __fmul2_rn(ee, __ffma2_rn(ch2, chm[mc], __fmul2_rn(sh2, shm[mc])));
+                                    p1 = pow2_t<PW>(d.zlog1, d.zeta - 1.f, d.zeta_int - 1, tt);
+                                }
+                                const float2 U = __fmul2_rn(p1, y), Q = __fmul2_rn(p1, ef);
+                                const float2 Cp = P ? make_float2(C[2], C[3]) : make_float2(C[0], C[1]);
+                                const float2 Xp = P ? make_float2(X[2], X[3]) : make_float2(X[0], X[1]);
+                                S0[P] = mc ? __ffma2_rn(U, Cp, S0[P]) : __fmul2_rn(U, Cp);
+                                S1[P] = mc ? __ffma2_rn(U, Xp, S1[P]) : __fmul2_rn(U, Xp);
+                                Tc[P] = mc ? __ffma2_rn(Q, Cp, Tc[P]) : __fmul2_rn(Q, Cp);
+                            }
+                        }
+                        // slots permuted per part so that the lanes' stores fall on different banks
+#pragma unroll
+                        for (int P = 0; P < 2; ++P) {
+                            const int p = 16 * h + 8 * P + g;
+                            pts[t * 32 + (p ^ (4 * t))] = make_float2(Tc[P].x + Tc[P].y, S0[P].x + S0[P].y);
+                            pt1[t * 32 + (p ^ (8 * t))] = S1[P].x + S1[P].y;
+                        }
+                    }
+                    __syncwarp();
+                    // step 3: chain rule of the lane's pair and its two entries' sums
+                    float4 q1 = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float tr2 = 0.f;
+                    if (on) {
+                        float2 s = pts[lane];
+                        float S1 = pt1[lane];
+#pragma unroll
+                        for (int j = 1; j < 4; ++j) {
+                            s = __fadd2_rn(s, pts[j * 32 + (lane ^ (4 * j))]);
+                            S1 += pt1[j * 32 + (lane ^ (8 * j))];
+                        }
+                        if (FAST) S1 = fmaf(rho, s.y, S1);
+                        const float Fp = f1.x * f2.x;
+                        const float dTc = 2.f * d.zeta * Fp * ise * s.x;   // dT/dcos
+                        q1.x = dTc * wx;
+                        q1.y = dTc * wy;
+                        q1.z = dTc * wz;
+                        const float sf = s1 * Fp * S1, S02 = 2.f * s.y;
+                        q1.w = fmaf(f1.y * f2.x, S02, sf);                 // dT/dr1
+                        tr2 = fmaf(f1.x * f2.y, S02, sf);                  // dT/dr2
+                    }
+                    const int q0 = __shfl_sync(0xffffffffu, bp.q, 0);
+                    const int qd = bp.q - q0;                             // diagonal within the round
+                    const int nd = __shfl_sync(0xffffffffu, bp.q, 31) - q0 + 1;
+                    for (int c0 = 0; c0 < nd; c0 += nc) {
+                        const bool act = on && qd >= c0 && qd < c0 + nc;
+                        float4* cp = sq + (qd - c0) * cap;
+                        if (act) {
+                            float4 o = cp[k1];
+                            cp[k1] = make_float4(o.x + q1.x, o.y + q1.y, o.z + q1.z, o.w + q1.w);
+                        }
+                        __syncwarp();
+                        if (act) {
+                            float4 o = cp[k2];
+                            cp[k2] = make_float4(o.x - q1.x, o.y - q1.y, o.z - q1.z, o.w + tr2);
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+
+        // entries' gradients, scattered to the forces
+        float fx = 0.f, fy = 0.f, fz = 0.f;
+        float vv[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) vv[k] = 0.f;
+        for (int k = lane; k < n; k += 32) {
+            float4 z = sq[k];
+            for (int c = 1; c < nc; ++c) {
+                const float4 o = sq[c * cap + k];
+                z.x += o.x; z.y += o.y; z.z += o.z; z.w += o.w;
+            }
+            float4 v = sv[k];
+            float q0, q1, q2;
+            if (FAST) {
+                // v is the unit vector: q = (Z x u) / r + T u
+                const float r = sr[k], ir = rcpf(r);
+                q0 = fmaf(z.w, v.x, fmaf(z.y, v.z, -z.z * v.y) * ir);
+                q1 = fmaf(z.w, v.y, fmaf(z.z, v.x, -z.x * v.z) * ir);
+                q2 = fmaf(z.w, v.z, fmaf(z.x, v.y, -z.y * v.x) * ir);
+                v = make_float4(v.x * r, v.y * r, v.z * r, r);
+            } else {
+                const float ir = sx4[k].z, ir2 = ir * ir, tr = z.w * ir;
+                q0 = fmaf(tr, v.x, dop(z.y, v.z, z.z, v.y) * ir2);
+                q1 = fmaf(tr, v.y, dop(z.z, v.x, z.x, v.z) * ir2);
+                q2 = fmaf(tr, v.z, dop(z.x, v.y, z.y, v.x) * ir2);
+            }
+            fx += q0; fy += q1; fz += q2;
+            const int64_t j = w.nb_idx[sb + k].x;
+            atomicAdd(&F[3 * j + 0], -q0);
+            atomicAdd(&F[3 * j + 1], -q1);
+            atomicAdd(&F[3 * j + 2], -q2);
+            const float rv[3] = {v.x, v.y, v.z}, qq[3] = {q0, q1, q2};
+#pragma unroll
+            for (int aa = 0; aa < 3; ++aa)
+#pragma unroll
+                for (int bb = 0; bb < 3; ++bb) vv[3 * aa + bb] -= qq[aa] * rv[bb];
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            fx += __shfl_xor_sync(0xffffffffu, fx, o);
+            fy += __shfl_xor_sync(0xffffffffu, fy, o);
+            fz += __shfl_xor_sync(0xffffffffu, fz, o);
+        }
+        if (lane == 0) {
+            atomicAdd(&F[3 * i + 0], fx);
+            atomicAdd(&F[3 * i + 1], fy);
+            atomicAdd(&F[3 * i + 2], fz);
+        }
+        if (vir_atom) {
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < 9; ++k) vv[k] += __shfl_xor_sync(0xffffffffu, vv[k], o);
+            float val = vv[0];
+#pragma unroll
+            for (int k = 1; k < 9; ++k) if (lane == k) val = vv[k];
+            if (lane < 9) vir_atom[9 * i + lane] = val;
+        }
+    }
+}
+
 int sm_count()
 {
     int dev = 0, n = 0;
@@ -545,8 +936,10 @@ constexpr size_t kMaxSmem = 200 * 1024;
 
 }  // namespace
 
-// FAST needs exponents for which the splits' truncation stays below the hardware log2's error
+// FAST needs exponents for which the splits' truncation (descriptor) and |y|^(zeta - 1) in place of
+// the clamp at y = 0 (adjoint) stay below the hardware log2's error
 static bool desc_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 16.f; }
+static bool adj_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 2.f; }
 
 static size_t desc_smem(const Work& w, const DescDev& d, bool fast)
 {
@@ -556,6 +949,21 @@ static size_t desc_smem(const Work& w, const DescDev& d, bool fast)
 bool desc_mma_fits(const Work& w, const DescDev& d, bool fast)
 {
     return d.ang_kind == 0 && desc_smem(w, d, fast) <= kMaxSmem;
+}
+
+// four copies of the entries' sums when five CTAs per SM still fit, else fewer
+static int adj_copies(const Work& w, const DescDev& d, bool fast)
+{
+    int nc = 4;
+    while (nc > 1 && (size_t)kMW * adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total > 44 * 1024) nc /= 2;
+    return nc;
+}
+
+// one shell chunk and at most two sector chunks: the block's gradient tile stays in registers
+bool adj_mma_fits(const Work& w, const DescDev& d, bool fast)
+{
+    return d.ang_kind == 0 && d.n_ang_r <= 8 && d.n_theta <= 16 &&
+           (size_t)kMW * adj_mma_smem(d, w.cap, 1, adj_fast(d, fast)).total <= kMaxSmem;
 }
 
 cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_map, float* G_rows,
@@ -570,6 +978,21 @@ cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_
     if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8>) : run(k_desc_mma<false, 1, 8>);
     if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13>) : run(k_desc_mma<false, 1, 13>);
     return two ? run(k_desc_mma<false, 2, 0>) : run(k_desc_mma<false, 1, 0>);
+}
+
+cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows, float* F, float* vir_atom,
+                           bool fast, cudaStream_t s)
+{
+    if (!adj_mma_fits(w, d, fast)) return cudaErrorNotSupported;
+    if (w.N == 0) return cudaSuccess;
+    int nc = adj_copies(w, d, fast);
+    const size_t smem = (size_t)kMW * adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total;
+    auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, g_rows, F, vir_atom, nc); };
+    const bool two = d.n_theta > 8;
+    if (adj_fast(d, fast)) return two ? run(k_adj_mma<true, 2, 0>) : run(k_adj_mma<true, 1, 0>);
+    if (d.zeta >= 33.f) return two ? run(k_adj_mma<false, 2, 8>) : run(k_adj_mma<false, 1, 8>);
+    if (d.zeta >= 17.f) return two ? run(k_adj_mma<false, 2, 13>) : run(k_adj_mma<false, 1, 13>);
+    return two ? run(k_adj_mma<false, 2, 0>) : run(k_adj_mma<false, 1, 0>);
 }
 
 }  // namespace panna

@@ -64,10 +64,10 @@ struct Arena {
     }
 };
 
-constexpr int kNumVariants = 6;   // most variants of one descriptor-family kernel
-// variants per kernel: descriptor 0..5, adjoint 0..5, JVP 0..4; the matrix form's number (-1: none)
-constexpr int kMmaVariant[3] = {5, -1, -1};
-constexpr int kKindVariants[3] = {6, 6, 5};
+constexpr int kNumVariants = 7;   // most variants of one descriptor-family kernel
+// variants per kernel: descriptor 0..5, adjoint 0..6, JVP 0..4; the matrix form's number (-1: none)
+constexpr int kMmaVariant[3] = {5, 6, -1};
+constexpr int kKindVariants[3] = {6, 7, 5};
 const char* kStages[] = {"neighbors", "descriptor", "mlp", "adjoint", "forces", "jvp", "mlp_grad", "loss"};
 constexpr int kNumStages = 8;
 
@@ -381,14 +381,15 @@ template <class Launch>
 int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int prec, int kind, cudaStream_t s,
                    Launch launch, bool acc);
 
-// The matrix form (descriptor 5) where it applies, without measuring anything: from
-// kSplitAtoms atoms on it was the fastest on every workload measured, from 5-29-atom molecules
+// The matrix forms (descriptor 5, adjoint 6) where they apply, without measuring anything: from
+// kSplitAtoms atoms on they were the fastest on every workload measured, from 5-29-atom molecules
 // (descriptor 0.144 -> 0.068 ms for 1024 of them) to the 1M-atom box (below that size the old kernels
 // spread one atom over several warps).
 int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
 {
     if (w.N < kSplitAtoms) return -1;
     if (kind == KV_DESC && desc_mma_fits(w, c->d, !acc)) return 5;
+    if (kind == KV_ADJ && adj_mma_fits(w, c->d, !acc)) return 6;
     return -1;
 }
 
@@ -423,7 +424,7 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
     const int fallback = (sys->n_atoms < kSplitAtoms || ext) ? 0 : (kind == KV_ADJ ? 5 : 2);
     if (!c->autotune || c->async || sys->n_atoms == 0) return fallback;
     float ms[kNumVariants] = {};
-    const bool mma = kind == KV_DESC && desc_mma_fits(w, c->d, !acc);
+    const bool mma = kind == KV_DESC ? desc_mma_fits(w, c->d, !acc) : kind == KV_ADJ && adj_mma_fits(w, c->d, !acc);
     auto candidate = [&](int v) {
         if (v == kMmaVariant[kind]) return mma;
         return !ext || v < 2;

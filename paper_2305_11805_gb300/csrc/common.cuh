@@ -163,11 +163,14 @@ cudaError_t launch_descriptor_bf16(const Work& w, const DescDev& d, __nv_bfloat1
                                    const int32_t* row_map, int variant, cudaStream_t s, int* launches, bool fast);
 // Matrix form of the angular kernels (angular_mma.cu): the products over sectors and shells on the
 // warp-level tensor cores.  cudaErrorNotSupported when the descriptor or the batch is outside what
-// they take (desc_mma_fits).  Rows in FP32 (G_rows) or as BF16 hi (+ lo) parts.
+// they take (desc_mma_fits, adj_mma_fits).  Rows in FP32 (G_rows) or as BF16 hi (+ lo) parts.
 // fast: the forms of the BF16 networks; otherwise those of the FP32 ones.
 bool desc_mma_fits(const Work& w, const DescDev& d, bool fast);
+bool adj_mma_fits(const Work& w, const DescDev& d, bool fast);
 cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_map, float* G_rows,
                             __nv_bfloat16* Gh, __nv_bfloat16* Gl, bool fast, cudaStream_t s);
+cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows, float* F, float* vir_atom,
+                           bool fast, cudaStream_t s);
 cudaError_t launch_jvp(const Work& w, const DescDev& d, const float* u, float* wdot_rows, bool acc, cudaStream_t s,
                        int* launches, int variant = 0);
 

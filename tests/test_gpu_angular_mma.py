@@ -44,6 +44,15 @@ def test_matrix_forms_match(shape):
     Go = O.batch(system, desc, archs, theta, want_G=True)["G"]
     pot = P.Potential(desc, archs)
     sysd = P.DeviceSystem(system)
+    th = torch.as_tensor(theta, dtype=torch.float32, device="cuda")
+
+    def forces(adjoint, mode):
+        P.panna_set_angular_precision(pot.ctx, mode)
+        P.panna_set_tuning(pot.ctx, "descriptor", 0)
+        P.panna_set_tuning(pot.ctx, "adjoint", adjoint)
+        _, _, F, V = pot.energy_forces(sysd, th, P.PANNA_MLP_FP32)
+        return F.cpu().numpy().astype(np.float64), V.cpu().numpy()
+
     P.panna_set_tuning(pot.ctx, "descriptor", 5)
     for mode, tol in ((0, H.TOL_G), (2, 3e-5)):
         P.panna_set_angular_precision(pot.ctx, mode)
@@ -52,3 +61,11 @@ def test_matrix_forms_match(shape):
         err = H.descriptor_error(G.cpu().numpy().astype(np.float64), Go, desc)
         print("%s mode %d: descriptors %.3g" % (name, mode, err))
         assert err <= tol
+    for mode, tol in ((0, 2e-5), (2, 5e-4)):
+        F0, V0 = forces(0, 0 if mode == 0 else 2)
+        F6, V6 = forces(6, mode)
+        err, rms = H.force_error(F6, F0)
+        verr = float(np.abs(V6 - V0).max() / (np.abs(V0).max() + 1e-30))
+        print("%s mode %d: forces %.3g (rms %.3g), virial %.3g" % (name, mode, err, rms, verr))
+        assert (err if rms > 1e-6 else np.abs(F6).max()) <= (tol if rms > 1e-6 else 1e-5)
+        assert verr <= 10 * tol
