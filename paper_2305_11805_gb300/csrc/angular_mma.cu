@@ -168,57 +168,6 @@ __device__ __forceinline__ void half_pair(float c, float cl, float& h, float& l)
     l = h > 0.f ? fmaf(0.5f, ql, fmaf(-h, h, qh)) * (0.5f * rcpf(h)) : 0.f;
 }
 
-// The pairs of one species block as positions p = 0 .. n - 1: entries of the smaller segment (M of
-// them) against those of the larger one by diagonals, k1 = r, k2 = r + q (mod) with q = p / M,
-// r = p mod M; inside one segment (k, k + q + 1 mod M), each unordered pair once.  All positions of
-// one q have distinct first entries and distinct second entries.  A lane starts at p = lane and
-// steps by 32.
-struct BlockPairs {
-    int b1, b2, M, mod, off, n;
-    int q, r, dq, dr;
-    __device__ __forceinline__ BlockPairs(int sa, int na, int sb, int nb, bool same, int lane)
-    {
-        const bool sw = na > nb;
-        M = max(same ? na : (sw ? nb : na), 1);
-        mod = same ? na : (sw ? na : nb);
-        b1 = same || !sw ? sa : sb;
-        b2 = same || sw ? sa : sb;
-        off = same ? 1 : 0;
-        n = same ? na * (na - 1) / 2 : na * nb;
-        // quotients of small integers: the exact one is at least 1/(2M) from the next integer
-        const float inv = rcpf((float)M);
-        q = (int)(((float)lane + 0.5f) * inv);
-        r = lane - q * M;
-        dq = (int)(32.5f * inv);
-        dr = 32 - dq * M;
-    }
-    __device__ __forceinline__ void get(bool on, int& k1, int& k2) const
-    {
-        const int s = r + q + off;
-        const int y = s >= mod ? s - mod : s;
-        k1 = on ? b1 + r : 0;
-        k2 = on ? b2 + y : 0;
-    }
-    __device__ __forceinline__ void next()
-    {
-        r += dr;
-        q += dq;
-        if (r >= M) { r -= M; ++q; }
-    }
-};
-
-// species segments of an atom's entries (grouped by species) into seg[0..S]
-__device__ __forceinline__ void species_segments(const DescDev& d, const int2* __restrict__ idx, int n, int* seg,
-                                                 int lane)
-{
-    // entry k starts the segments of every species after its predecessor's up to its own
-    for (int k = lane; k <= n; k += 32) {
-        const int s1 = k < n ? meta_species(idx[k].y) : d.S;
-        const int s0 = k > 0 ? meta_species(idx[k - 1].y) : -1;
-        for (int s = s0 + 1; s <= s1; ++s) seg[s] = k;
-    }
-}
-
 // ------------------------------------------------------------------ descriptor
 
 // Arithmetic of the descriptor kernel.  FAST: see the file comment.  PAIR (FP32 networks, whose
@@ -887,27 +836,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
 #pragma unroll
                 for (int bb = 0; bb < 3; ++bb) vv[3 * aa + bb] -= qq[aa] * rv[bb];
         }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            fx += __shfl_xor_sync(0xffffffffu, fx, o);
-            fy += __shfl_xor_sync(0xffffffffu, fy, o);
-            fz += __shfl_xor_sync(0xffffffffu, fz, o);
-        }
-        if (lane == 0) {
-            atomicAdd(&F[3 * i + 0], fx);
-            atomicAdd(&F[3 * i + 1], fy);
-            atomicAdd(&F[3 * i + 2], fz);
-        }
-        if (vir_atom) {
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1)
-#pragma unroll
-                for (int k = 0; k < 9; ++k) vv[k] += __shfl_xor_sync(0xffffffffu, vv[k], o);
-            float val = vv[0];
-#pragma unroll
-            for (int k = 1; k < 9; ++k) if (lane == k) val = vv[k];
-            if (lane < 9) vir_atom[9 * i + lane] = val;
-        }
+        add_centre(w, i, fx, fy, fz, vv, F, vir_atom, lane);
     }
 }
 

@@ -387,6 +387,7 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
 // spread one atom over several warps).
 int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
 {
+    if (c->d.ang_kind != 0) return 0;   // the standard BP term has one kernel
     if (w.N < kSplitAtoms) return -1;
     if (kind == KV_DESC && desc_mma_fits(w, c->d, !acc)) return 5;
     if (kind == KV_ADJ && adj_mma_fits(w, c->d, !acc)) return 6;
