@@ -514,22 +514,31 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
     const bool tc = rq.prec == PANNA_MLP_BF16 || rq.prec == PANNA_MLP_BF16_FAST;
     const int tfm = tf32_mask(c, tc, grad);
     const bool tf = tfm != 0;
+    bool fused = false;
     if (tc) {
         // BF16 operands on the tensor cores: energies and dE/dG together
         CU(mlp_bf16_energy_grad(c->plan, L.mb, rq.theta, N, L.tc_ws, rq.prec == PANNA_MLP_BF16, L.E_rows, L.g,
                                 L.w.status, s, &nl, g16_ready));
-    } else if (tf) {
-        // FP32 networks: first-layer products on the tensor cores (TF32 parts), the rest on CUDA cores
-        CU(tf32_prepare(c->plan, L.mb, rq.theta, N, L.tf_ws, tfm, s, &nl));
-        if (tfm & TF32_FWD) CU(tf32_forward1(c->plan, L.mb, N, L.tf_ws, tfm, L.w.status, s, &nl));
-        CU(mlp_forward(c->plan, L.mb, rq.theta, N, s, &nl, (tfm & TF32_FWD) ? 1 : 0));
-        CU(mlp_energy_rows(c->plan, L.mb, N, L.E_rows, s, &nl));
     } else {
-        CU(mlp_forward(c->plan, L.mb, rq.theta, N, s, &nl));
-        CU(mlp_energy_rows(c->plan, L.mb, N, L.E_rows, s, &nl));
+        // FP32 networks: first-layer products of the mask on the tensor cores (TF32 parts), the rest on
+        // CUDA cores; small batches take forward pass, energies and input gradient in one launch
+        if (tf) CU(tf32_prepare(c->plan, L.mb, rq.theta, N, L.tf_ws, tfm, s, &nl));
+        if (!(tfm & TF32_FWD)) {
+            const cudaError_t es = mlp_small_rows(c->plan, L.mb, rq.theta, N, L.E_rows, need_forces ? L.g : nullptr,
+                                                  grad, s, &nl);
+            if (es != cudaErrorNotSupported) {
+                CU(es);
+                fused = true;
+            }
+        }
+        if (!fused) {
+            if (tfm & TF32_FWD) CU(tf32_forward1(c->plan, L.mb, N, L.tf_ws, tfm, L.w.status, s, &nl));
+            CU(mlp_forward(c->plan, L.mb, rq.theta, N, s, &nl, (tfm & TF32_FWD) ? 1 : 0));
+            CU(mlp_energy_rows(c->plan, L.mb, N, L.E_rows, s, &nl));
+        }
     }
     if (need_forces) {
-        if (!tc) {
+        if (!tc && !fused) {
             CU(mlp_input_grad(c->plan, L.mb, rq.theta, N, L.g, s, &nl));
         }
         stage_mark(c, 3, s);

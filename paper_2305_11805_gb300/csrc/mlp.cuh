@@ -52,6 +52,12 @@ cudaError_t mlp_energy_rows(const MlpPlan& p, const MlpBuffers& b, int64_t N, fl
 // seeded: b.Ab already holds the output seeds (rows, stride ld[L]) instead of dE/da_L = 1
 cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, float* g,
                            cudaStream_t s, int* launches, float** ab1 = nullptr, bool seeded = false);
+// Small batches (at most kSmallBatch rows, one output): forward pass, energies and, with g, the input
+// gradient in one launch (mlp_small.cu); keep: Z and A of every layer are written as mlp_forward does.
+// cudaErrorNotSupported for other batches and for networks too wide for its shared memory.
+constexpr int64_t kSmallBatch = 2048;
+cudaError_t mlp_small_rows(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, float* E_rows,
+                           float* g, bool keep, cudaStream_t s, int* launches);
 // BF16 tensor-core networks (mlp_tc.cu): energies and input gradients; ws from tc_workspace_bytes
 size_t tc_workspace_bytes(const MlpPlan& p, int64_t N, bool split);
 // g16_ready: the descriptor kernel already wrote the BF16 operand rows (tc_g16), else the FP32
