@@ -182,6 +182,8 @@ void carve(panna_ctx* c, Arena& a, int64_t N, int64_t C, bool train, bool bf16, 
     w.row_of_atom = a.take<int32_t>(N);
     w.atom_of_row = a.take<int32_t>(N);
     w.seg_off = a.take<int32_t>(S + 1);
+    w.tile_start = a.take<int32_t>(S + 1);
+    w.rows_ready = false;
     w.blk_counts = a.take<int32_t>(((N + 1023) / 1024 + 1) * S);
     w.split_part = nullptr;
     w.split_rows = 0;
@@ -207,7 +209,7 @@ void carve(panna_ctx* c, Arena& a, int64_t N, int64_t C, bool train, bool bf16, 
     b.Ab = a.take<float>((size_t)N * p.max_hidden);
     b.Ab2 = a.take<float>((size_t)N * p.max_hidden);
     b.seg_off = w.seg_off;
-    b.tile_start = a.take<int32_t>(S + 1);
+    b.tile_start = w.tile_start;
     b.splits = kSplits;
     if (bf16) L.tc_ws = a.take<char>(tc_workspace_bytes(p, N, true));
     if (const int m = tf32_mask(c, bf16, train)) L.tf_ws = a.take<char>(tf32_workspace_bytes(p, N, m));
@@ -285,21 +287,26 @@ void stage_mark(panna_ctx* c, int k, cudaStream_t s)
     }
 }
 
+// The error that a status word holds (and its message)
+panna_status status_error(const panna_ctx* c, const DevStatus& d)
+{
+    if (d.code == 0) return PANNA_OK;
+    if (d.code == PANNA_ERR_NEIGHBOR_OVERFLOW)
+        return fail(PANNA_ERR_NEIGHBOR_OVERFLOW, "atom %d has %d neighbours, capacity %d", d.bad_index, d.need_cap,
+                    c->cap);
+    if (d.code == PANNA_ERR_BAD_INPUT)
+        return fail(PANNA_ERR_BAD_INPUT, "invalid input at index %d (species out of range, non-finite or coincident"
+                    " positions, or singular cell)", d.bad_index);
+    return fail((panna_status)d.code, "device error %d at index %d", d.code, d.bad_index);
+}
+
 // Reads the status word (synchronising); returns it and the overflow requirement.
 panna_status collect(panna_ctx* c, const Layout& L, cudaStream_t s, int* need)
 {
     CU(cudaMemcpyAsync(c->h_status, L.w.status, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
     *need = c->h_status->need_cap;
-    if (c->h_status->code == 0) return PANNA_OK;
-    if (c->h_status->code == PANNA_ERR_NEIGHBOR_OVERFLOW)
-        return fail(PANNA_ERR_NEIGHBOR_OVERFLOW, "atom %d has %d neighbours, capacity %d", c->h_status->bad_index,
-                    c->h_status->need_cap, c->cap);
-    if (c->h_status->code == PANNA_ERR_BAD_INPUT)
-        return fail(PANNA_ERR_BAD_INPUT, "invalid input at index %d (species out of range, non-finite or coincident"
-                    " positions, or singular cell)", c->h_status->bad_index);
-    return fail((panna_status)c->h_status->code, "device error %d at index %d", c->h_status->code,
-                c->h_status->bad_index);
+    return status_error(c, *c->h_status);
 }
 
 // each stage lasts from its mark to the next mark in time (the last one to the end event)
@@ -489,7 +496,6 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
             return PANNA_OK;
         }
         CU(species_order(L.w, c->d.S, s, &nl));
-        CU(mlp_tiles(c->plan, L.w.seg_off, L.mb.tile_start, s, &nl));
         stage_mark(c, 1, s);
         int dummy = 0;
         const int v = tuned_variant(c, sys, L.w, rq.prec, KV_DESC, s, [&](int vv) {
@@ -643,6 +649,7 @@ panna_status md_build(panna_ctx* c, const panna_system* sys, Layout& L, Work& wc
     dc.rc = (float)dc.rc_d;
     int nl = 0;
     CU(build_neighbors(wc, dc, s, &nl));
+    L.w.rows_ready = L.w.rows_ready || wc.rows_ready;   // the species do not change
     CU(cudaMemcpyAsync(L.pos_ref, sys->pos, sizeof(double) * 3 * (size_t)sys->n_atoms, cudaMemcpyDeviceToDevice, s));
     return PANNA_OK;
 }
@@ -876,25 +883,35 @@ panna_status panna_md_run(panna_ctx* c, const panna_system* sys, double* vel, co
         ++builds;
         break;
     }
+    // Each step: integrate, read the status word (the step before's errors, this step's stale flag),
+    // forces.  With a skin the forces are enqueued before the status is waited for, so that the host's
+    // wait and launches overlap the GPU's work; a stale list (rare) is rebuilt and the forces redone.
+    // The closing half kick of a step runs in the next step's integration kernel.
     for (int64_t t = 0; t < n_steps; ++t) {
-        CU(launch_md_baoa(N, sys->species, ms, pos, vel, F, p->dt, c1, c2, thermostat, p->seed, p->step0 + t,
-                          L.pos_ref, lim2, &L.w.status->stale, s));
-        const panna_status st = md_status(c, L, s, &stale, &need);
-        if (st != PANNA_OK) {
-            collect(c, L, s, &need);
-            return fail(st, "step %lld: %s (raise the neighbour capacity and restart)", (long long)t,
+        CU(launch_md_baoa(L.w, ms, pos, vel, F, p->dt, c1, c2, thermostat, p->seed, p->step0 + t, t > 0, L.pos_ref,
+                          lim2, s));
+        CU(cudaMemcpyAsync(c->h_status, L.w.status, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
+        CU(cudaEventRecord(c->tev[2], s));
+        const bool ahead = p->skin > 0.0;
+        if (ahead) ST(run_once(c, sys, rq, L, s));
+        CU(cudaEventSynchronize(c->tev[2]));
+        const DevStatus now = *c->h_status;
+        if (now.code != PANNA_OK) {
+            CU(cudaStreamSynchronize(s));
+            status_error(c, now);
+            return fail((panna_status)now.code, "step %lld: %s (raise the neighbour capacity and restart)", (long long)t,
                         panna_last_error());
         }
-        if (stale || p->skin == 0.0) {
+        if (now.stale || !ahead) {
             ST(md_build(c, sys, L, wc, p->skin, s));
             ++builds;
+            ST(run_once(c, sys, rq, L, s));
         }
-        ST(run_once(c, sys, rq, L, s));
-        CU(launch_md_b(N, sys->species, ms, vel, F, p->dt, s));
         if (E_traj)
             CU(cudaMemcpyAsync(E_traj + t * sys->n_cfg, E_cfg, sizeof(double) * (size_t)sys->n_cfg,
                                cudaMemcpyDeviceToDevice, s));
     }
+    if (n_steps > 0) CU(launch_md_b(N, sys->species, ms, vel, F, p->dt, s));
     if (n_builds) *n_builds = builds;
     return collect(c, L, s, &need);
 }
@@ -1090,7 +1107,6 @@ panna_status panna_qeq_energy_forces(panna_ctx* c, const panna_system* sys, cons
         stage_mark(c, 0, s);
         CU(build_neighbors(L.w, c->d, s, &nl));
         CU(species_order(L.w, c->d.S, s, &nl));
-        CU(mlp_tiles(c->plan, L.w.seg_off, L.mb.tile_start, s, &nl));
         stage_mark(c, 1, s);
         int dummy = 0;
         const int vd = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {
@@ -1164,7 +1180,6 @@ panna_status panna_qeq_loss_grad(panna_ctx* c, const panna_system* sys, const fl
         stage_mark(c, 0, s);
         CU(build_neighbors(L.w, c->d, s, &nl));
         CU(species_order(L.w, c->d.S, s, &nl));
-        CU(mlp_tiles(c->plan, L.w.seg_off, L.mb.tile_start, s, &nl));
         stage_mark(c, 1, s);
         int dummy = 0;
         const int vd = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_DESC, s, [&](int vv) {

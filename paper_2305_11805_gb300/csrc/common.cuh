@@ -122,6 +122,8 @@ struct Work {
     int32_t* row_of_atom;        // [N]
     int32_t* atom_of_row;        // [N]
     int32_t* seg_off;            // [S+1] rows of species s: seg_off[s]..seg_off[s+1]-1
+    int32_t* tile_start;         // [S+1] row tiles of the networks (mlp.cuh) before each species
+    bool rows_ready;             // host: the species order of this batch is in place
     int32_t* blk_counts;         // species sort scratch
     // small batches: per-split partial descriptor rows [split_rows / N][N][D] (null: no splits)
     float* split_part;
@@ -139,9 +141,12 @@ constexpr int64_t kSplitTargetWarps = 2432;
 int64_t scan_scratch_elems(int64_t n);
 cudaError_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s, int* launches);
 cudaError_t build_neighbors(Work& w, const DescDev& d, cudaStream_t s, int* launches);
+// rows by species, their offsets and tiles; nothing to do when w.rows_ready (the search of a small
+// batch leaves them, and in dynamics the species stay)
 cudaError_t species_order(Work& w, int S, cudaStream_t s, int* launches);
 // Verlet list: `cand` holds the candidates of a build with cutoff rc + skin (its nb_count,
-// nb_idx, cap); writes w's neighbour slots for cutoff d.rc at the current positions
+// nb_idx, cap); writes w's neighbour slots for cutoff d.rc at the folded positions in w.pos_hi / pos_lo
+// (left there by the build, then by every integration step)
 cudaError_t refresh_neighbors(const Work& cand, Work& w, const DescDev& d, cudaStream_t s, int* launches);
 cudaError_t export_neighbors(const Work& w, int64_t* off, int64_t* nbr_j, int32_t* shift, int64_t cap_total, cudaStream_t s, int* launches);
 
@@ -246,9 +251,9 @@ cudaError_t launch_qeq_response(const QeqDev& qp, const Work& w, const float* ou
 // Langevin dynamics (md.cu): per species a = (eV/A)/m in A/fs^2 and the thermal velocity
 // scale sigma = sqrt(kB T a) in A/fs
 struct MdSpecies { double acc[kMaxSpecies]; double sigma[kMaxSpecies]; };
-cudaError_t launch_md_baoa(int64_t N, const int32_t* species, const MdSpecies& ms, double* pos, double* vel,
-                           const float* F, double dt, double c1, double c2, int thermostat, uint64_t seed,
-                           int64_t step, const double* pos_ref, double lim2, int32_t* stale, cudaStream_t s);
+cudaError_t launch_md_baoa(const Work& w, const MdSpecies& ms, double* pos, double* vel, const float* F, double dt,
+                           double c1, double c2, int thermostat, uint64_t seed, int64_t step, bool pending_b,
+                           const double* pos_ref, double lim2, cudaStream_t s);
 cudaError_t launch_md_b(int64_t N, const int32_t* species, const MdSpecies& ms, double* vel, const float* F,
                         double dt, cudaStream_t s);
 

@@ -28,50 +28,67 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
     return c;
 }
 
-// three standard normals of atom a at step t (Box-Muller on u = (x + 1/2) 2^-32)
-__device__ __forceinline__ void gauss3(uint64_t seed, int64_t a, int64_t t, double g[3])
+// component d of the three standard normals of atom a at step t: Box-Muller on u = (x + 1/2) 2^-32,
+// components 0 and 1 from the first two words, 2 from the others
+__device__ __forceinline__ double gauss_component(uint64_t seed, int64_t a, int64_t t, int d)
 {
     const uint4 x = philox4x32_10(make_uint4((uint32_t)a, (uint32_t)((uint64_t)a >> 32), (uint32_t)t,
                                              (uint32_t)((uint64_t)t >> 32)),
                                   make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
     const double s32 = 1.0 / 4294967296.0;
-    const double u0 = ((double)x.x + 0.5) * s32, u1 = ((double)x.y + 0.5) * s32;
-    const double u2 = ((double)x.z + 0.5) * s32, u3 = ((double)x.w + 0.5) * s32;
-    const double r01 = sqrt(-2.0 * log(u0)), r23 = sqrt(-2.0 * log(u2));
-    double s1, c1, s3, c3;
-    sincospi(2.0 * u1, &s1, &c1);
-    sincospi(2.0 * u3, &s3, &c3);
-    g[0] = r01 * c1;
-    g[1] = r01 * s1;
-    g[2] = r23 * c3;
+    const double u = ((double)(d < 2 ? x.x : x.z) + 0.5) * s32, w = ((double)(d < 2 ? x.y : x.w) + 0.5) * s32;
+    double sn, cs;
+    sincospi(2.0 * w, &sn, &cs);
+    return sqrt(-2.0 * log(u)) * (d == 1 ? sn : cs);
 }
 
-// B A O A: v += dt/2 a F; x += dt/2 v; v = c1 v + c2 sigma g; x += dt/2 v.  With a
-// reference (positions of the last neighbour build), an atom that has moved more than
-// sqrt(lim2) since then raises *stale.
+// (B of the step before when pending) B A O A: v += dt/2 a F; x += dt/2 v; v = c1 v + c2 sigma g;
+// x += dt/2 v.  Four lanes per atom, one per component: the normals' FP64 logarithm, root and sine are
+// the kernel's time (one lane per atom took all three in turn: 10 -> 5 us).  With a reference (positions
+// of the last neighbour build), an atom that has moved more than sqrt(lim2) since then raises *stale,
+// and the positions folded with the lattice offsets of that build (wrap) go to pos_hi / pos_lo for the
+// list's refresh, so the image shifts stored with the candidates stay valid while atoms move.
 __global__ void k_md_baoa(int64_t N, const int32_t* __restrict__ species, MdSpecies ms, double* __restrict__ pos,
                           double* __restrict__ vel, const float* __restrict__ F, double dt, double c1, double c2,
-                          int thermostat, uint64_t seed, int64_t step, const double* __restrict__ pos_ref,
-                          double lim2, int32_t* __restrict__ stale)
+                          int thermostat, uint64_t seed, int64_t step, int pending_b,
+                          const double* __restrict__ pos_ref, double lim2, int32_t* __restrict__ stale,
+                          const int32_t* __restrict__ atom_cfg, const CfgGeom* __restrict__ geom,
+                          const int32_t* __restrict__ wrap, float4* __restrict__ pos_hi, float4* __restrict__ pos_lo)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int sp = species[i];
-    const double a = ms.acc[sp], sig = ms.sigma[sp];
-    double g[3] = {0.0, 0.0, 0.0};
-    if (thermostat) gauss3(seed, i, step, g);
-    double d2 = 0.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        double v = vel[3 * i + d] + 0.5 * dt * (double)F[3 * i + d] * a;
-        double x = pos[3 * i + d] + 0.5 * dt * v;
-        if (thermostat) v = c1 * v + c2 * sig * g[d];
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = idx >> 2;
+    const int lane = threadIdx.x & 31, d = lane & 3, q = lane & ~3;
+    const bool on = i < N;
+    double x = 0.0, e2 = 0.0;
+    if (on && d < 3) {
+        const int sp = species[i];
+        const double a = ms.acc[sp], f = 0.5 * dt * (double)F[3 * i + d] * a;
+        double v = vel[3 * i + d];
+        if (pending_b) v += f;
+        v += f;
+        x = pos[3 * i + d] + 0.5 * dt * v;
+        if (thermostat) v = c1 * v + c2 * ms.sigma[sp] * gauss_component(seed, i, step, d);
         x += 0.5 * dt * v;
         vel[3 * i + d] = v;
         pos[3 * i + d] = x;
-        if (pos_ref) { const double e = x - pos_ref[3 * i + d]; d2 += e * e; }
+        const double e = x - pos_ref[3 * i + d];
+        e2 = e * e;
     }
-    if (pos_ref && d2 > lim2) *stale = 1;
+    float h = 0.f, l = 0.f;
+    if (on && d < 3) {
+        const CfgGeom& g = geom[atom_cfg[i]];
+        const double xw = x + wrap[3 * i] * g.cell[d] + wrap[3 * i + 1] * g.cell[3 + d] + wrap[3 * i + 2] * g.cell[6 + d];
+        h = (float)xw;
+        l = (float)(xw - h);
+    }
+    const double s0 = __shfl_sync(0xffffffffu, e2, q), s1 = __shfl_sync(0xffffffffu, e2, q + 1),
+                 s2 = __shfl_sync(0xffffffffu, e2, q + 2);
+    const float h1 = __shfl_sync(0xffffffffu, h, q + 1), h2 = __shfl_sync(0xffffffffu, h, q + 2);
+    const float l1 = __shfl_sync(0xffffffffu, l, q + 1), l2 = __shfl_sync(0xffffffffu, l, q + 2);
+    if (on && d == 0) {
+        if ((s0 + s1) + s2 > lim2) *stale = 1;
+        pos_hi[i] = make_float4(h, h1, h2, pos_hi[i].w);
+        pos_lo[i] = make_float4(l, l1, l2, 0.f);
+    }
 }
 
 // B: v += dt/2 a F
@@ -85,13 +102,15 @@ __global__ void k_md_b(int64_t N, const int32_t* __restrict__ species, MdSpecies
     for (int d = 0; d < 3; ++d) vel[3 * i + d] += 0.5 * dt * (double)F[3 * i + d] * a;
 }
 
-cudaError_t launch_md_baoa(int64_t N, const int32_t* species, const MdSpecies& ms, double* pos, double* vel,
-                           const float* F, double dt, double c1, double c2, int thermostat, uint64_t seed,
-                           int64_t step, const double* pos_ref, double lim2, int32_t* stale, cudaStream_t s)
+cudaError_t launch_md_baoa(const Work& w, const MdSpecies& ms, double* pos, double* vel, const float* F, double dt,
+                           double c1, double c2, int thermostat, uint64_t seed, int64_t step, bool pending_b,
+                           const double* pos_ref, double lim2, cudaStream_t s)
 {
-    if (N == 0) return cudaSuccess;
-    k_md_baoa<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, species, ms, pos, vel, F, dt, c1, c2, thermostat, seed,
-                                                          step, pos_ref, lim2, stale);
+    if (w.N == 0) return cudaSuccess;
+    k_md_baoa<<<(unsigned)((4 * w.N + 255) / 256), 256, 0, s>>>(w.N, w.sys->species, ms, pos, vel, F, dt, c1, c2,
+                                                                thermostat, seed, step, pending_b ? 1 : 0, pos_ref,
+                                                                lim2, &w.status->stale, w.atom_cfg, w.geom, w.wrap,
+                                                                w.pos_hi, w.pos_lo);
     return cudaGetLastError();
 }
 

@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "mlp.cuh"
 
 namespace panna {
 
@@ -160,12 +161,12 @@ __device__ __forceinline__ double warp_max_d(double v)
     return v;
 }
 
-__global__ void __launch_bounds__(kCfgWarps * 32)
-k_cfg_geom(panna_system sys, double rc, CfgGeom* __restrict__ geom, int64_t* __restrict__ cfg_cells, DevStatus* st)
+// Geometry of configuration c by one warp: frame and inverse, grid of cells, image shifts; returns the
+// number of cells.  Axes (and cofactors) go to lanes of their own: FP64 divisions and square roots take
+// hundreds of cycles each on this GPU, and one lane doing all of them was 11 us.
+__device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc, int64_t c, CfgGeom* __restrict__ geom,
+                                             DevStatus* st, int lane)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t c = (int64_t)blockIdx.x * kCfgWarps + (threadIdx.x >> 5);
-    if (c >= sys.n_cfg) return;
     const int64_t a0 = sys.atom_off[c], a1 = sys.atom_off[c + 1];
     int per[3];
     for (int a = 0; a < 3; ++a) per[a] = sys.pbc[3 * c + a] ? 1 : 0;
@@ -218,51 +219,69 @@ k_cfg_geom(panna_system sys, double rc, CfgGeom* __restrict__ geom, int64_t* __r
             g.sh_lo[lane][d] = (float)(S - (double)sh);
         }
     }
-    if (lane != 0) return;
-    for (int k = 0; k < 9; ++k) { g.cell[k] = frame[k]; g.cinv[k] = finv[k]; }
-    // perpendicular widths of the frame
-    const double* A = frame; const double* B = frame + 3; const double* Cc = frame + 6;
-    double bxc[3] = {B[1] * Cc[2] - B[2] * Cc[1], B[2] * Cc[0] - B[0] * Cc[2], B[0] * Cc[1] - B[1] * Cc[0]};
-    double cxa[3] = {Cc[1] * A[2] - Cc[2] * A[1], Cc[2] * A[0] - Cc[0] * A[2], Cc[0] * A[1] - Cc[1] * A[0]};
-    double axb[3] = {A[1] * B[2] - A[2] * B[1], A[2] * B[0] - A[0] * B[2], A[0] * B[1] - A[1] * B[0]};
-    double vol = fabs(A[0] * bxc[0] + A[1] * bxc[1] + A[2] * bxc[2]);
-    double h[3] = {vol / sqrt(bxc[0] * bxc[0] + bxc[1] * bxc[1] + bxc[2] * bxc[2]),
-                   vol / sqrt(cxa[0] * cxa[0] + cxa[1] * cxa[1] + cxa[2] * cxa[2]),
-                   vol / sqrt(axb[0] * axb[0] + axb[1] * axb[1] + axb[2] * axb[2])};
+    // lane a (0..2): axis a
+    const int ax = lane < 3 ? lane : 0, a1x = (ax + 1) % 3, a2x = (ax + 2) % 3;
+    // perpendicular width of the frame along the axis
+    double u[3], v[3];
+    for (int d = 0; d < 3; ++d) {
+        u[d] = a1x == 0 ? frame[d] : a1x == 1 ? frame[3 + d] : frame[6 + d];
+        v[d] = a2x == 0 ? frame[d] : a2x == 1 ? frame[3 + d] : frame[6 + d];
+    }
+    const double x0 = u[1] * v[2] - u[2] * v[1], x1 = u[2] * v[0] - u[0] * v[2], x2 = u[0] * v[1] - u[1] * v[0];
+    const double vol = __shfl_sync(0xffffffffu, fabs(frame[0] * x0 + frame[1] * x1 + frame[2] * x2), 0);
+    const double h = vol / sqrt(x0 * x0 + x1 * x1 + x2 * x2);
     const double rcw = rc * (1.0 + 1e-9);   // cells strictly wider than rc
-    double ext[3];
     const int64_t n_at = a1 - a0;
-    for (int a = 0; a < 3; ++a) {
-        g.per[a] = per[a];
-        if (per[a]) {
-            g.lo[a] = 0.0;
-            ext[a] = 1.0;
-        } else {
-            g.lo[a] = n_at > 0 ? lo[a] : 0.0;
-            ext[a] = n_at > 0 ? fmax(hi[a] - lo[a], 0.0) : 0.0;
-        }
-        double nc = floor(ext[a] * h[a] / rcw);
-        g.n[a] = nc < 1.0 ? 1 : (nc > 1024.0 ? 1024 : (int)nc);
-    }
+    const int pa = ax == 0 ? per[0] : ax == 1 ? per[1] : per[2];
+    const double la = ax == 0 ? lo[0] : ax == 1 ? lo[1] : lo[2], ha = ax == 0 ? hi[0] : ax == 1 ? hi[1] : hi[2];
+    const double ext = pa ? 1.0 : (n_at > 0 ? fmax(ha - la, 0.0) : 0.0);
+    const double nc = floor(ext * h / rcw);
+    const int na = nc < 1.0 ? 1 : (nc > 1024.0 ? 1024 : (int)nc);
     // no more cells than max(1, 2 * atoms): wider cells keep the search exact
+    int n[3];
+    for (int a = 0; a < 3; ++a) n[a] = __shfl_sync(0xffffffffu, na, a);
     const int64_t lim = n_at > 0 ? 2 * n_at : 1;
-    while ((int64_t)g.n[0] * g.n[1] * g.n[2] > lim) {
+    while ((int64_t)n[0] * n[1] * n[2] > lim) {
         int a = 0;
-        if (g.n[1] > g.n[a]) a = 1;
-        if (g.n[2] > g.n[a]) a = 2;
-        g.n[a] = (g.n[a] + 1) / 2;
+        if (n[1] > n[a]) a = 1;
+        if (n[2] > n[a]) a = 2;
+        if (a == 0) n[0] = (n[0] + 1) / 2;
+        else if (a == 1) n[1] = (n[1] + 1) / 2;
+        else n[2] = (n[2] + 1) / 2;
     }
-    for (int a = 0; a < 3; ++a) {
-        const double e = ext[a] > 0.0 ? ext[a] : 1.0;
-        g.inv_w[a] = (double)g.n[a] / e;
-        const double cw = h[a] * e / g.n[a];   // perpendicular cell width
-        int K = 1;
-        if (per[a] && cw < rcw) K = (int)ceil(rcw / cw);
-        g.K[a] = K;
+    if (lane < 3) {
+        const int nx = ax == 0 ? n[0] : ax == 1 ? n[1] : n[2];
+        const double e = ext > 0.0 ? ext : 1.0;
+        const double cw = h * e / nx;   // perpendicular cell width
+        g.per[ax] = pa;
+        g.lo[ax] = pa || n_at == 0 ? 0.0 : la;
+        g.n[ax] = nx;
+        g.inv_w[ax] = (double)nx / e;
+        g.K[ax] = pa && cw < rcw ? (int)ceil(rcw / cw) : 1;
     }
-    g.ncells = g.n[0] * g.n[1] * g.n[2];
-    g.cell_base = 0;
-    cfg_cells[c] = g.ncells;
+    if (lane < 9) {
+        double fr = frame[0], fi = finv[0];
+        for (int k = 1; k < 9; ++k)
+            if (lane == k) { fr = frame[k]; fi = finv[k]; }
+        g.cell[lane] = fr;
+        g.cinv[lane] = fi;
+    }
+    const int ncells = n[0] * n[1] * n[2];
+    if (lane == 0) {
+        g.ncells = ncells;
+        g.cell_base = 0;
+    }
+    return ncells;
+}
+
+__global__ void __launch_bounds__(kCfgWarps * 32)
+k_cfg_geom(panna_system sys, double rc, CfgGeom* __restrict__ geom, int64_t* __restrict__ cfg_cells, DevStatus* st)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t c = (int64_t)blockIdx.x * kCfgWarps + (threadIdx.x >> 5);
+    if (c >= sys.n_cfg) return;
+    const int ncells = cfg_geom_warp(sys, rc, c, geom, st, lane);
+    if (lane == 0) cfg_cells[c] = ncells;
 }
 
 __global__ void k_set_cell_base(CfgGeom* __restrict__ geom, const int64_t* __restrict__ base, int64_t C)
@@ -271,17 +290,14 @@ __global__ void k_set_cell_base(CfgGeom* __restrict__ geom, const int64_t* __res
     if (c < C) geom[c].cell_base = base[c];
 }
 
-__global__ void k_bin(panna_system sys, int S, const CfgGeom* __restrict__ geom,
-                      const int32_t* __restrict__ atom_cfg, int32_t* __restrict__ atom_cell,
-                      int64_t* __restrict__ cell_count, float4* __restrict__ pos_hi,
-                      float4* __restrict__ pos_lo, int32_t* __restrict__ wrap, DevStatus* st)
+// Folds atom i into configuration c's cell, writes its hi + lo position and lattice offset; returns
+// its cell within the configuration
+__device__ __forceinline__ int bin_atom(const panna_system& sys, int S, const CfgGeom& g, int64_t i,
+                                        float4* __restrict__ pos_hi, float4* __restrict__ pos_lo,
+                                        int32_t* __restrict__ wrap, DevStatus* st, int& sp)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= sys.n_atoms) return;
-    const int c = atom_cfg[i];
-    const CfgGeom& g = geom[c];
     double x[3] = {sys.pos[3 * i], sys.pos[3 * i + 1], sys.pos[3 * i + 2]};
-    int sp = sys.species[i];
+    sp = sys.species[i];
     if (sp < 0 || sp >= S) { set_status(st, PANNA_ERR_BAD_INPUT, (int)i); sp = 0; }
     if (!(isfinite(x[0]) && isfinite(x[1]) && isfinite(x[2]))) {
         set_status(st, PANNA_ERR_BAD_INPUT, (int)i);
@@ -303,7 +319,19 @@ __global__ void k_bin(panna_system sys, int S, const CfgGeom* __restrict__ geom,
     pos_hi[i] = make_float4(h0, h1, h2, __int_as_float(sp));
     pos_lo[i] = make_float4((float)(xw[0] - h0), (float)(xw[1] - h1), (float)(xw[2] - h2), 0.f);
     wrap[3 * i] = m[0]; wrap[3 * i + 1] = m[1]; wrap[3 * i + 2] = m[2];
-    int local = (ci[0] * g.n[1] + ci[1]) * g.n[2] + ci[2];
+    return (ci[0] * g.n[1] + ci[1]) * g.n[2] + ci[2];
+}
+
+__global__ void k_bin(panna_system sys, int S, const CfgGeom* __restrict__ geom,
+                      const int32_t* __restrict__ atom_cfg, int32_t* __restrict__ atom_cell,
+                      int64_t* __restrict__ cell_count, float4* __restrict__ pos_hi,
+                      float4* __restrict__ pos_lo, int32_t* __restrict__ wrap, DevStatus* st)
+{
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= sys.n_atoms) return;
+    const CfgGeom& g = geom[atom_cfg[i]];
+    int sp;
+    const int local = bin_atom(sys, S, g, i, pos_hi, pos_lo, wrap, st, sp);
     atom_cell[i] = local;
     atomicAdd((unsigned long long*)&cell_count[g.cell_base + local], 1ull);
 }
@@ -400,6 +428,164 @@ k_sort_cells(int64_t C, const CfgGeom* __restrict__ geom, int64_t ncells, const 
     for (int64_t c = (int64_t)blockIdx.x * kSortWarps + (threadIdx.x >> 5); c < used; c += stride) {
         const int64_t b = cell_start[c], e = cell_start[c + 1];
         if (e > b) sort_cell(b, e, lane, cell_atoms, pos_hi, pos_lo, pos_hi_s, pos_lo_s);
+    }
+}
+
+// ------------------------------------------------------------------ small batches: one CTA
+
+// Everything before the search proper for a small batch, in one CTA: configuration geometry, binning,
+// cell offsets, the cells' atoms in index order with their positions, and the network rows by species
+// (k_atom_cfg .. k_sort_cells and k_species_*, sixteen launches otherwise, whose launches and not their
+// work take the time: 64 atoms 62 -> 15 us, 850 atoms in 50 molecules 75 -> 26 us).  Counters and the
+// cells' atoms live in shared memory.
+constexpr int kSmallThreads = 1024;
+constexpr int64_t kSmallAtoms = 4096, kSmallCfgs = 1024;
+
+__host__ __device__ inline size_t cells_small_smem(int64_t N, int64_t C)
+{
+    return sizeof(int32_t) * (size_t)(2 * (2 * N + C + 1) + N + C);
+}
+
+// exclusive scan of v over the CTA; total in *sum (shared)
+__device__ __forceinline__ int cta_scan(int v, int* wsum, int& sum)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) wsum[wid] = inc;
+    __syncthreads();
+    int w = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += t;
+    }
+    sum = __shfl_sync(0xffffffffu, w, 31);
+    const int before = __shfl_sync(0xffffffffu, w, wid > 0 ? wid - 1 : 0);
+    __syncthreads();   // wsum is free again
+    return (wid > 0 ? before : 0) + inc - v;
+}
+
+__global__ void __launch_bounds__(kSmallThreads)
+k_cells_small(panna_system sys, Work w, int S, double rc)
+{
+    extern __shared__ int sm_cells[];
+    __shared__ int wsum[32];
+    __shared__ int s_cnt[kMaxSpecies][kSmallAtoms / 32];   // atoms of a species per group of 32
+    __shared__ int s_tot[kMaxSpecies];
+    const int N = (int)sys.n_atoms, C = (int)sys.n_cfg, M = 2 * N + C + 1;
+    int* start = sm_cells;          // [M] counts, then first slots
+    int* fill = start + M;          // [M]
+    int* atoms = fill + M;          // [N] atoms in cell order, unsorted
+    int* cells = atoms + N;         // [C] cells per configuration, then the first one
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int c = warp; c < C; c += kSmallThreads / 32) {
+        const int n = cfg_geom_warp(sys, rc, c, w.geom, w.status, lane);
+        if (lane == 0) cells[c] = n;
+        for (int64_t i = sys.atom_off[c] + lane; i < sys.atom_off[c + 1]; i += 32) w.atom_cfg[i] = c;
+    }
+    for (int k = tid; k < M; k += kSmallThreads) start[k] = 0;
+    __syncthreads();
+    int used;
+    {
+        const int v = tid < C ? cells[tid] : 0;   // C <= kSmallCfgs = kSmallThreads
+        const int ex = cta_scan(v, wsum, used);
+        if (tid < C) {
+            cells[tid] = ex;
+            w.geom[tid].cell_base = ex;
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < N; i += kSmallThreads) {
+        const int c = w.atom_cfg[i];
+        int sp;
+        const int local = bin_atom(sys, S, w.geom[c], i, w.pos_hi, w.pos_lo, w.wrap, w.status, sp);
+        w.atom_cell[i] = local;
+        atomicAdd(&start[cells[c] + local], 1);
+    }
+    __syncthreads();
+    for (int k0 = 0, carry = 0; k0 < used; k0 += kSmallThreads) {
+        const int k = k0 + tid;
+        int tot;
+        const int ex = carry + cta_scan(k < used ? start[k] : 0, wsum, tot);
+        if (k < used) {
+            start[k] = fill[k] = ex;
+            w.cell_start[k] = ex;
+        }
+        carry += tot;
+    }
+    if (tid == 0) {
+        start[used] = N;
+        w.cell_start[used] = N;
+    }
+    __syncthreads();
+    for (int i = tid; i < N; i += kSmallThreads)
+        atoms[atomicAdd(&fill[cells[w.atom_cfg[i]] + w.atom_cell[i]], 1)] = i;
+    __syncthreads();
+    // each atom to the slot given by the number of its cell's atoms with a smaller index
+    for (int i = tid; i < N; i += kSmallThreads) {
+        const int gc = cells[w.atom_cfg[i]] + w.atom_cell[i], b = start[gc], e = start[gc + 1];
+        int slot = b;
+        for (int k = b; k < e; ++k) slot += atoms[k] < i ? 1 : 0;
+        w.cell_atoms[slot] = i;
+        w.pos_hi_s[slot] = w.pos_hi[i];
+        w.pos_lo_s[slot] = w.pos_lo[i];
+    }
+    // network rows: the non-ghost atoms by species, in index order
+    const uint8_t* ghost = sys.ghost;
+    auto species_of = [&](int i) {
+        return i < N && !(ghost && ghost[i]) ? __float_as_int(w.pos_hi[i].w) : -1;
+    };
+    const int groups = (N + 31) / 32;
+    for (int q = warp; q < groups; q += kSmallThreads / 32) {
+        const int sp = species_of(32 * q + lane);
+        for (int s = 0; s < S; ++s) {
+            const unsigned m = __ballot_sync(0xffffffffu, sp == s);
+            if (lane == 0) s_cnt[s][q] = __popc(m);
+        }
+    }
+    __syncthreads();
+    if (warp < S) {
+        int run = 0;
+        for (int q0 = 0; q0 < groups; q0 += 32) {
+            const int v = q0 + lane < groups ? s_cnt[warp][q0 + lane] : 0;
+            int inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += t;
+            }
+            if (q0 + lane < groups) s_cnt[warp][q0 + lane] = run + inc - v;
+            run += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        if (lane == 0) s_tot[warp] = run;
+    }
+    __syncthreads();
+    int first[kMaxSpecies + 1];
+    first[0] = 0;
+    for (int s = 0; s < S; ++s) first[s + 1] = first[s] + s_tot[s];
+    if (tid == 0) {
+        for (int s = 0, t = 0; s <= S; ++s) {
+            w.seg_off[s] = first[s];
+            w.tile_start[s] = t;
+            if (s < S) t += (s_tot[s] + kGM - 1) / kGM;
+        }
+    }
+    for (int q = warp; q < groups; q += kSmallThreads / 32) {
+        const int i = 32 * q + lane, sp = species_of(i);
+        int row = -1;
+        for (int s = 0; s < S; ++s) {
+            const unsigned m = __ballot_sync(0xffffffffu, sp == s);
+            if (sp == s) row = first[s] + s_cnt[s][q] + __popc(m & ((1u << lane) - 1u));
+        }
+        if (i < N) {
+            w.row_of_atom[i] = row;
+            if (row >= 0) w.atom_of_row[row] = i;
+        }
     }
 }
 
@@ -668,24 +854,6 @@ k_neighbors(int64_t N, int S, double rc_d, float rc, const CfgGeom* __restrict__
 
 // ------------------------------------------------------------------ Verlet-list refresh
 
-// Positions folded with the lattice offsets recorded when the list was built (wrap), so the
-// image shifts stored with the candidates stay valid while atoms move; species in .w kept.
-__global__ void k_fold_frozen(int64_t N, const double* __restrict__ pos, const int32_t* __restrict__ atom_cfg,
-                              const CfgGeom* __restrict__ geom, const int32_t* __restrict__ wrap,
-                              float4* __restrict__ pos_hi, float4* __restrict__ pos_lo)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const CfgGeom& g = geom[atom_cfg[i]];
-    const int m0 = wrap[3 * i], m1 = wrap[3 * i + 1], m2 = wrap[3 * i + 2];
-    double xw[3];
-    for (int d = 0; d < 3; ++d) xw[d] = pos[3 * i + d] + m0 * g.cell[d] + m1 * g.cell[3 + d] + m2 * g.cell[6 + d];
-    const float h0 = (float)xw[0], h1 = (float)xw[1], h2 = (float)xw[2];
-    const float w = pos_hi[i].w;
-    pos_hi[i] = make_float4(h0, h1, h2, w);
-    pos_lo[i] = make_float4((float)(xw[0] - h0), (float)(xw[1] - h1), (float)(xw[2] - h2), 0.f);
-}
-
 // The candidates (j, image) found within rc + skin when the list was built are re-tested
 // at the current positions with the arithmetic of the full search (FP32 band filter,
 // double-float relative vector, FP64 re-test near rc); those with r < rc are kept in their
@@ -759,12 +927,10 @@ cudaError_t refresh_neighbors(const Work& cand, Work& w, const DescDev& d, cudaS
 {
     const int64_t N = w.N;
     if (N == 0) return cudaSuccess;
-    k_fold_frozen<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, w.sys->pos, w.atom_cfg, w.geom, w.wrap, w.pos_hi,
-                                                              w.pos_lo);
     k_refresh<<<(unsigned)((N + kNbWarps - 1) / kNbWarps), kNbWarps * 32, 0, s>>>(
         N, d.rc_d, d.rc, w.geom, w.atom_cfg, cand.nb_count, cand.nb_idx, cand.cap, w.pos_hi, w.pos_lo, w.cap,
         w.nb_count, w.nb_vec, w.nb_idx, w.nb_vlo, w.status);
-    *launches += 2;
+    ++*launches;
     return cudaGetLastError();
 }
 
@@ -817,34 +983,44 @@ cudaError_t build_neighbors(Work& w, const DescDev& d, cudaStream_t s, int* laun
     const int64_t N = w.N, C = w.C;
     const panna_system& sys = *w.sys;
     cudaError_t e;
-    unsigned nbA = (unsigned)((N + 255) / 256);
-    if (nbA == 0) nbA = 1;
-    k_atom_cfg<<<nbA, 256, 0, s>>>(sys.atom_off, C, N, w.atom_cfg);
-    k_cfg_geom<<<(unsigned)((C + kCfgWarps - 1) / kCfgWarps), kCfgWarps * 32, 0, s>>>(sys, d.rc_d, w.geom,
-                                                                                      w.cell_count, w.status);
-    *launches += 2;
-    // cell bases: scan of per-config cell counts (stored temporarily in cell_count[0..C))
-    e = exclusive_scan_i64(w.cell_count, w.cell_start, C, w.scan_tmp, s, launches);
-    if (e != cudaSuccess) return e;
-    k_set_cell_base<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(w.geom, w.cell_start, C);
-    ++*launches;
-    // total cells <= 2N + C by construction; clear the counters
-    e = cudaMemsetAsync(w.cell_count, 0, sizeof(int64_t) * (w.cap_cells + 1), s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(w.cell_fill, 0, sizeof(int32_t) * w.cap_cells, s);
-    if (e != cudaSuccess) return e;
-    k_bin<<<nbA, 256, 0, s>>>(sys, d.S, w.geom, w.atom_cfg, w.atom_cell, w.cell_count, w.pos_hi, w.pos_lo,
-                              w.wrap, w.status);
-    ++*launches;
-    e = exclusive_scan_i64(w.cell_count, w.cell_start, w.cap_cells, w.scan_tmp, s, launches);
-    if (e != cudaSuccess) return e;
-    k_scatter<<<nbA, 256, 0, s>>>(N, w.atom_cfg, w.atom_cell, w.geom, w.cell_start, w.cell_fill, w.cell_atoms);
-    {
-        const int64_t warps = std::min<int64_t>(w.cap_cells, kSortMaxWarps);
-        k_sort_cells<<<(unsigned)((warps + kSortWarps - 1) / kSortWarps), kSortWarps * 32, 0, s>>>(
-            C, w.geom, w.cap_cells, w.cell_start, w.cell_atoms, w.pos_hi, w.pos_lo, w.pos_hi_s, w.pos_lo_s);
+    w.rows_ready = false;
+    if (N > 0 && N <= kSmallAtoms && C <= kSmallCfgs && w.row_of_atom) {
+        const size_t smem_c = cells_small_smem(N, C);
+        e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
+        if (e != cudaSuccess) return e;
+        k_cells_small<<<1, kSmallThreads, smem_c, s>>>(sys, w, d.S, d.rc_d);
+        ++*launches;
+        w.rows_ready = true;
+    } else {
+        unsigned nbA = (unsigned)((N + 255) / 256);
+        if (nbA == 0) nbA = 1;
+        k_atom_cfg<<<nbA, 256, 0, s>>>(sys.atom_off, C, N, w.atom_cfg);
+        k_cfg_geom<<<(unsigned)((C + kCfgWarps - 1) / kCfgWarps), kCfgWarps * 32, 0, s>>>(sys, d.rc_d, w.geom,
+                                                                                          w.cell_count, w.status);
+        *launches += 2;
+        // cell bases: scan of per-config cell counts (stored temporarily in cell_count[0..C))
+        e = exclusive_scan_i64(w.cell_count, w.cell_start, C, w.scan_tmp, s, launches);
+        if (e != cudaSuccess) return e;
+        k_set_cell_base<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(w.geom, w.cell_start, C);
+        ++*launches;
+        // total cells <= 2N + C by construction; clear the counters
+        e = cudaMemsetAsync(w.cell_count, 0, sizeof(int64_t) * (w.cap_cells + 1), s);
+        if (e != cudaSuccess) return e;
+        e = cudaMemsetAsync(w.cell_fill, 0, sizeof(int32_t) * w.cap_cells, s);
+        if (e != cudaSuccess) return e;
+        k_bin<<<nbA, 256, 0, s>>>(sys, d.S, w.geom, w.atom_cfg, w.atom_cell, w.cell_count, w.pos_hi, w.pos_lo,
+                                  w.wrap, w.status);
+        ++*launches;
+        e = exclusive_scan_i64(w.cell_count, w.cell_start, w.cap_cells, w.scan_tmp, s, launches);
+        if (e != cudaSuccess) return e;
+        k_scatter<<<nbA, 256, 0, s>>>(N, w.atom_cfg, w.atom_cell, w.geom, w.cell_start, w.cell_fill, w.cell_atoms);
+        {
+            const int64_t warps = std::min<int64_t>(w.cap_cells, kSortMaxWarps);
+            k_sort_cells<<<(unsigned)((warps + kSortWarps - 1) / kSortWarps), kSortWarps * 32, 0, s>>>(
+                C, w.geom, w.cap_cells, w.cell_start, w.cell_atoms, w.pos_hi, w.pos_lo, w.pos_hi_s, w.pos_lo_s);
+        }
+        *launches += 2;
     }
-    *launches += 2;
     size_t smem = (size_t)kNbWarps * w.cap * (sizeof(float4) + sizeof(int2) + (w.nb_vlo ? sizeof(float4) : 0));
     e = cudaFuncSetAttribute(k_neighbors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -879,9 +1055,11 @@ constexpr int kOffThreads = 1024;
 
 // Offsets of every (block, species) count: per species an exclusive scan over the blocks (one
 // CTA; each thread walks a contiguous run of blocks, a block-wide scan joins the runs), shifted
-// by the totals of the species before it; seg_off[s] = first row of species s.
+// by the totals of the species before it; seg_off[s] = first row of species s,
+// tile_start[s] = its first tile of kGM rows.
 __global__ void __launch_bounds__(kOffThreads)
-k_species_offsets(int64_t nblk, int S, int32_t* __restrict__ blk_counts, int32_t* __restrict__ seg_off)
+k_species_offsets(int64_t nblk, int S, int32_t* __restrict__ blk_counts, int32_t* __restrict__ seg_off,
+                  int32_t* __restrict__ tile_start)
 {
     __shared__ int wsum[kOffThreads / 32];
     __shared__ int s_base;
@@ -925,7 +1103,14 @@ k_species_offsets(int64_t nblk, int S, int32_t* __restrict__ blk_counts, int32_t
         }
         __syncthreads();
     }
-    if (t == 0) seg_off[S] = s_base;
+    if (t == 0) {
+        seg_off[S] = s_base;
+        // the networks' row tiles of every species
+        for (int s = 0, k = 0; s <= S; ++s) {
+            tile_start[s] = k;
+            if (s < S) k += (seg_off[s + 1] - seg_off[s] + kGM - 1) / kGM;
+        }
+    }
 }
 
 __global__ void k_species_rank(int64_t N, int S, const float4* __restrict__ pos_hi, const uint8_t* __restrict__ ghost,
@@ -955,14 +1140,16 @@ __global__ void k_species_rank(int64_t N, int S, const float4* __restrict__ pos_
 
 cudaError_t species_order(Work& w, int S, cudaStream_t s, int* launches)
 {
+    if (w.rows_ready) return cudaSuccess;
     int64_t nblk = (w.N + kSpBlock - 1) / kSpBlock;
     if (nblk == 0) nblk = 1;
     const uint8_t* ghost = w.sys->ghost;
     k_species_count<<<(unsigned)nblk, kSpBlock, 0, s>>>(w.N, S, w.pos_hi, ghost, w.blk_counts);
-    k_species_offsets<<<1, kOffThreads, 0, s>>>(nblk, S, w.blk_counts, w.seg_off);
+    k_species_offsets<<<1, kOffThreads, 0, s>>>(nblk, S, w.blk_counts, w.seg_off, w.tile_start);
     k_species_rank<<<(unsigned)nblk, kSpBlock, 0, s>>>(w.N, S, w.pos_hi, ghost, w.blk_counts, w.row_of_atom,
                                                       w.atom_of_row);
     *launches += 3;
+    w.rows_ready = true;
     return cudaGetLastError();
 }
 

@@ -72,6 +72,8 @@ size_t carve_static(char* base, int64_t N, int64_t C, int cap, Work& w)
     w.row_of_atom = nullptr;
     w.atom_of_row = nullptr;
     w.seg_off = nullptr;
+    w.tile_start = nullptr;
+    w.rows_ready = false;
     w.blk_counts = nullptr;
     return a.off;
 }
