@@ -162,9 +162,10 @@ __device__ __forceinline__ double warp_max_d(double v)
 }
 
 // Geometry of configuration c by one warp: frame and inverse, grid of cells, image shifts; returns the
-// number of cells.  Axes (and cofactors) go to lanes of their own: FP64 divisions and square roots take
-// hundreds of cycles each on this GPU, and one lane doing all of them was 11 us.
-__device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc, int64_t c, CfgGeom* __restrict__ geom,
+// number of cells.  FP64 runs at 1/64 of the FP32 rate (a warp's instruction holds the SM's pipe for 16
+// cycles, a division or square root takes hundreds), so the axes go to lanes of their own, and without
+// a periodic direction (the frame is the identity) no product with the frame is formed: the same values.
+__device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc, int64_t c, CfgGeom& g,
                                              DevStatus* st, int lane)
 {
     const int64_t a0 = sys.atom_off[c], a1 = sys.atom_off[c + 1];
@@ -201,20 +202,19 @@ __device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc,
         for (int64_t i = a0 + lane; i < a1; i += 32) {
             const double* x = sys.pos + 3 * i;
             for (int a = 0; a < 3; ++a) {
-                double sa = x[0] * finv[a] + x[1] * finv[3 + a] + x[2] * finv[6 + a];
+                const double sa = any ? x[0] * finv[a] + x[1] * finv[3 + a] + x[2] * finv[6 + a] : x[a];
                 lo[a] = fmin(lo[a], sa);
                 hi[a] = fmax(hi[a], sa);
             }
         }
         for (int a = 0; a < 3; ++a) { lo[a] = warp_min_d(lo[a]); hi[a] = warp_max_d(hi[a]); }
     }
-    CfgGeom& g = geom[c];
     // image shift table for t in [-1,1]^3, one entry per lane
     if (lane < 27) {
         const int t0 = lane / 9 - 1, t1 = (lane / 3) % 3 - 1, t2 = lane % 3 - 1;
         for (int d = 0; d < 3; ++d) {
-            double S = t0 * frame[d] + t1 * frame[3 + d] + t2 * frame[6 + d];
-            float sh = (float)S;
+            const double S = any ? t0 * frame[d] + t1 * frame[3 + d] + t2 * frame[6 + d] : 0.0;   // unused then
+            const float sh = (float)S;
             g.sh_hi[lane][d] = sh;
             g.sh_lo[lane][d] = (float)(S - (double)sh);
         }
@@ -222,14 +222,17 @@ __device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc,
     // lane a (0..2): axis a
     const int ax = lane < 3 ? lane : 0, a1x = (ax + 1) % 3, a2x = (ax + 2) % 3;
     // perpendicular width of the frame along the axis
-    double u[3], v[3];
-    for (int d = 0; d < 3; ++d) {
-        u[d] = a1x == 0 ? frame[d] : a1x == 1 ? frame[3 + d] : frame[6 + d];
-        v[d] = a2x == 0 ? frame[d] : a2x == 1 ? frame[3 + d] : frame[6 + d];
+    double h = 1.0;
+    if (any) {
+        double u[3], v[3];
+        for (int d = 0; d < 3; ++d) {
+            u[d] = a1x == 0 ? frame[d] : a1x == 1 ? frame[3 + d] : frame[6 + d];
+            v[d] = a2x == 0 ? frame[d] : a2x == 1 ? frame[3 + d] : frame[6 + d];
+        }
+        const double x0 = u[1] * v[2] - u[2] * v[1], x1 = u[2] * v[0] - u[0] * v[2], x2 = u[0] * v[1] - u[1] * v[0];
+        const double vol = __shfl_sync(0xffffffffu, fabs(frame[0] * x0 + frame[1] * x1 + frame[2] * x2), 0);
+        h = vol / sqrt(x0 * x0 + x1 * x1 + x2 * x2);
     }
-    const double x0 = u[1] * v[2] - u[2] * v[1], x1 = u[2] * v[0] - u[0] * v[2], x2 = u[0] * v[1] - u[1] * v[0];
-    const double vol = __shfl_sync(0xffffffffu, fabs(frame[0] * x0 + frame[1] * x1 + frame[2] * x2), 0);
-    const double h = vol / sqrt(x0 * x0 + x1 * x1 + x2 * x2);
     const double rcw = rc * (1.0 + 1e-9);   // cells strictly wider than rc
     const int64_t n_at = a1 - a0;
     const int pa = ax == 0 ? per[0] : ax == 1 ? per[1] : per[2];
@@ -280,7 +283,7 @@ k_cfg_geom(panna_system sys, double rc, CfgGeom* __restrict__ geom, int64_t* __r
     const int lane = threadIdx.x & 31;
     const int64_t c = (int64_t)blockIdx.x * kCfgWarps + (threadIdx.x >> 5);
     if (c >= sys.n_cfg) return;
-    const int ncells = cfg_geom_warp(sys, rc, c, geom, st, lane);
+    const int ncells = cfg_geom_warp(sys, rc, c, geom[c], st, lane);
     if (lane == 0) cfg_cells[c] = ncells;
 }
 
@@ -433,11 +436,12 @@ k_sort_cells(int64_t C, const CfgGeom* __restrict__ geom, int64_t ncells, const 
 
 // ------------------------------------------------------------------ small batches: one CTA
 
-// Everything before the search proper for a small batch, in one CTA: configuration geometry, binning,
-// cell offsets, the cells' atoms in index order with their positions, and the network rows by species
-// (k_atom_cfg .. k_sort_cells and k_species_*, sixteen launches otherwise, whose launches and not their
-// work take the time: 64 atoms 62 -> 15 us, 850 atoms in 50 molecules 75 -> 26 us).  Counters and the
-// cells' atoms live in shared memory.
+// A small batch is prepared by two launches instead of sixteen, whose launches and not their work took
+// the time: k_cfg_bin the configurations' geometry and binning (FP64, hence spread over the SMs: CTA (c,
+// y) takes every gridDim.y-th group of kBinThreads atoms of configuration c, repeating its geometry),
+// k_cells_small the integer part in one CTA: cell offsets, the cells' atoms in index order with their
+// positions, and the network rows by species.  Counters and the cells' atoms live in shared memory.
+// Sum of the launches: 64 atoms 62 -> 19 us, 850 atoms in 50 molecules 75 -> 21 us.
 constexpr int kSmallThreads = 1024;
 constexpr int64_t kSmallAtoms = 4096, kSmallCfgs = 1024;
 
@@ -470,8 +474,33 @@ __device__ __forceinline__ int cta_scan(int v, int* wsum, int& sum)
     return (wid > 0 ? before : 0) + inc - v;
 }
 
+constexpr int kBinThreads = 128;
+
+__global__ void __launch_bounds__(kBinThreads)
+k_cfg_bin(panna_system sys, Work w, int S, double rc)
+{
+    __shared__ CfgGeom g;
+    const int c = blockIdx.x, tid = threadIdx.x;
+    if (tid < 32) {
+        cfg_geom_warp(sys, rc, c, g, w.status, tid);
+        __syncwarp();
+        if (blockIdx.y == 0) {
+            const int* src = reinterpret_cast<const int*>(&g);
+            int* dst = reinterpret_cast<int*>(w.geom + c);
+            for (int k = tid; k < (int)(sizeof(CfgGeom) / 4); k += 32) dst[k] = src[k];
+        }
+    }
+    __syncthreads();
+    const int64_t a1 = sys.atom_off[c + 1];
+    for (int64_t i = sys.atom_off[c] + blockIdx.y * kBinThreads + tid; i < a1; i += gridDim.y * kBinThreads) {
+        int sp;
+        w.atom_cfg[i] = c;
+        w.atom_cell[i] = bin_atom(sys, S, g, i, w.pos_hi, w.pos_lo, w.wrap, w.status, sp);
+    }
+}
+
 __global__ void __launch_bounds__(kSmallThreads)
-k_cells_small(panna_system sys, Work w, int S, double rc)
+k_cells_small(panna_system sys, Work w, int S)
 {
     extern __shared__ int sm_cells[];
     __shared__ int wsum[32];
@@ -483,16 +512,10 @@ k_cells_small(panna_system sys, Work w, int S, double rc)
     int* atoms = fill + M;          // [N] atoms in cell order, unsorted
     int* cells = atoms + N;         // [C] cells per configuration, then the first one
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int c = warp; c < C; c += kSmallThreads / 32) {
-        const int n = cfg_geom_warp(sys, rc, c, w.geom, w.status, lane);
-        if (lane == 0) cells[c] = n;
-        for (int64_t i = sys.atom_off[c] + lane; i < sys.atom_off[c + 1]; i += 32) w.atom_cfg[i] = c;
-    }
     for (int k = tid; k < M; k += kSmallThreads) start[k] = 0;
-    __syncthreads();
     int used;
     {
-        const int v = tid < C ? cells[tid] : 0;   // C <= kSmallCfgs = kSmallThreads
+        const int v = tid < C ? w.geom[tid].ncells : 0;   // C <= kSmallCfgs = kSmallThreads
         const int ex = cta_scan(v, wsum, used);
         if (tid < C) {
             cells[tid] = ex;
@@ -500,13 +523,7 @@ k_cells_small(panna_system sys, Work w, int S, double rc)
         }
     }
     __syncthreads();
-    for (int i = tid; i < N; i += kSmallThreads) {
-        const int c = w.atom_cfg[i];
-        int sp;
-        const int local = bin_atom(sys, S, w.geom[c], i, w.pos_hi, w.pos_lo, w.wrap, w.status, sp);
-        w.atom_cell[i] = local;
-        atomicAdd(&start[cells[c] + local], 1);
-    }
+    for (int i = tid; i < N; i += kSmallThreads) atomicAdd(&start[cells[w.atom_cfg[i]] + w.atom_cell[i]], 1);
     __syncthreads();
     for (int k0 = 0, carry = 0; k0 < used; k0 += kSmallThreads) {
         const int k = k0 + tid;
@@ -988,8 +1005,10 @@ cudaError_t build_neighbors(Work& w, const DescDev& d, cudaStream_t s, int* laun
         const size_t smem_c = cells_small_smem(N, C);
         e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
         if (e != cudaSuccess) return e;
-        k_cells_small<<<1, kSmallThreads, smem_c, s>>>(sys, w, d.S, d.rc_d);
-        ++*launches;
+        const unsigned per_cfg = (unsigned)((N + C * kBinThreads - 1) / (C * kBinThreads));
+        k_cfg_bin<<<dim3((unsigned)C, per_cfg), kBinThreads, 0, s>>>(sys, w, d.S, d.rc_d);
+        k_cells_small<<<1, kSmallThreads, smem_c, s>>>(sys, w, d.S);
+        *launches += 2;
         w.rows_ready = true;
     } else {
         unsigned nbA = (unsigned)((N + 255) / 256);
