@@ -230,9 +230,10 @@ panna_status panna_set_angular_precision(panna_ctx* ctx, int32_t mode);
  * (k, k + d mod n), whose rounds of min(32, n - 1) pairs touch distinct entries on each side,
  * so the per-entry gradients are summed without atomics in a fixed order (bit-reproducible).
  * Matrix forms: descriptor 5 (any descriptor of the modified term) and adjoint 6 (at most 16 sectors
- * and 8 shells): one warp per atom, the products over sectors and shells on the tensor cores from
- * operands split into TF32 parts; sums in a fixed order.  Where they apply, batches of at least 1216
- * atoms take them without measuring.  With FP32 networks (extended angular terms) the descriptor's
+ * and 8 shells): one warp per atom (below 1216 atoms with FP32 networks: 2 to 64 warps of a cluster),
+ * the products over sectors and shells on the tensor cores from operands split into TF32 parts; sums in
+ * a fixed order.  Where they apply, batches of at least 1216 atoms and all batches with FP32 networks
+ * take them without measuring.  With FP32 networks (extended angular terms) the descriptor's
  * candidates are variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that
  * the matrix forms do not take use variant 2 (adjoint: 5; the descriptor with FP32 networks: 0) and
  * smaller ones variant 0 (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks): a bit mask of the first layer's

@@ -45,6 +45,7 @@
 // zeta t^(d+1)/(d+1) (1-t)^zeta <= 1.5e-9 (d = 8, zeta >= 32), 1.1e-9 (d = 13, zeta >= 16) of its
 // maximum; all terms have one sign, so for t near 1 the sum still underflows as y^zeta does.  Below
 // zeta = 16 the power comes from the float pair 1 - t.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -57,7 +58,38 @@ namespace panna {
 
 namespace {
 
-constexpr int kMW = 4;   // warps per CTA
+constexpr int kMW = 4;        // warps per CTA, an atom each
+constexpr int kTeamMax = 8;   // warps of a CTA that share one atom (TEAM), and
+constexpr int kTeamCtas = 8;  // CTAs (a cluster), at most
+
+namespace cg = cooperative_groups;
+
+// TEAM: the part of a warp in the rounds of 32 pairs of one species block.  All blocks' rounds, in order,
+// are dealt to the warps in consecutive runs [lo, hi); rb counts the rounds before the block.
+struct TeamRounds {
+    int R = 0, lo, hi, rb = 0;
+    __device__ __forceinline__ TeamRounds(const DescDev& d, const int* seg, int warp, int warps)
+    {
+        for (int a = 0; a < d.S; ++a)
+            for (int b = a; b < d.S; ++b) R += rounds(block_pairs(seg, a, b));
+        lo = R * warp / warps;
+        hi = R * (warp + 1) / warps;
+    }
+    static __device__ __forceinline__ int block_pairs(const int* seg, int a, int b)
+    {
+        const int na = seg[a + 1] - seg[a];
+        return a == b ? na * (na - 1) / 2 : na * (seg[b + 1] - seg[b]);
+    }
+    static __device__ __forceinline__ int rounds(int pairs) { return (pairs + 31) / 32; }
+    // the warp's rounds [first, last) of the next block
+    __device__ __forceinline__ void next(int pairs, int& first, int& last)
+    {
+        const int nr = rounds(pairs);
+        first = max(lo - rb, 0);
+        last = min(hi - rb, nr);
+        rb += nr;
+    }
+};
 
 // D += A B, m16n8k8, TF32 operands (the leading 19 bits of each register), FP32 accumulators
 __device__ __forceinline__ void mma8(float (&c)[4], float a0, float a1, float a2, float a3, float b0, float b1)
@@ -178,23 +210,47 @@ __device__ __forceinline__ void half_pair(float c, float cl, float& h, float& l)
 // the bracket by an FMA-compensated difference of products, delta_m the same error of the sector's
 // constants.  Distances enter as the exact sum r1 + r2 = 2 (hi + lo).
 
-// shared bytes per warp: unit vectors and distances (PAIR: and their low parts), r, f_c, the pairs
+// TEAM (small batches): all warps of a cluster of CTAs share one atom and its rounds (TeamRounds), those of
+// a CTA its staging area.  The runs are consecutive, so a warp writes the blocks that are wholly its own;
+// of a block shared with the warps after it the first warp adds up the others' sums, in order, those of
+// the cluster's other CTAs CTA by CTA through distributed shared memory.
+
+// shared bytes of an atom: unit vectors and distances (PAIR: and their low parts), r, f_c
 template <bool FAST>
-__host__ __device__ inline size_t desc_mma_warp_bytes(int cap)
+__host__ __device__ inline size_t desc_mma_atom_bytes(int cap)
 {
-    return FAST ? (size_t)((cap + 1) & ~1) * (16 + 4 + 4) + 16 * (16 + 16) : (size_t)cap * (16 + 16) + 16 * (16 + 16 + 16);
+    return FAST ? (size_t)((cap + 1) & ~1) * (16 + 4 + 4) : (size_t)cap * (16 + 16);
+}
+// and of a warp: the round's pairs (TEAM: and its part of a shared block)
+template <bool FAST>
+__host__ __device__ inline size_t desc_mma_warp_bytes(int part)
+{
+    return 16 * (FAST ? 16 + 16 : 16 + 16 + 16) + part * 512;
 }
 
-template <bool FAST, int CM, int PW>
-__global__ void __launch_bounds__(kMW * 32, FAST ? (CM == 1 ? 8 : 7) : (CM == 1 ? 6 : 5))
+template <bool FAST, int CM, int PW, bool TEAM>
+__global__ void __launch_bounds__((TEAM ? kTeamMax : kMW) * 32,
+                                  TEAM ? 2 : FAST ? (CM == 1 ? 8 : 7) : (CM == 1 ? 6 : 5))
 k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __restrict__ out,
            __nv_bfloat16* __restrict__ Gh, __nv_bfloat16* __restrict__ Gl)
 {
     extern __shared__ float4 sm4[];
-    __shared__ int s_seg[kMW][kMaxSpecies + 1];
+    __shared__ int s_seg[TEAM ? kTeamMax : kMW][kMaxSpecies + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int cap = w.cap, cap2 = (cap + 1) & ~1;
-    char* base = reinterpret_cast<char*>(sm4) + (size_t)warp * desc_mma_warp_bytes<FAST>(cap);
+    const int warps = TEAM ? blockDim.x >> 5 : 1, tid = TEAM ? threadIdx.x : lane, threads = 32 * warps;
+    const size_t a_bytes = desc_mma_atom_bytes<FAST>(cap), w_bytes = desc_mma_warp_bytes<FAST>(TEAM ? CM : 0);
+    char* base = reinterpret_cast<char*>(sm4) + (TEAM ? 0 : warp * (a_bytes + w_bytes));
+    const int ctas = TEAM ? cg::this_cluster().num_blocks() : 1, rank = TEAM ? cg::this_cluster().block_rank() : 0;
+    const int wt = rank * warps + warp, team = ctas * warps;   // the warp's number among those of its atom
+    auto sync = [] {
+        if (TEAM) __syncthreads();
+        else __syncwarp();
+    };
+    auto cluster_sync = [&] {
+        if (ctas > 1) cg::this_cluster().sync();
+        else __syncthreads();
+    };
     // FAST: (unit vector, rho = (r - R_c) sqrt(eta_l) / 2), r, f_c; PAIR: (unit vector, r), (its low
     // part, f_c).  rho: distances relative to the middle shell R_c in units of the Gaussians' width, so
     // that exp(-eta (r_bar - R)^2) = 2^(-x^2) with x = rho_1 + rho_2 - (R - R_c) sqrt(eta_l); rounding
@@ -207,9 +263,10 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
     // geometry of the round's pairs, each for pairs t and t + 4 of a group.  pa: sin, cos of th'/2;
     // pr: FAST x + nR, f_c f_c; PAIR: the halves of r_bar; pd: PAIR delta, f_c f_c.  Groups 2 and 3
     // swap the two halves of each float4, so that the 32 lanes' stores fall on 32 banks
-    float4* pa = FAST ? reinterpret_cast<float4*>(sf + cap2) : sl + cap;
+    float4* pa = reinterpret_cast<float4*>(base + a_bytes + (TEAM ? warp * w_bytes : 0));
     float4* pr = pa + 16;
     float4* pd = pr + 16;
+    float4* part = pd + 16;   // TEAM: [CM][32] accumulators of a block begun by a warp before this one
     // this lane's slot of the pair buffers when it owns pair `lane`
     const int slot = (lane >> 3) * 4 + t, half = (lane >> 2) & 1;
     const int off0 = slot * 4 + half + ((lane >> 4) << 1), off1 = slot * 4 + half + (2 - ((lane >> 4) << 1));
@@ -242,13 +299,14 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
             *reinterpret_cast<float2*>(out + idx) = make_float2(v0, v1);
         }
     };
-    for (int64_t i = (int64_t)blockIdx.x * kMW + warp; i < w.N; i += (int64_t)gridDim.x * kMW) {
+    for (int64_t i = TEAM ? blockIdx.x / ctas : (int64_t)blockIdx.x * kMW + warp; i < w.N;
+         i += TEAM ? gridDim.x / ctas : (int64_t)gridDim.x * kMW) {
         const int64_t row = row_map ? row_map[i] : i;
         if (row < 0) continue;   // ghosts are not centres
         const int n = w.nb_count[i];
         const size_t sb = (size_t)i * cap;
-        __syncwarp();   // the previous atom's reads of the staging area are done
-        for (int k = lane; k < n; k += 32) {
+        sync();   // the previous atom's reads of the staging area are done
+        for (int k = tid; k < n; k += threads) {
             const float4 v = w.nb_vec[sb + k];
             if (FAST) {
                 const float ir = 1.f / v.w;
@@ -283,10 +341,28 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
             }
         }
         species_segments(d, w.nb_idx + sb, n, seg, lane);
-        __syncwarp();
+        sync();
 
+        if (TEAM) {
+            // radial terms: eight lanes per species and shell, each every eighth entry
+            const int items = d.S * d.n_rad;
+            for (int x0 = rank * (threads / 8); x0 < items; x0 += ctas * (threads / 8)) {
+                const int x = x0 + tid / 8, sp = x / d.n_rad, nn = x - sp * d.n_rad;
+                float acc = 0.f;
+                if (x < items) {
+                    const float rs = d.rs_rad[nn];
+                    for (int k = seg[sp] + (tid & 7); k < seg[sp + 1]; k += 8) {
+                        const float xr = sv[k].w - rs;
+                        acc = fmaf(ex2f(-eta_rl * (xr * xr)), sl[k].w, acc);
+                    }
+                }
+#pragma unroll
+                for (int o = 4; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (x < items && (tid & 7) == 0) put((size_t)row * d.D + x, acc);
+            }
+        }
         // radial terms: lanes over shells
-        for (int nn = lane; nn < d.n_rad; nn += 32) {
+        for (int nn = lane; !TEAM && nn < d.n_rad; nn += 32) {
             const float rs = d.rs_rad[nn];
             for (int sp = 0; sp < d.S; ++sp) {
                 float acc = 0.f;
@@ -316,16 +392,59 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
             // where it is not small (y near 1)
             const float two = FAST ? fmaf(2.f * d.zeta, d.r_half - (y0.x - 1.f), 2.f) : 2.f;
             const float2 me = dup(-d.eta_ang * 1.4426950408889634f);
+            // rows g (A_hi) and g + 8 (A_lo), shells 2 t and 2 t + 1 of a block's sums
+            auto flush = [&](int blk, const float (&acc)[CM][4]) {
+#pragma unroll
+                for (int mc = 0; mc < CM; ++mc) {
+                    const int m = m0 + mc * 8 + g, nq = n0 + 2 * t;
+                    const float v0 = two * (acc[mc][0] + acc[mc][2]), v1 = two * (acc[mc][1] + acc[mc][3]);
+                    const size_t o = (size_t)row * d.D + d.rad_cols + blk * nbins + m * d.n_ang_r + nq;
+                    if (m < d.n_theta) {
+                        if (even && nq < d.n_ang_r) {
+                            put2(o, v0, v1);
+                        } else {
+                            if (nq < d.n_ang_r) put(o, v0);
+                            if (nq + 1 < d.n_ang_r) put(o + 1, v1);
+                        }
+                    }
+                }
+            };
+            auto put_part = [&](const float (&v)[CM][4], float4* to) {
+#pragma unroll
+                for (int mc = 0; mc < CM; ++mc) to[mc * 32 + lane] = make_float4(v[mc][0], v[mc][1], v[mc][2], v[mc][3]);
+            };
+            auto add_part = [&](float (&v)[CM][4], const float4* from) {
+#pragma unroll
+                for (int mc = 0; mc < CM; ++mc) {
+                    const float4 x = from[mc * 32 + lane];
+                    v[mc][0] += x.x; v[mc][1] += x.y; v[mc][2] += x.z; v[mc][3] += x.w;
+                }
+            };
+            TeamRounds rounds(d, seg, wt, team);   // not TEAM: unused
+            // TEAM: block that later warps share, the end of its rounds; that of a block begun by earlier ones
+            int open = -1, open_end = 0, cont_end = 0;
             int blk = 0;
+            float acc[CM][4], comp[FAST ? 1 : CM][4];
             for (int a = 0; a < d.S; ++a)
                 for (int b = a; b < d.S; ++b, ++blk) {
-                    BlockPairs bp(seg[a], seg[a + 1] - seg[a], seg[b], seg[b + 1] - seg[b], a == b, lane);
-                    float acc[CM][4], comp[FAST ? 1 : CM][4];
+                    int first = 0, last = 0;
+                    if (TEAM) {
+                        const int np = TeamRounds::block_pairs(seg, a, b);
+                        rounds.next(np, first, last);
+                        if (np == 0 && wt == 0) {
+                            const float zero[CM][4] = {};
+                            flush(blk, zero);
+                        }
+                        if (first >= last) continue;
+                    }
+                    BlockPairs bp(seg[a], seg[a + 1] - seg[a], seg[b], seg[b + 1] - seg[b], a == b,
+                                  lane + 32 * first);
+                    const int end = TEAM ? min(bp.n, 32 * last) : bp.n;
 #pragma unroll
                     for (int mc = 0; mc < CM; ++mc)
 #pragma unroll
                         for (int q = 0; q < 4; ++q) acc[mc][q] = comp[FAST ? 0 : mc][q] = 0.f;
-                    for (int p0 = 0; p0 < bp.n; p0 += 32, bp.next()) {
+                    for (int p0 = 32 * first; p0 < end; p0 += 32, bp.next()) {
                         // step 1: geometry of the lane's pair (weight 0 past the block's end)
                         {
                             const bool on = p0 + lane < bp.n;
@@ -449,22 +568,44 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
                             }
                         __syncwarp();
                     }
-                    // rows g (A_hi) and g + 8 (A_lo), shells 2 t and 2 t + 1
-#pragma unroll
-                    for (int mc = 0; mc < CM; ++mc) {
-                        const int m = m0 + mc * 8 + g, nq = n0 + 2 * t;
-                        const float v0 = two * (acc[mc][0] + acc[mc][2]), v1 = two * (acc[mc][1] + acc[mc][3]);
-                        const size_t o = (size_t)row * d.D + d.rad_cols + blk * nbins + m * d.n_ang_r + nq;
-                        if (m < d.n_theta) {
-                            if (even && nq < d.n_ang_r) {
-                                put2(o, v0, v1);
-                            } else {
-                                if (nq < d.n_ang_r) put(o, v0);
-                                if (nq + 1 < d.n_ang_r) put(o + 1, v1);
-                            }
-                        }
+                    if (TEAM && first > 0) {
+                        put_part(acc, part);
+                        cont_end = rounds.rb;
+                    } else if (TEAM && 32 * last < bp.n) {
+                        open = blk;   // the warp's last block: its sums stay in acc
+                        open_end = rounds.rb;
+                    } else {
+                        flush(blk, acc);
                     }
                 }
+            if (TEAM) {
+                // sums of the CTA's warps after this one in the block that ends before round `end`
+                const int R = rounds.R;
+                auto add_later = [&](int end) {
+                    for (int j = wt + 1; j < (rank + 1) * warps && R * j / team < end; ++j) {
+                        if (R * j / team == R * (j + 1) / team) continue;   // no rounds
+                        add_part(acc, part + (j - wt) * (int)(w_bytes / 16));
+                    }
+                };
+                __syncthreads();
+                if (open >= 0) add_later(open_end);
+                if (cont_end > 0 && R * (rank * warps) / team == rounds.lo) {
+                    // begun by an earlier CTA: the CTA's sum where its warp 0 would leave its part
+                    // (that of this warp, or of one without rounds)
+                    float sum[CM][4] = {};
+                    for (int j = wt; j < (rank + 1) * warps && R * j / team < cont_end; ++j)
+                        if (R * j / team < R * (j + 1) / team) add_part(sum, part + (j - wt) * (int)(w_bytes / 16));
+                    put_part(sum, part - warp * (int)(w_bytes / 16));
+                }
+                cluster_sync();
+                if (open >= 0) {
+                    for (int q = rank + 1; q < ctas && R * (q * warps) / team < open_end; ++q)
+                        if (R * (q * warps) / team < R * ((q + 1) * warps) / team)
+                            add_part(acc, cg::this_cluster().map_shared_rank(part - warp * (int)(w_bytes / 16), q));
+                    flush(open, acc);
+                }
+                cluster_sync();   // the parts are free again
+            }
         }
     }
 }
@@ -490,8 +631,14 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
 // takes the SM's data path for a cycle, also when lanes share addresses), so the pair buffers carry
 // single floats, f_c and f_c' stay in registers from step 1 to step 3, and FAST stages unit vectors.
 
+//
+// TEAM: as in the descriptor; each warp adds to copies of its own, which the CTAs and then the cluster's
+// first CTA sum at the end.
+
 struct AdjSmem {
-    int sv, sx, sr, sq, g, pa, pr, pts, pt1, total;   // byte offsets within a warp's area
+    int sv, sx, sr, g, atom;            // byte offsets within an atom's area, its size
+    int sq, pa, pr, pts, pt1, warp;     // and within a warp's
+    int total(int warps) const { return atom + warps * warp; }
 };
 __host__ __device__ inline AdjSmem adj_mma_smem(const DescDev& d, int cap, int nc, bool fast)
 {
@@ -500,38 +647,48 @@ __host__ __device__ inline AdjSmem adj_mma_smem(const DescDev& d, int cap, int n
     a.sv = 0;
     a.sx = a.sv + cap * 16;
     a.sr = a.sx + c2 * (fast ? 8 : 16);
-    a.sq = a.sr + (fast ? c4 * 4 : 0);
-    a.g = a.sq + nc * cap * 16;
-    a.pa = a.g + ((d.D + 3) & ~3) * 4;
+    a.g = a.sr + (fast ? c4 * 4 : 0);
+    a.atom = a.g + ((d.D + 3) & ~3) * 4;
+    a.sq = 0;
+    a.pa = a.sq + nc * cap * 16;
     a.pr = a.pa + 16 * 16;
     a.pts = a.pr + 16 * (fast ? 8 : 16);
     a.pt1 = a.pts + 128 * 8;
-    a.total = a.pt1 + 128 * 4;
+    a.warp = a.pt1 + 128 * 4;
     return a;
 }
 
-template <bool FAST, int CM, int PW>
-__global__ void __launch_bounds__(kMW * 32, CM == 1 ? 5 : 4)
+template <bool FAST, int CM, int PW, bool TEAM>
+__global__ void __launch_bounds__((TEAM ? kTeamMax : kMW) * 32, TEAM ? 2 : CM == 1 ? 5 : 4)
 k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict__ F, float* __restrict__ vir_atom,
           int nc)
 {
     extern __shared__ float4 sm4[];
-    __shared__ int s_seg[kMW][kMaxSpecies + 1];
+    __shared__ int s_seg[TEAM ? kTeamMax : kMW][kMaxSpecies + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int cap = w.cap;
+    const int warps = TEAM ? blockDim.x >> 5 : 1, tid = TEAM ? threadIdx.x : lane, threads = 32 * warps;
+    const int ctas = TEAM ? cg::this_cluster().num_blocks() : 1, rank = TEAM ? cg::this_cluster().block_rank() : 0;
+    const int wt = TEAM ? rank * warps + warp : 0, team = ctas * warps;   // its number among the atom's warps
     const AdjSmem lay = adj_mma_smem(d, cap, nc, FAST);
-    char* base = reinterpret_cast<char*>(sm4) + (size_t)warp * lay.total;
+    char* base = reinterpret_cast<char*>(sm4) + (TEAM ? 0 : (size_t)warp * (lay.atom + lay.warp));
+    char* base_w = base + lay.atom + (TEAM ? warp * lay.warp : 0);
+    auto sync = [&] {
+        if (!TEAM) __syncwarp();
+        else if (ctas > 1) cg::this_cluster().sync();
+        else __syncthreads();
+    };
     float4* sv = reinterpret_cast<float4*>(base + lay.sv);   // FAST: (unit vector, rho), else (v, r)
     float2* sx2 = reinterpret_cast<float2*>(base + lay.sx);  // FAST: (f_c, f_c')
     float4* sx4 = reinterpret_cast<float4*>(base + lay.sx);  // else (f_c, f_c', 1/r, -)
     float* sr = reinterpret_cast<float*>(base + lay.sr);     // FAST: r
-    float4* sq = reinterpret_cast<float4*>(base + lay.sq);   // nc copies of (sum X, sum dT/dr)
+    float4* sq = reinterpret_cast<float4*>(base_w + lay.sq); // nc copies of (sum X, sum dT/dr)
     float* sg = reinterpret_cast<float*>(base + lay.g);      // the atom's gradient row
-    float4* pa = reinterpret_cast<float4*>(base + lay.pa);   // pairs p, p + 8: sin, cos of th'/2 (FAST: cos, sin_eps)
-    float2* pr2 = reinterpret_cast<float2*>(base + lay.pr);  // pairs p, p + 8: FAST distance,
-    float4* pr4 = reinterpret_cast<float4*>(base + lay.pr);  // else its hi and lo parts
-    float2* pts = reinterpret_cast<float2*>(base + lay.pts); // the four lanes' parts of a pair's sums
-    float* pt1 = reinterpret_cast<float*>(base + lay.pt1);
+    float4* pa = reinterpret_cast<float4*>(base_w + lay.pa); // pairs p, p + 8: sin, cos of th'/2 (FAST: cos, sin_eps)
+    float2* pr2 = reinterpret_cast<float2*>(base_w + lay.pr);  // pairs p, p + 8: FAST distance,
+    float4* pr4 = reinterpret_cast<float4*>(base_w + lay.pr);  // else its hi and lo parts
+    float2* pts = reinterpret_cast<float2*>(base_w + lay.pts); // the four lanes' parts of a pair's sums
+    float* pt1 = reinterpret_cast<float*>(base_w + lay.pt1);
     const int my = (lane >> 4) * 8 + (lane & 7), half = (lane >> 3) & 1;
     float* pa_my = reinterpret_cast<float*>(pa) + my * 4 + half;
     float* pr_my = reinterpret_cast<float*>(pr2) + my * (FAST ? 2 : 4) + half;
@@ -556,22 +713,23 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
     const float s1 = FAST ? -2.f * d.eta_ang / s_eta : -2.f * d.eta_ang;
     const bool gvec = (d.D & 3) == 0 && (reinterpret_cast<uintptr_t>(g_rows) & 15) == 0;
 
-    for (int64_t i = (int64_t)blockIdx.x * kMW + warp; i < w.N; i += (int64_t)gridDim.x * kMW) {
+    for (int64_t i = TEAM ? blockIdx.x / ctas : (int64_t)blockIdx.x * kMW + warp; i < w.N;
+         i += TEAM ? gridDim.x / ctas : (int64_t)gridDim.x * kMW) {
         const int64_t row = w.row_of_atom[i];
         if (row < 0) continue;   // ghosts are not centres
         const int n = w.nb_count[i];
         const size_t sb = (size_t)i * cap;
-        __syncwarp();   // the previous atom's reads of the staging area are done
+        sync();   // the previous atom's reads of the staging area are done
         {
             const float* gi = g_rows + (size_t)row * d.D;
             if (gvec) {
-                for (int c = lane; c < d.D / 4; c += 32)
+                for (int c = tid; c < d.D / 4; c += threads)
                     reinterpret_cast<float4*>(sg)[c] = reinterpret_cast<const float4*>(gi)[c];
             } else {
-                for (int c = lane; c < d.D; c += 32) sg[c] = gi[c];
+                for (int c = tid; c < d.D; c += threads) sg[c] = gi[c];
             }
         }
-        for (int k = lane; k < n; k += 32) {
+        for (int k = tid; k < n; k += threads) {
             const float4 v = w.nb_vec[sb + k];
             const float ir = 1.f / v.w;
             float s_, c_;
@@ -585,13 +743,15 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
                 sv[k] = v;
                 sx4[k] = make_float4(fc, dfc, ir, 0.f);
             }
-            for (int c = 0; c < nc; ++c) sq[c * cap + k] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        for (int c = 0; c < nc; ++c)
+            for (int k = lane; k < n; k += 32) sq[c * cap + k] = make_float4(0.f, 0.f, 0.f, 0.f);
         species_segments(d, w.nb_idx + sb, n, seg, lane);
-        __syncwarp();
+        if (TEAM) __syncthreads();
+        else __syncwarp();
 
         // radial terms: four lanes per entry, each every fourth shell
-        for (int k0 = 0; k0 < n; k0 += 8) {
+        for (int k0 = 8 * wt; k0 < n; k0 += 8 * team) {
             const int k = k0 + g;
             float T0 = 0.f, T1 = 0.f;
             if (k < n) {
@@ -612,15 +772,22 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
             T1 += __shfl_xor_sync(0xffffffffu, T1, 2);
             if (k < n && t == 0) {
                 const float fc = FAST ? sx2[k].x : sx4[k].x, dfc = FAST ? sx2[k].y : sx4[k].y;
-                sq[k].w = fmaf(dfc, T0, -2.f * d.eta_rad * fc * T1);
+                sq[k].w = fmaf(dfc, T0, -2.f * d.eta_rad * fc * T1);   // the warp's own copy
             }
         }
         __syncwarp();
 
+        TeamRounds rounds(d, seg, wt, team);   // not TEAM: unused
         int blk = 0;
         for (int a = 0; a < d.S; ++a)
             for (int b = a; b < d.S; ++b, ++blk) {
-                BlockPairs bp(seg[a], seg[a + 1] - seg[a], seg[b], seg[b + 1] - seg[b], a == b, lane);
+                int first = 0, last = 0;
+                if (TEAM) {
+                    rounds.next(TeamRounds::block_pairs(seg, a, b), first, last);
+                    if (first >= last) continue;
+                }
+                BlockPairs bp(seg[a], seg[a + 1] - seg[a], seg[b], seg[b + 1] - seg[b], a == b, lane + 32 * first);
+                const int end = TEAM ? min(bp.n, 32 * last) : bp.n;
                 if (bp.n == 0) continue;
                 // T^T as B operands (sector g, shells t and t + 4), hi and lo
                 // FAST: and of T^T with its columns scaled by R - R_c (in the units of x)
@@ -635,7 +802,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
                     tf_split<true>(T, th[mc], tl[mc]);
                     if (FAST) tf_split<true>(__fmul2_rn(T, make_float2(nR0.x, nR1.x)), uh[mc], ul[mc]);
                 }
-                for (int p0 = 0; p0 < bp.n; p0 += 32, bp.next()) {
+                for (int p0 = 32 * first; p0 < end; p0 += 32, bp.next()) {
                     // step 1: geometry of the lane's pair
                     const bool on = p0 + lane < bp.n;
                     int k1, k2;
@@ -799,6 +966,25 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
                 }
             }
 
+        // TEAM: the warps' copies into the CTA's first; warp 0 of the cluster's first CTA then has them all
+        if (TEAM) {
+            __syncthreads();
+            for (int k = tid; k < n; k += threads) {
+                float4* q0 = reinterpret_cast<float4*>(base + lay.atom + lay.sq) + k;
+                float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int j = 0; j < warps; ++j) {
+                    const float4* qj = reinterpret_cast<float4*>(base + lay.atom + j * lay.warp + lay.sq) + k;
+                    for (int c = 0; c < nc; ++c) {
+                        const float4 o = qj[c * cap];
+                        z.x += o.x; z.y += o.y; z.z += o.z; z.w += o.w;
+                    }
+                }
+                *q0 = z;
+            }
+            sync();
+            if (wt > 0) continue;
+        }
+
         // entries' gradients, scattered to the forces
         float fx = 0.f, fy = 0.f, fz = 0.f;
         float vv[9];
@@ -806,8 +992,8 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
         for (int k = 0; k < 9; ++k) vv[k] = 0.f;
         for (int k = lane; k < n; k += 32) {
             float4 z = sq[k];
-            for (int c = 1; c < nc; ++c) {
-                const float4 o = sq[c * cap + k];
+            for (int c = 1; c < (TEAM ? ctas : nc); ++c) {
+                const float4 o = TEAM ? cg::this_cluster().map_shared_rank(sq, c)[k] : sq[c * cap + k];
                 z.x += o.x; z.y += o.y; z.z += o.z; z.w += o.w;
             }
             float4 v = sv[k];
@@ -838,6 +1024,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
         }
         add_centre(w, i, fx, fy, fz, vv, F, vir_atom, lane);
     }
+    if (TEAM) sync();   // the other CTAs' shared memory is read until here
 }
 
 int sm_count()
@@ -861,6 +1048,29 @@ cudaError_t launch_resident(Kern kern, int64_t N, size_t smem, cudaStream_t s, A
     return cudaGetLastError();
 }
 
+// a cluster per atom (TEAM)
+struct Team {
+    int ctas, warps;   // CTAs per cluster, warps per CTA
+};
+template <class Kern, class... Args>
+cudaError_t launch_team(Kern kern, int64_t N, Team tm, size_t smem, cudaStream_t s, Args... args)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)tm.ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(N * tm.ctas));
+    cfg.blockDim = dim3((unsigned)tm.warps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 constexpr size_t kMaxSmem = 200 * 1024;
 
 }  // namespace
@@ -872,7 +1082,23 @@ static bool adj_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 2.f
 
 static size_t desc_smem(const Work& w, const DescDev& d, bool fast)
 {
-    return kMW * (desc_fast(d, fast) ? desc_mma_warp_bytes<true>(w.cap) : desc_mma_warp_bytes<false>(w.cap));
+    return kMW * (desc_fast(d, fast) ? desc_mma_atom_bytes<true>(w.cap) + desc_mma_warp_bytes<true>(0)
+                                     : desc_mma_atom_bytes<false>(w.cap) + desc_mma_warp_bytes<false>(0));
+}
+
+// Warps per atom below kSplitAtoms atoms, where one warp each leaves SMs idle and its chain of rounds is the
+// kernel's time (descriptor / adjoint, us): 16 carbon atoms 117 / 112 with one warp, 23 / 23 with one CTA of
+// 16 warps, 14 / 15 with 64 warps of 8 CTAs; 850 atoms in molecules 17 / 22 with one, 20 / 18 with two.  The largest power of two with which all atoms are resident at 16
+// warps per SM (128 registers a thread).  Not with FAST, whose rows are those of large batches.
+static Team team_of(const Work& w, bool fast)
+{
+    Team tm{1, 1};
+    if (fast || w.N >= kSplitAtoms) return tm;
+    int n = 2;
+    while (n < kTeamMax * kTeamCtas && 2 * n * w.N <= (int64_t)16 * sm_count()) n *= 2;
+    tm.warps = std::min(n, kTeamMax);
+    tm.ctas = n / tm.warps;
+    return tm;
 }
 
 bool desc_mma_fits(const Work& w, const DescDev& d, bool fast)
@@ -884,7 +1110,7 @@ bool desc_mma_fits(const Work& w, const DescDev& d, bool fast)
 static int adj_copies(const Work& w, const DescDev& d, bool fast)
 {
     int nc = 4;
-    while (nc > 1 && (size_t)kMW * adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total > 44 * 1024) nc /= 2;
+    while (nc > 1 && (size_t)adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total(1) * kMW > 44 * 1024) nc /= 2;
     return nc;
 }
 
@@ -892,7 +1118,7 @@ static int adj_copies(const Work& w, const DescDev& d, bool fast)
 bool adj_mma_fits(const Work& w, const DescDev& d, bool fast)
 {
     return d.ang_kind == 0 && d.n_ang_r <= 8 && d.n_theta <= 16 &&
-           (size_t)kMW * adj_mma_smem(d, w.cap, 1, adj_fast(d, fast)).total <= kMaxSmem;
+           (size_t)kMW * adj_mma_smem(d, w.cap, 1, adj_fast(d, fast)).total(1) <= kMaxSmem;
 }
 
 cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_map, float* G_rows,
@@ -900,13 +1126,21 @@ cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_
 {
     if (!desc_mma_fits(w, d, fast)) return cudaErrorNotSupported;
     if (w.N == 0) return cudaSuccess;
+    const bool two = ((d.n_theta + 7) / 8) % 2 == 0;
+    const Team tm = team_of(w, desc_fast(d, fast));
+    if (tm.warps > 1) {
+        const size_t smem = desc_mma_atom_bytes<false>(w.cap) + tm.warps * desc_mma_warp_bytes<false>(two ? 2 : 1);
+        auto run = [&](auto kern) { return launch_team(kern, w.N, tm, smem, s, d, w, row_map, G_rows, Gh, Gl); };
+        if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8, true>) : run(k_desc_mma<false, 1, 8, true>);
+        if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13, true>) : run(k_desc_mma<false, 1, 13, true>);
+        return two ? run(k_desc_mma<false, 2, 0, true>) : run(k_desc_mma<false, 1, 0, true>);
+    }
     const size_t smem = desc_smem(w, d, fast);
     auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, row_map, G_rows, Gh, Gl); };
-    const bool two = ((d.n_theta + 7) / 8) % 2 == 0;
-    if (desc_fast(d, fast)) return two ? run(k_desc_mma<true, 2, 0>) : run(k_desc_mma<true, 1, 0>);
-    if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8>) : run(k_desc_mma<false, 1, 8>);
-    if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13>) : run(k_desc_mma<false, 1, 13>);
-    return two ? run(k_desc_mma<false, 2, 0>) : run(k_desc_mma<false, 1, 0>);
+    if (desc_fast(d, fast)) return two ? run(k_desc_mma<true, 2, 0, false>) : run(k_desc_mma<true, 1, 0, false>);
+    if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8, false>) : run(k_desc_mma<false, 1, 8, false>);
+    if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13, false>) : run(k_desc_mma<false, 1, 13, false>);
+    return two ? run(k_desc_mma<false, 2, 0, false>) : run(k_desc_mma<false, 1, 0, false>);
 }
 
 cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows, float* F, float* vir_atom,
@@ -914,14 +1148,27 @@ cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows,
 {
     if (!adj_mma_fits(w, d, fast)) return cudaErrorNotSupported;
     if (w.N == 0) return cudaSuccess;
-    int nc = adj_copies(w, d, fast);
-    const size_t smem = (size_t)kMW * adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total;
-    auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, g_rows, F, vir_atom, nc); };
     const bool two = d.n_theta > 8;
-    if (adj_fast(d, fast)) return two ? run(k_adj_mma<true, 2, 0>) : run(k_adj_mma<true, 1, 0>);
-    if (d.zeta >= 33.f) return two ? run(k_adj_mma<false, 2, 8>) : run(k_adj_mma<false, 1, 8>);
-    if (d.zeta >= 17.f) return two ? run(k_adj_mma<false, 2, 13>) : run(k_adj_mma<false, 1, 13>);
-    return two ? run(k_adj_mma<false, 2, 0>) : run(k_adj_mma<false, 1, 0>);
+    int nc = adj_copies(w, d, fast);
+    Team tm = team_of(w, adj_fast(d, fast));
+    if (tm.warps > 1) {
+        auto bytes = [&] { return (size_t)adj_mma_smem(d, w.cap, nc, false).total(tm.warps); };
+        while (nc > 1 && bytes() > 100 * 1024) nc /= 2;
+        while (tm.warps > 2 && bytes() > kMaxSmem) tm.warps /= 2;
+        const size_t smem = bytes();
+        auto run = [&](auto kern) { return launch_team(kern, w.N, tm, smem, s, d, w, g_rows, F, vir_atom, nc); };
+        if (d.zeta >= 33.f) return two ? run(k_adj_mma<false, 2, 8, true>) : run(k_adj_mma<false, 1, 8, true>);
+        if (d.zeta >= 17.f) return two ? run(k_adj_mma<false, 2, 13, true>) : run(k_adj_mma<false, 1, 13, true>);
+        return two ? run(k_adj_mma<false, 2, 0, true>) : run(k_adj_mma<false, 1, 0, true>);
+    }
+    const size_t smem = (size_t)adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total(1) * kMW;
+    auto run = [&](auto kern) {
+        return launch_resident(kern, w.N, smem, s, d, w, g_rows, F, vir_atom, nc);
+    };
+    if (adj_fast(d, fast)) return two ? run(k_adj_mma<true, 2, 0, false>) : run(k_adj_mma<true, 1, 0, false>);
+    if (d.zeta >= 33.f) return two ? run(k_adj_mma<false, 2, 8, false>) : run(k_adj_mma<false, 1, 8, false>);
+    if (d.zeta >= 17.f) return two ? run(k_adj_mma<false, 2, 13, false>) : run(k_adj_mma<false, 1, 13, false>);
+    return two ? run(k_adj_mma<false, 2, 0, false>) : run(k_adj_mma<false, 1, 0, false>);
 }
 
 }  // namespace panna

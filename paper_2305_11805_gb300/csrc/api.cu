@@ -390,12 +390,14 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
 
 // The matrix forms (descriptor 5, adjoint 6) where they apply, without measuring anything: from
 // kSplitAtoms atoms on they were the fastest on every workload measured, from 5-29-atom molecules
-// (descriptor 0.144 -> 0.068 ms for 1024 of them) to the 1M-atom box (below that size the old kernels
-// spread one atom over several warps).
+// (descriptor 0.144 -> 0.068 ms for 1024 of them) to the 1M-atom box.  Below, FP32 networks take them
+// with several warps per atom (descriptor + adjoint: 16 carbon atoms 93 -> 28 us, 64 diamond atoms 42 ->
+// 20 us, 850 atoms in 50 molecules 60 -> 38 us); with BF16 networks, whose rows are those of large
+// batches, the old kernels spread an atom over several warps and are tuned against them.
 int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
 {
     if (c->d.ang_kind != 0) return 0;   // the standard BP term has one kernel
-    if (w.N < kSplitAtoms) return -1;
+    if (w.N < kSplitAtoms && !acc) return -1;
     if (kind == KV_DESC && desc_mma_fits(w, c->d, !acc)) return 5;
     if (kind == KV_ADJ && adj_mma_fits(w, c->d, !acc)) return 6;
     return -1;
