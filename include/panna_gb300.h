@@ -236,14 +236,11 @@ panna_status panna_set_angular_precision(panna_ctx* ctx, int32_t mode);
  * take them without measuring.  With FP32 networks (extended angular terms) the descriptor's
  * candidates are variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that
  * the matrix forms do not take use variant 2 (adjoint: 5; the descriptor with FP32 networks: 0) and
- * smaller ones variant 0 (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks): a bit mask of the first layer's
- * products (descriptor width to first hidden width, almost all of the networks'
- * arithmetic) that run on the tensor cores with operands split into TF32 parts, the rest
- * staying on the CUDA cores in plain FP32: 1 = forward (three parts), 4 = tangent of the
- * weight-gradient pass (two parts), 8 = weight gradient (two parts); bit 2 (the input
- * gradient, whose forces sat at the 1e-5 bar rather than within it) is not accepted.  Default 4 | 8 = 12: the training-only products, so that energies
- * and forces are those of the plain FP32 path; the tensor cores' accumulation makes the
- * forward product about 6x less accurate than an FP32 dot product rounded to nearest.
+ * smaller ones variant 0 (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks):
+ * a bit mask of the products that run on the tensor cores, from FP32 operands split into TF32 parts with
+ * partial sums rounded to nearest in FP32 (more accurate than an FP32 dot product of the same length): 1 or
+ * 4 = the layers' products of at least 128 summands (forward, input gradient, tangents; batches past the
+ * single-launch path), 8 = the weight gradient's wide layers; bit 2 is not accepted.  Default 4 | 8 = 12.
  * 0 = everything on the CUDA cores.  Returns PANNA_ERR_INVALID_ARG for an unknown knob or
  * value.
  */

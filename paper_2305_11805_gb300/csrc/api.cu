@@ -84,7 +84,7 @@ struct panna_ctx {
     int ang_mode = 0;
     int autotune = 1;
     int force_variant[3] = {-1, -1, -1};   // descriptor, adjoint, jvp: -1 = tuned
-    int fp32_tc = TF32_TAN | TF32_WGRAD;   // FP32 networks: first-layer products on the tensor cores
+    int fp32_tc = 4 | X3_WGRAD;   // FP32 networks: products on the tensor cores (X3_* bits)
     int64_t norm_C = 0, norm_N = 0;   // loss normalisers (0 = the batch's own counts)
     LossOpts loss_opts{0, 0, 0, 0.0, 0.0};
     bool frozen[kMaxSpecies][kMaxLayers] = {};
@@ -134,7 +134,7 @@ struct Layout {
     float* wdot = nullptr;
     double* loss_part = nullptr;
     void* tc_ws = nullptr;   // BF16 tensor-core network buffers
-    void* tf_ws = nullptr;   // FP32 networks: TF32 first-layer buffers
+    float* wgrad_part = nullptr;   // FP32 networks: parts of the weight gradient on the tensor cores
     // dynamics: candidates of the last neighbour build (cutoff rc + skin), its positions
     int32_t* cand_count = nullptr;
     float4* cand_vec = nullptr;
@@ -144,13 +144,6 @@ struct Layout {
 };
 
 constexpr int kSplits = 16;
-
-// TF32_* products of the first layer that run on the tensor cores in this evaluation
-int tf32_mask(const panna_ctx* c, bool bf16, bool train)
-{
-    if (bf16 || !tf32_first_layer_ok(c->plan)) return 0;
-    return c->fp32_tc & (train ? (TF32_FWD | TF32_TAN | TF32_WGRAD) : TF32_FWD);
-}
 
 void carve(panna_ctx* c, Arena& a, int64_t N, int64_t C, bool train, bool bf16, Layout& L, int cap_c = 0)
 {
@@ -211,8 +204,9 @@ void carve(panna_ctx* c, Arena& a, int64_t N, int64_t C, bool train, bool bf16, 
     b.seg_off = w.seg_off;
     b.tile_start = w.tile_start;
     b.splits = kSplits;
+    b.status = w.status;
     if (bf16) L.tc_ws = a.take<char>(tc_workspace_bytes(p, N, true));
-    if (const int m = tf32_mask(c, bf16, train)) L.tf_ws = a.take<char>(tf32_workspace_bytes(p, N, m));
+    if (train && !bf16 && (c->fp32_tc & X3_WGRAD)) L.wgrad_part = a.take<float>(wgrad_workspace_bytes(p, N) / sizeof(float));
     if (cap_c > 0) {
         L.cand_count = a.take<int32_t>(N);
         L.cand_vec = a.take<float4>((size_t)N * cap_c);
@@ -520,28 +514,19 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
     double* E_cfg = rq.E_cfg ? rq.E_cfg : L.E_cfg_int;
     const bool need_forces = rq.forces || rq.train;
     const bool tc = rq.prec == PANNA_MLP_BF16 || rq.prec == PANNA_MLP_BF16_FAST;
-    const int tfm = tf32_mask(c, tc, grad);
-    const bool tf = tfm != 0;
     bool fused = false;
     if (tc) {
         // BF16 operands on the tensor cores: energies and dE/dG together
         CU(mlp_bf16_energy_grad(c->plan, L.mb, rq.theta, N, L.tc_ws, rq.prec == PANNA_MLP_BF16, L.E_rows, L.g,
                                 L.w.status, s, &nl, g16_ready));
     } else {
-        // FP32 networks: first-layer products of the mask on the tensor cores (TF32 parts), the rest on
-        // CUDA cores; small batches take forward pass, energies and input gradient in one launch
-        if (tf) CU(tf32_prepare(c->plan, L.mb, rq.theta, N, L.tf_ws, tfm, s, &nl));
-        if (!(tfm & TF32_FWD)) {
-            const cudaError_t es = mlp_small_rows(c->plan, L.mb, rq.theta, N, L.E_rows, need_forces ? L.g : nullptr,
-                                                  grad, s, &nl);
-            if (es != cudaErrorNotSupported) {
-                CU(es);
-                fused = true;
-            }
-        }
+        // FP32 networks: small batches take forward pass, energies and input gradient in one launch
+        const cudaError_t es = mlp_small_rows(c->plan, L.mb, rq.theta, N, L.E_rows, need_forces ? L.g : nullptr, grad,
+                                              s, &nl);
+        fused = es == cudaSuccess;
         if (!fused) {
-            if (tfm & TF32_FWD) CU(tf32_forward1(c->plan, L.mb, N, L.tf_ws, tfm, L.w.status, s, &nl));
-            CU(mlp_forward(c->plan, L.mb, rq.theta, N, s, &nl, (tfm & TF32_FWD) ? 1 : 0));
+            if (es != cudaErrorNotSupported) CU(es);
+            CU(mlp_forward(c->plan, L.mb, rq.theta, N, s, &nl));
             CU(mlp_energy_rows(c->plan, L.mb, N, L.E_rows, s, &nl));
         }
     }
@@ -596,10 +581,7 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
             CU(cudaMemsetAsync(L.wdot, 0, sizeof(float) * (size_t)N * c->d.D, s));
         }
         stage_mark(c, 6, s);
-        const bool tan_tc = tf && (tfm & TF32_TAN);
-        const WgradTc wtc{(tf && (tfm & TF32_WGRAD)) ? L.tf_ws : nullptr, tfm, L.w.status};
-        if (tan_tc) CU(tf32_tangent1(c->plan, L.mb, N, L.tf_ws, tfm, L.wdot, L.w.status, s, &nl));
-        CU(mlp_param_grad(c->plan, L.mb, rq.theta, N, L.wdot, L.alpha_rows, rq.dtheta, s, &nl, tan_tc, &wtc));
+        CU(mlp_param_grad(c->plan, L.mb, rq.theta, N, L.wdot, L.alpha_rows, rq.dtheta, s, &nl, L.wgrad_part));
         if (rq.train) CU(launch_penalty_grad(c->loss_opts, weight_ranges(c->plan), rq.theta, rq.dtheta, s, &nl));
     }
     if (c->profiling) cudaEventRecord(c->ev[kNumStages], s);
@@ -745,6 +727,7 @@ panna_status panna_create(const panna_desc_params* p, int32_t n_archs, const pan
     }
     pl.P = off;
     pl.n_out = archs[0].widths[archs[0].n_layers];
+    pl.x3 = (c->fp32_tc & X3_LAYERS) != 0;
     pl.max_hidden = 1;
     for (int l = 0; l <= pl.L; ++l) {
         int m = 0;
@@ -826,6 +809,7 @@ panna_status panna_set_tuning(panna_ctx* c, const char* knob, int32_t value)
         }
     if (strcmp(knob, "mlp_fp32") == 0 && value >= 0 && value <= 15 && !(value & 2)) {
         c->fp32_tc = value;
+        c->plan.x3 = (value & X3_LAYERS) != 0;
         return PANNA_OK;
     }
     return fail(PANNA_ERR_INVALID_ARG, "unknown tuning knob or value: %s=%d", knob, value);
@@ -1212,11 +1196,11 @@ panna_status panna_qeq_loss_grad(panna_ctx* c, const panna_system* sys, const fl
         }, acc_jvp);
         CU(launch_jvp(L.w, c->d, L.u, L.wdot, acc_jvp, s, &nl, vj));
         stage_mark(c, 6, s);
-        CU(mlp_param_grad(c->plan, L.mb, theta, N, L.wdot, nullptr, dtheta, s, &nl, false, nullptr,
+        CU(mlp_param_grad(c->plan, L.mb, theta, N, L.wdot, nullptr, dtheta, s, &nl, nullptr,
                           MLP_GRAD_TANGENT));
         QeqTrain tr{L.qbuf, L.u, L.mb.Ad[c->plan.L], L.alpha_cfg, q_ref, w_charge, L.mb.Adb, loss};
         CU(launch_qeq_response(c->qeq, L.w, L.mb.A[c->plan.L], ldL, tr, L.mb.Ab, ldL, s, &nl));
-        CU(mlp_param_grad(c->plan, L.mb, theta, N, L.wdot, nullptr, dtheta, s, &nl, false, nullptr,
+        CU(mlp_param_grad(c->plan, L.mb, theta, N, L.wdot, nullptr, dtheta, s, &nl, nullptr,
                           MLP_GRAD_REVERSE_SEEDED));
         CU(launch_penalty_grad(c->loss_opts, weight_ranges(c->plan), theta, dtheta, s, &nl));
         if (charges) CU(cudaMemcpyAsync(charges, L.qbuf, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));

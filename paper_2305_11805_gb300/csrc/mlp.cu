@@ -12,24 +12,6 @@
 
 namespace panna {
 
-__device__ __forceinline__ float act_f(int t, float z)
-{
-    switch (t) {
-    case PANNA_ACT_GAUSSIAN: return __expf(-z * z);
-    case PANNA_ACT_RELU: return z > 0.f ? z : 0.f;
-    case PANNA_ACT_TANH: return tanhf(z);
-    default: return z;
-    }
-}
-__device__ __forceinline__ float act_d1(int t, float z)
-{
-    switch (t) {
-    case PANNA_ACT_GAUSSIAN: return -2.f * z * __expf(-z * z);
-    case PANNA_ACT_RELU: return z > 0.f ? 1.f : 0.f;
-    case PANNA_ACT_TANH: { float h = tanhf(z); return 1.f - h * h; }
-    default: return 1.f;
-    }
-}
 __device__ __forceinline__ float act_d2(int t, float z)
 {
     switch (t) {
@@ -401,17 +383,30 @@ static int device_sms()
     return n_sm;
 }
 
-// One layer GEMM: the 64-row form (twice the CTAs, twice the resident warps per SM) when the
-// 128-row grid leaves SMs with fewer than two CTAs and the reduction is short (K <= 256);
-// else 128-row tiles.  On 17,780 rows the 64-row form took the K = 128 layers from 12.3 to
-// 10.1 us but the K = 768 first layer from 109 to 145 us (more weight-tile traffic and fewer
-// FMAs per shared-memory load), so long reductions keep the 128-row tiles.
+// One layer's product.  From 128 summands on the tensor cores' form (k_gemm_x3) is the faster and the more
+// accurate one (17,396 rows, K = 128, N = 32: 24 -> 16 us, error 2.0e-7 -> 1.1e-7; 300 rows: both 14.6 us);
+// with fewer, the split of its operands costs as much accuracy as the short sums do here (K = 65, input
+// gradient: 1.07e-7 against 1.03e-7) and it gains no time (10.5 and 12.5 us).
+// k_gemm: the 64-row form (twice the CTAs, twice the resident warps per SM) when the 128-row grid leaves SMs
+// with fewer than two CTAs and the reduction is short (K <= 256); else 128-row tiles.  On 17,780 rows the
+// 64-row form took the K = 128 layers from 12.3 to 10.1 us but the K = 768 first layer from 109 to 145 us
+// (more weight-tile traffic and fewer FMAs per shared-memory load), so long reductions keep the 128-row tiles.
+constexpr int kX3MinK = 128;
 template <bool B_TRANS, int PRO, int EPI>
-static void launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStream_t s, const LayerArgs& la,
-                        const float* theta, const int32_t* seg_off, const int32_t* tile_start, const float* A,
-                        int lda, const float* Zp, int ldp, float* C, int ldc, float* C2, const float* Ze, int lde)
+static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStream_t s, const LayerArgs& la,
+                               const float* theta, const MlpBuffers& b, const float* A, int lda, const float* Zp,
+                               int ldp, float* C, int ldc, float* C2, const float* Ze, int lde)
 {
+    const int32_t *seg_off = b.seg_off, *tile_start = b.tile_start;
     dim3 g = gemm_grid(p, N, n_max);
+    int kmin = la.K[0];
+    for (int q = 1; q < la.S; ++q) kmin = std::min(kmin, la.K[q]);
+    if (p.x3 && kmin >= kX3MinK) {
+        // a CTA takes a row tile's column tiles in turn once the row tiles fill the SMs
+        g.y = std::min<unsigned>(g.y, std::max(1u, (unsigned)device_sms() / g.x));
+        return launch_gemm_x3<B_TRANS, PRO, EPI>(g, s, la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc, C2, Ze,
+                                                 lde, b.status);
+    }
     int kmax = 0;
     for (int q = 0; q < la.S; ++q) kmax = std::max(kmax, la.K[q]);
     if ((int64_t)g.x * g.y < 2 * (int64_t)device_sms() && kmax <= 256) {
@@ -422,6 +417,7 @@ static void launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStream_t s, 
         k_gemm<B_TRANS, PRO, EPI, 128><<<g, 256, 0, s>>>(la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc,
                                                          C2, Ze, lde);
     }
+    return cudaGetLastError();
 }
 
 cudaError_t mlp_tiles(const MlpPlan& p, const int32_t* seg_off, int32_t* tile_start, cudaStream_t s, int* launches)
@@ -432,14 +428,15 @@ cudaError_t mlp_tiles(const MlpPlan& p, const int32_t* seg_off, int32_t* tile_st
 }
 
 cudaError_t mlp_forward(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, cudaStream_t s,
-                        int* launches, int l0)
+                        int* launches)
 {
-    for (int l = l0; l < p.L; ++l) {
+    for (int l = 0; l < p.L; ++l) {
         LayerArgs la = layer_args(p, l, false);
         const float* Ain = l == 0 ? b.G : b.A[l];
         const int lda = p.ld[l];
-        launch_gemm<true, PRO_NONE, EPI_FWD>(p, N, p.ld[l + 1], s, la, theta, b.seg_off, b.tile_start, Ain, lda,
+        cudaError_t e = launch_gemm<true, PRO_NONE, EPI_FWD>(p, N, p.ld[l + 1], s, la, theta, b, Ain, lda,
                                              nullptr, 0, b.Z[l + 1], p.ld[l + 1], b.A[l + 1], nullptr, 0);
+        if (e != cudaSuccess) return e;
         ++*launches;
     }
     return cudaGetLastError();
@@ -460,8 +457,9 @@ cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         LayerArgs la = layer_args(p, l, true);
         float* out = l == 0 ? g : nxt;
         const int ldo = p.ld[l];
-        launch_gemm<false, PRO_DACT, EPI_STORE>(p, N, p.ld[l], s, la, theta, b.seg_off, b.tile_start, cur,
+        cudaError_t e = launch_gemm<false, PRO_DACT, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, cur,
                                                 p.ld[l + 1], b.Z[l + 1], p.ld[l + 1], out, ldo, nullptr, nullptr, 0);
+        if (e != cudaSuccess) return e;
         ++*launches;
         float* t = cur; cur = out; nxt = t;
     }
@@ -471,15 +469,16 @@ cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
 
 cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N,
                            const float* wdot, const float* alpha_rows, float* dtheta, cudaStream_t s,
-                           int* launches, bool tan_tc, const WgradTc* wtc, MlpGradPart part)
+                           int* launches, float* wgrad_part, MlpGradPart part)
 {
     // forward tangent along wdot: zdot_l = adot_{l-1} W_l^T, adot_l = act'(z_l) zdot_l
-    for (int l = tan_tc ? 1 : 0; l < p.L && part != MLP_GRAD_REVERSE_SEEDED; ++l) {
+    for (int l = 0; l < p.L && part != MLP_GRAD_REVERSE_SEEDED; ++l) {
         LayerArgs la = layer_args(p, l, false);
         const float* Ain = l == 0 ? wdot : b.Ad[l];
-        launch_gemm<true, PRO_NONE, EPI_TAN>(p, N, p.ld[l + 1], s, la, theta, b.seg_off, b.tile_start, Ain,
+        cudaError_t e = launch_gemm<true, PRO_NONE, EPI_TAN>(p, N, p.ld[l + 1], s, la, theta, b, Ain,
                                              p.ld[l], nullptr, 0, b.Zd[l + 1], p.ld[l + 1], b.Ad[l + 1], b.Z[l + 1],
                                              p.ld[l + 1]);
+        if (e != cudaSuccess) return e;
         ++*launches;
     }
     if (part == MLP_GRAD_TANGENT) return cudaGetLastError();
@@ -497,8 +496,8 @@ cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         LayerArgs lw = layer_args(p, l, false);
         const float* Ain = l == 0 ? b.G : b.A[l];
         const float* Adin = l == 0 ? wdot : b.Ad[l];
-        if (wtc && wtc->ws) {
-            cudaError_t e = tf32_wgrad(p, b, N, wtc->ws, wtc->mask, l, Ain, Adin, dtheta, wtc->status, s, launches);
+        if (wgrad_part) {
+            cudaError_t e = wgrad_layer(p, b, N, wgrad_part, l, lw, Ain, Adin, dtheta, s, launches);
             if (e != cudaSuccess) return e;
         } else {
             int kmax = 0, nmax = 0;
@@ -511,14 +510,16 @@ cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         if (l > 0) {
             // abar_{l} = Zb W_{l+1}, adotbar_{l} = Zdb W_{l+1}
             LayerArgs la = layer_args(p, l, true);
-            launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b.seg_off, b.tile_start, b.Zb,
+            cudaError_t e = launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, b.Zb,
                                                     ldl, nullptr, 0, b.Ab, p.ld[l], nullptr, nullptr, 0);
-            launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b.seg_off, b.tile_start, b.Zdb,
+            if (e != cudaSuccess) return e;
+            e = launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, b.Zdb,
                                                     ldl, nullptr, 0, b.Adb, p.ld[l], nullptr, nullptr, 0);
+            if (e != cudaSuccess) return e;
             *launches += 2;
         }
     }
-    if (!(wtc && wtc->ws)) {
+    if (!wgrad_part) {
         k_reduce_splits<<<(unsigned)((p.P + 255) / 256), 256, 0, s>>>(p.P, b.splits, b.part, dtheta);
         ++*launches;
     }

@@ -10,6 +10,26 @@ constexpr int kGM = 128, kGN = 128, kGK = 8;     // layer GEMM tiles (k_gemm): 2
 enum { PRO_NONE = 0, PRO_DACT = 1 };
 enum { EPI_STORE = 0, EPI_FWD = 1, EPI_TAN = 2 };
 
+// activations and their derivatives
+__device__ __forceinline__ float act_f(int t, float z)
+{
+    switch (t) {
+    case PANNA_ACT_GAUSSIAN: return __expf(-z * z);
+    case PANNA_ACT_RELU: return z > 0.f ? z : 0.f;
+    case PANNA_ACT_TANH: return tanhf(z);
+    default: return z;
+    }
+}
+__device__ __forceinline__ float act_d1(int t, float z)
+{
+    switch (t) {
+    case PANNA_ACT_GAUSSIAN: return -2.f * z * __expf(-z * z);
+    case PANNA_ACT_RELU: return z > 0.f ? 1.f : 0.f;
+    case PANNA_ACT_TANH: { float h = tanhf(z); return 1.f - h * h; }
+    default: return 1.f;
+    }
+}
+
 // Per-species shape of one layer as a kernel argument.
 struct LayerArgs {
     int S;
@@ -27,6 +47,7 @@ struct MlpPlan {
     int64_t P;                // total parameters
     int max_hidden;           // max over l >= 1 of ld[l]
     int n_out;                // output width: 1 (energy) or 3 (charge equilibration)
+    bool x3;                  // FP32 layer products on the tensor cores (mlp_x3.cu)
 };
 
 // Device buffers of one evaluation (rows in species order).
@@ -41,12 +62,17 @@ struct MlpBuffers {
     int splits;
     const int32_t* seg_off;
     int32_t* tile_start;
+    DevStatus* status;
 };
 
+// One layer's product on the tensor cores from split FP32 operands (mlp_x3.cu); arguments of k_gemm
+template <bool B_TRANS, int PRO, int EPI>
+cudaError_t launch_gemm_x3(dim3 grid, cudaStream_t s, const LayerArgs& la, const float* theta, const int32_t* seg_off,
+                           const int32_t* tile_start, const float* A, int lda, const float* Zp, int ldp, float* C,
+                           int ldc, float* C2, const float* Ze, int lde, DevStatus* status);
+
 cudaError_t mlp_tiles(const MlpPlan& p, const int32_t* seg_off, int32_t* tile_start, cudaStream_t s, int* launches);
-// layers l0 .. L-1 (l0 = 1 when the first layer ran on the tensor cores)
-cudaError_t mlp_forward(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, cudaStream_t s, int* launches,
-                        int l0 = 0);
+cudaError_t mlp_forward(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, cudaStream_t s, int* launches);
 cudaError_t mlp_energy_rows(const MlpPlan& p, const MlpBuffers& b, int64_t N, float* E_rows, cudaStream_t s, int* launches);
 // g = dE/dG; with ab1 != nullptr the chain stops at dE/dA_1 (row stride ld[1]), returned in *ab1;
 // seeded: b.Ab already holds the output seeds (rows, stride ld[L]) instead of dE/da_L = 1
@@ -68,37 +94,23 @@ cudaError_t mlp_bf16_energy_grad(const MlpPlan& p, const MlpBuffers& b, const fl
 // the BF16 descriptor operand rows (hi, lo; lo null without split) inside the workspace ws, or
 // null when the descriptor width is not a multiple of 8
 void tc_g16(const MlpPlan& p, int64_t N, bool split, void* ws, __nv_bfloat16** hi, __nv_bfloat16** lo);
-struct WgradTc;
 // Parts of the weight-gradient pass: both (default); the forward tangent along wdot only (the
 // output tangents land in b.Ad[L]); or the reverse pass only, with the output seeds already in
 // b.Ab (energy part) and b.Adb (force part), rows of stride ld[L]
 enum MlpGradPart { MLP_GRAD_ALL = 0, MLP_GRAD_TANGENT = 1, MLP_GRAD_REVERSE_SEEDED = 2 };
-// tan_tc: the first layer's tangent ran on the tensor cores (tf32_tangent1); wtc (non-null
-// ws): every layer's weight gradient on the tensor cores (tf32_wgrad)
+// wgrad_part (non-null: wgrad_workspace_bytes): the weight gradients on the tensor cores (wgrad_layer)
 cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, const float* wdot,
                            const float* alpha_rows, float* dtheta, cudaStream_t s, int* launches,
-                           bool tan_tc = false, const WgradTc* wtc = nullptr, MlpGradPart part = MLP_GRAD_ALL);
+                           float* wgrad_part = nullptr, MlpGradPart part = MLP_GRAD_ALL);
 
-// FP32 networks with the first layer on the tensor cores as TF32 hi + lo pairs (mlp_tc.cu).
-// Order per call: tf32_prepare, tf32_forward1, mlp_forward(l0 = 1); mlp_input_grad; for
-// training tf32_tangent1, then mlp_param_grad(tan_tc, wtc), which calls tf32_wgrad for every
-// layer.
-// Each of the four products may also stay on the CUDA cores (TF32_* bits below).
-enum { TF32_FWD = 1, TF32_INGRAD = 2, TF32_TAN = 4, TF32_WGRAD = 8 };   // TF32_INGRAD: not offered
-bool tf32_first_layer_ok(const MlpPlan& p);
-// mask: the TF32_* products used in this evaluation (the same value in every call of one evaluation)
-size_t tf32_workspace_bytes(const MlpPlan& p, int64_t N, int mask);
-cudaError_t tf32_prepare(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, void* ws, int mask,
-                         cudaStream_t s, int* launches);
-cudaError_t tf32_forward1(const MlpPlan& p, const MlpBuffers& b, int64_t N, void* ws, int mask, DevStatus* status,
-                          cudaStream_t s, int* launches);
-cudaError_t tf32_tangent1(const MlpPlan& p, const MlpBuffers& b, int64_t N, void* ws, int mask, const float* Gdot,
-                          DevStatus* status, cudaStream_t s, int* launches);
-// weight gradient of layer l+1 from b.Zb, b.Zdb (its adjoints) and its inputs A, Ad
-cudaError_t tf32_wgrad(const MlpPlan& p, const MlpBuffers& b, int64_t N, void* ws, int mask, int l, const float* A,
-                       const float* Ad, float* dtheta, DevStatus* status, cudaStream_t s, int* launches);
+// Weight gradient of layer l + 1 (mlp_x3.cu): dW = Zb^T A + Zdb^T Ad, db = sum of Zb over the species'
+// atoms, into dtheta.  A, Ad: the layer's inputs [N, ld[l]]; b.Zb, b.Zdb: its adjoints [N, ld[l + 1]]
+size_t wgrad_workspace_bytes(const MlpPlan& p, int64_t N);
+cudaError_t wgrad_layer(const MlpPlan& p, const MlpBuffers& b, int64_t N, float* part, int l, const LayerArgs& la,
+                        const float* A, const float* Ad, float* dtheta, cudaStream_t s, int* launches);
 
-// context of the tensor-core weight gradients inside mlp_param_grad (null ws: CUDA cores)
-struct WgradTc { void* ws; int mask; DevStatus* status; };
+// FP32 networks' products on the tensor cores (knob "mlp_fp32"): the layers' (forward, input gradient and
+// tangents; either bit), the weight gradient's
+enum { X3_LAYERS = 1 | 4, X3_WGRAD = 8 };
 
 }  // namespace panna
