@@ -2,8 +2,8 @@
 //
 // Stages, all on the caller's stream:
 //   k_cfg_geom     one warp per configuration: frame, fractional bounding box, cell grid
-//                  (cells at least rc wide), image-shift table;
-//   k_bin          one thread per atom: fold into the cell, split the folded FP64
+//                  (cells at least rc wide), first cell, image-shift table;
+//   k_bin          one thread per atom: its configuration, fold into the cell, split the folded FP64
 //                  position into FP32 hi + lo, count atoms per cell;
 //   scan           exclusive scan of the cell counts;
 //   k_scatter / k_sort_cells   atoms of each cell, sorted by index (deterministic);
@@ -139,12 +139,6 @@ __device__ __forceinline__ int atom_config(const int64_t* __restrict__ off, int6
     return (int)lo;
 }
 
-__global__ void k_atom_cfg(const int64_t* __restrict__ off, int64_t C, int64_t N, int32_t* __restrict__ atom_cfg)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) atom_cfg[i] = atom_config(off, C, i);
-}
-
 // One warp per configuration (kCfgWarps per block).
 constexpr int kCfgWarps = 8;
 
@@ -161,12 +155,11 @@ __device__ __forceinline__ double warp_max_d(double v)
     return v;
 }
 
-// Geometry of configuration c by one warp: frame and inverse, grid of cells, image shifts; returns the
-// number of cells.  FP64 runs at 1/64 of the FP32 rate (a warp's instruction holds the SM's pipe for 16
+// Geometry of configuration c by one warp: frame and inverse, grid of cells, image shifts.  FP64 runs at 1/64 of the FP32 rate (a warp's instruction holds the SM's pipe for 16
 // cycles, a division or square root takes hundreds), so the axes go to lanes of their own, and without
 // a periodic direction (the frame is the identity) no product with the frame is formed: the same values.
-__device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc, int64_t c, CfgGeom& g,
-                                             DevStatus* st, int lane)
+__device__ __forceinline__ void cfg_geom_warp(const panna_system& sys, double rc, int64_t c, CfgGeom& g,
+                                              DevStatus* st, int lane)
 {
     const int64_t a0 = sys.atom_off[c], a1 = sys.atom_off[c + 1];
     int per[3];
@@ -272,25 +265,16 @@ __device__ __forceinline__ int cfg_geom_warp(const panna_system& sys, double rc,
     const int ncells = n[0] * n[1] * n[2];
     if (lane == 0) {
         g.ncells = ncells;
-        g.cell_base = 0;
+        // at most max(1, 2 atoms) cells: every configuration's first cell follows from its first atom
+        g.cell_base = 2 * a0 + c;
     }
-    return ncells;
 }
 
 __global__ void __launch_bounds__(kCfgWarps * 32)
-k_cfg_geom(panna_system sys, double rc, CfgGeom* __restrict__ geom, int64_t* __restrict__ cfg_cells, DevStatus* st)
+k_cfg_geom(panna_system sys, double rc, CfgGeom* __restrict__ geom, DevStatus* st)
 {
-    const int lane = threadIdx.x & 31;
     const int64_t c = (int64_t)blockIdx.x * kCfgWarps + (threadIdx.x >> 5);
-    if (c >= sys.n_cfg) return;
-    const int ncells = cfg_geom_warp(sys, rc, c, geom[c], st, lane);
-    if (lane == 0) cfg_cells[c] = ncells;
-}
-
-__global__ void k_set_cell_base(CfgGeom* __restrict__ geom, const int64_t* __restrict__ base, int64_t C)
-{
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < C) geom[c].cell_base = base[c];
+    if (c < sys.n_cfg) cfg_geom_warp(sys, rc, c, geom[c], st, threadIdx.x & 31);
 }
 
 // Folds atom i into configuration c's cell, writes its hi + lo position and lattice offset; returns
@@ -326,13 +310,15 @@ __device__ __forceinline__ int bin_atom(const panna_system& sys, int S, const Cf
 }
 
 __global__ void k_bin(panna_system sys, int S, const CfgGeom* __restrict__ geom,
-                      const int32_t* __restrict__ atom_cfg, int32_t* __restrict__ atom_cell,
+                      int32_t* __restrict__ atom_cfg, int32_t* __restrict__ atom_cell,
                       int64_t* __restrict__ cell_count, float4* __restrict__ pos_hi,
                       float4* __restrict__ pos_lo, int32_t* __restrict__ wrap, DevStatus* st)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= sys.n_atoms) return;
-    const CfgGeom& g = geom[atom_cfg[i]];
+    const int c = atom_config(sys.atom_off, sys.n_cfg, i);
+    atom_cfg[i] = c;
+    const CfgGeom& g = geom[c];
     int sp;
     const int local = bin_atom(sys, S, g, i, pos_hi, pos_lo, wrap, st, sp);
     atom_cell[i] = local;
@@ -1013,14 +999,7 @@ cudaError_t build_neighbors(Work& w, const DescDev& d, cudaStream_t s, int* laun
     } else {
         unsigned nbA = (unsigned)((N + 255) / 256);
         if (nbA == 0) nbA = 1;
-        k_atom_cfg<<<nbA, 256, 0, s>>>(sys.atom_off, C, N, w.atom_cfg);
-        k_cfg_geom<<<(unsigned)((C + kCfgWarps - 1) / kCfgWarps), kCfgWarps * 32, 0, s>>>(sys, d.rc_d, w.geom,
-                                                                                          w.cell_count, w.status);
-        *launches += 2;
-        // cell bases: scan of per-config cell counts (stored temporarily in cell_count[0..C))
-        e = exclusive_scan_i64(w.cell_count, w.cell_start, C, w.scan_tmp, s, launches);
-        if (e != cudaSuccess) return e;
-        k_set_cell_base<<<(unsigned)((C + 255) / 256), 256, 0, s>>>(w.geom, w.cell_start, C);
+        k_cfg_geom<<<(unsigned)((C + kCfgWarps - 1) / kCfgWarps), kCfgWarps * 32, 0, s>>>(sys, d.rc_d, w.geom, w.status);
         ++*launches;
         // total cells <= 2N + C by construction; clear the counters
         e = cudaMemsetAsync(w.cell_count, 0, sizeof(int64_t) * (w.cap_cells + 1), s);
