@@ -45,6 +45,7 @@ __device__ __forceinline__ bool tile_species(int S, const int32_t* tile_start, i
 //   B_TRANS (forward / tangent): op(B)[k][n] = W[n*K + k] (W is [N, K])
 //   else     (input gradient):   op(B)[k][n] = W[k*N + n] (W is [K, N])
 // PRO_DACT: A[r][k] is multiplied by act'(Zp[r][k]) on load (layer activation la.pact).
+// blockIdx.z = 1 (PRO_NONE, EPI_STORE): the same product of Zp into C2.
 // EPI_FWD:  C = Z = acc + b, C2 = act(Z);  EPI_TAN: C = acc, C2 = act'(Ze) * acc.
 //
 // BM x 128 tile per CTA of 256 threads, BM = 128 or 64; each thread owns BM/16 x 8 outputs
@@ -147,6 +148,10 @@ k_gemm(LayerArgs la, const float* __restrict__ theta, const int32_t* __restrict_
     __shared__ __align__(16) float As[2][kGK][kGM];
     __shared__ __align__(16) float Bs[2][kGK][kGN];
     constexpr int P = BM / 16;   // output rows per thread
+    if (PRO == PRO_NONE && EPI == EPI_STORE && blockIdx.z) {
+        A = Zp;
+        C = C2;
+    }
     const int tile = BM == 128 ? (int)blockIdx.x : (int)(blockIdx.x >> 1);
     int s;
     if (!tile_species(la.S, tile_start, tile, s)) return;
@@ -316,24 +321,59 @@ __global__ void k_reduce_splits(int64_t P, int splits, const float* __restrict__
 
 // Reverse-pass seeds and elementwise adjoints of one layer:
 //   Zb  = Ab * act'(Z) + Adb * act''(Z) * Zd,   Zdb = Adb * act'(Z)
-__global__ void k_layer_adjoint(LayerArgs la, const int32_t* __restrict__ seg_off, int64_t N, int ld,
-                                const float* __restrict__ Ab, const float* __restrict__ Adb,
-                                const float* __restrict__ Z, const float* __restrict__ Zd,
-                                float* __restrict__ Zb, float* __restrict__ Zdb)
+// 2^lg threads per row, V columns each at a time (V = 4 where rows are 16-byte aligned).  Bound: HBM traffic,
+// 24 bytes an element; a thread per element, with its 64-bit division, took 16.5 us for 17,396 x 128.
+template <int V>
+__global__ void __launch_bounds__(256)
+k_layer_adjoint(LayerArgs la, const int32_t* __restrict__ seg_off, int64_t N, int ld, int lg,
+                const float* __restrict__ Ab, const float* __restrict__ Adb, const float* __restrict__ Z,
+                const float* __restrict__ Zd, float* __restrict__ Zb, float* __restrict__ Zdb)
 {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * ld) return;
-    const int64_t r = idx / ld;
-    const int c = (int)(idx % ld);
-    if (r >= seg_off[la.S]) return;     // rows past the last species (ghost atoms have none)
+    const int64_t r = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> lg;
+    if (r >= N || r >= seg_off[la.S]) return;     // rows past the last species (ghost atoms have none)
     int s = 0;
     while (s < la.S - 1 && r >= seg_off[s + 1]) ++s;
-    if (c >= la.N[s]) return;
-    const int t = la.act[s];
-    const float z = Z[idx];
-    const float d1 = act_d1(t, z);
-    Zb[idx] = Ab[idx] * d1 + Adb[idx] * act_d2(t, z) * Zd[idx];
-    Zdb[idx] = Adb[idx] * d1;
+    const int t = la.act[s], n = la.N[s];
+    for (int c = (threadIdx.x & ((1 << lg) - 1)) * V; c < n; c += V << lg) {
+        const size_t at = (size_t)r * ld + c;
+        float z[V], zd[V], ab[V], adb[V], zb[V], zdb[V];
+        if (V == 4) {
+            *reinterpret_cast<float4*>(z) = *reinterpret_cast<const float4*>(Z + at);
+            *reinterpret_cast<float4*>(zd) = *reinterpret_cast<const float4*>(Zd + at);
+            *reinterpret_cast<float4*>(ab) = *reinterpret_cast<const float4*>(Ab + at);
+            *reinterpret_cast<float4*>(adb) = *reinterpret_cast<const float4*>(Adb + at);
+        } else {
+            z[0] = Z[at]; zd[0] = Zd[at]; ab[0] = Ab[at]; adb[0] = Adb[at];
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const float d1 = act_d1(t, z[j]);
+            zb[j] = ab[j] * d1 + adb[j] * act_d2(t, z[j]) * zd[j];
+            zdb[j] = adb[j] * d1;
+        }
+        // columns past the species' width (within its rows' ld) hold values that nothing reads
+        if (V == 4) {
+            *reinterpret_cast<float4*>(Zb + at) = *reinterpret_cast<const float4*>(zb);
+            *reinterpret_cast<float4*>(Zdb + at) = *reinterpret_cast<const float4*>(zdb);
+        } else {
+            Zb[at] = zb[0]; Zdb[at] = zdb[0];
+        }
+    }
+}
+
+static void launch_layer_adjoint(const LayerArgs& la, const MlpBuffers& b, int64_t N, int ld, const float* Z,
+                                 const float* Zd, cudaStream_t s)
+{
+    auto aligned = [](const float* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    const bool vec = ld % 4 == 0 && aligned(b.Ab) && aligned(b.Adb) && aligned(Z) && aligned(Zd) && aligned(b.Zb) &&
+                     aligned(b.Zdb);
+    const int per = vec ? ld / 4 : ld;
+    int lg = 0;
+    while (lg < 5 && (1 << lg) < per) ++lg;
+    const unsigned nb = (unsigned)(((N << lg) + 255) / 256);
+    if (nb == 0) return;
+    if (vec) k_layer_adjoint<4><<<nb, 256, 0, s>>>(la, b.seg_off, N, ld, lg, b.Ab, b.Adb, Z, Zd, b.Zb, b.Zdb);
+    else k_layer_adjoint<1><<<nb, 256, 0, s>>>(la, b.seg_off, N, ld, lg, b.Ab, b.Adb, Z, Zd, b.Zb, b.Zdb);
 }
 
 // last-layer seeds: Ab = alpha_row (energy part), Adb = -1 (force part), widths 1
@@ -404,12 +444,18 @@ static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStrea
     if (p.x3 && kmin >= kX3MinK) {
         // a CTA takes a row tile's column tiles in turn once the row tiles fill the SMs
         g.y = std::min<unsigned>(g.y, std::max(1u, (unsigned)device_sms() / g.x));
+        if (PRO == PRO_NONE && EPI == EPI_STORE) {
+            cudaError_t e = launch_gemm_x3<B_TRANS, PRO, EPI>(g, s, la, theta, seg_off, tile_start, Zp, lda, nullptr, 0, C2,
+                                                              ldc, nullptr, nullptr, 0, b.status);
+            if (e != cudaSuccess) return e;
+        }
         return launch_gemm_x3<B_TRANS, PRO, EPI>(g, s, la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc, C2, Ze,
                                                  lde, b.status);
     }
     int kmax = 0;
     for (int q = 0; q < la.S; ++q) kmax = std::max(kmax, la.K[q]);
-    if ((int64_t)g.x * g.y < 2 * (int64_t)device_sms() && kmax <= 256) {
+    if (PRO == PRO_NONE && EPI == EPI_STORE) g.z = 2;   // only used for pairs of products
+    if ((int64_t)g.x * g.y * g.z < 2 * (int64_t)device_sms() && kmax <= 256) {
         g.x *= 2;
         k_gemm<B_TRANS, PRO, EPI, 64><<<g, 256, 0, s>>>(la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc,
                                                         C2, Ze, lde);
@@ -489,8 +535,7 @@ cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
     }
     for (int l = p.L - 1; l >= 0; --l) {
         const int ldl = p.ld[l + 1];
-        k_layer_adjoint<<<(unsigned)((N * ldl + 255) / 256), 256, 0, s>>>(
-            layer_args(p, l, false), b.seg_off, N, ldl, b.Ab, b.Adb, b.Z[l + 1], b.Zd[l + 1], b.Zb, b.Zdb);
+        launch_layer_adjoint(layer_args(p, l, false), b, N, ldl, b.Z[l + 1], b.Zd[l + 1], s);
         ++*launches;
         // weight gradient of layer l+1
         LayerArgs lw = layer_args(p, l, false);
@@ -510,13 +555,10 @@ cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         if (l > 0) {
             // abar_{l} = Zb W_{l+1}, adotbar_{l} = Zdb W_{l+1}
             LayerArgs la = layer_args(p, l, true);
-            cudaError_t e = launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, b.Zb,
-                                                    ldl, nullptr, 0, b.Ab, p.ld[l], nullptr, nullptr, 0);
+            cudaError_t e = launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, b.Zb, ldl, b.Zdb, ldl,
+                                                                    b.Ab, p.ld[l], b.Adb, nullptr, 0);
             if (e != cudaSuccess) return e;
-            e = launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, b.Zdb,
-                                                    ldl, nullptr, 0, b.Adb, p.ld[l], nullptr, nullptr, 0);
-            if (e != cudaSuccess) return e;
-            *launches += 2;
+            ++*launches;
         }
     }
     if (!wgrad_part) {
