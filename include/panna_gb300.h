@@ -233,7 +233,7 @@ panna_status panna_set_angular_precision(panna_ctx* ctx, int32_t mode);
  * and 8 shells): one warp per atom (below 1216 atoms with FP32 networks: 2 to 64 warps of a cluster),
  * the products over sectors and shells on the tensor cores from operands split into TF32 parts; sums in
  * a fixed order.  Where they apply, batches of at least 1216 atoms and all batches with FP32 networks
- * take them without measuring.  With FP32 networks (extended angular terms) the descriptor's
+ * take them without measuring.  JVP 5: likewise (zeta >= 2, plain arithmetic), for batches of every size.  With FP32 networks (extended angular terms) the descriptor's
  * candidates are variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that
  * the matrix forms do not take use variant 2 (adjoint: 5; the descriptor with FP32 networks: 0) and
  * smaller ones variant 0 (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks):
@@ -249,8 +249,8 @@ panna_status panna_set_tuning(panna_ctx* ctx, const char* knob, int32_t value);
 /* The kernel variant that knob "descriptor", "adjoint" or "jvp" ran with in the last compute
  * call that used it (tuned or forced): 0 blocked, 1 flattened, 2 / 3 / 4 compensated with 32 / 16
  * / 8 lanes per (species block, theta chunk, R chunk) unit (adjoint 4: flattened units), 5
- * compensated in diagonal pair order (adjoint) or the matrix form (descriptor), 6 the adjoint's
- * matrix form; -1 before any such call or for an unknown knob. */
+ * compensated in diagonal pair order (adjoint) or the matrix form (descriptor, JVP), 6 the
+ * adjoint's matrix form; -1 before any such call or for an unknown knob. */
 int32_t panna_tuning_choice(const panna_ctx* ctx, const char* knob);
 
 /*

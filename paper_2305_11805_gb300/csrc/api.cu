@@ -65,9 +65,9 @@ struct Arena {
 };
 
 constexpr int kNumVariants = 7;   // most variants of one descriptor-family kernel
-// variants per kernel: descriptor 0..5, adjoint 0..6, JVP 0..4; the matrix form's number (-1: none)
-constexpr int kMmaVariant[3] = {5, 6, -1};
-constexpr int kKindVariants[3] = {6, 7, 5};
+// variants per kernel: descriptor 0..5, adjoint 0..6, JVP 0..5; the matrix form's number
+constexpr int kMmaVariant[3] = {5, 6, 5};
+constexpr int kKindVariants[3] = {6, 7, 6};
 const char* kStages[] = {"neighbors", "descriptor", "mlp", "adjoint", "forces", "jvp", "mlp_grad", "loss"};
 constexpr int kNumStages = 8;
 
@@ -382,7 +382,7 @@ template <class Launch>
 int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int prec, int kind, cudaStream_t s,
                    Launch launch, bool acc);
 
-// The matrix forms (descriptor 5, adjoint 6) where they apply, without measuring anything: from
+// The matrix forms (descriptor 5, adjoint 6, JVP 5) where they apply, without measuring anything: from
 // kSplitAtoms atoms on they were the fastest on every workload measured, from 5-29-atom molecules
 // (descriptor 0.144 -> 0.068 ms for 1024 of them) to the 1M-atom box.  Below, FP32 networks take them
 // with several warps per atom (descriptor + adjoint: 16 carbon atoms 93 -> 28 us, 64 diamond atoms 42 ->
@@ -391,6 +391,7 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
 int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
 {
     if (c->d.ang_kind != 0) return 0;   // the standard BP term has one kernel
+    if (kind == KV_JVP) return !acc && jvp_mma_fits(w, c->d) ? 5 : -1;
     if (w.N < kSplitAtoms && !acc) return -1;
     if (kind == KV_DESC && desc_mma_fits(w, c->d, !acc)) return 5;
     if (kind == KV_ADJ && adj_mma_fits(w, c->d, !acc)) return 6;
@@ -428,7 +429,8 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
     const int fallback = (sys->n_atoms < kSplitAtoms || ext) ? 0 : (kind == KV_ADJ ? 5 : 2);
     if (!c->autotune || c->async || sys->n_atoms == 0) return fallback;
     float ms[kNumVariants] = {};
-    const bool mma = kind == KV_DESC ? desc_mma_fits(w, c->d, !acc) : kind == KV_ADJ && adj_mma_fits(w, c->d, !acc);
+    const bool mma = kind == KV_DESC ? desc_mma_fits(w, c->d, !acc)
+                     : kind == KV_ADJ ? adj_mma_fits(w, c->d, !acc) : !acc && jvp_mma_fits(w, c->d);
     auto candidate = [&](int v) {
         if (v == kMmaVariant[kind]) return mma;
         return !ext || v < 2;

@@ -176,6 +176,8 @@ cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_
                             __nv_bfloat16* Gh, __nv_bfloat16* Gl, bool fast, cudaStream_t s);
 cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows, float* F, float* vir_atom,
                            bool fast, cudaStream_t s);
+bool jvp_mma_fits(const Work& w, const DescDev& d);
+cudaError_t launch_jvp_mma(const Work& w, const DescDev& d, const float* u, float* wdot_rows, cudaStream_t s);
 cudaError_t launch_jvp(const Work& w, const DescDev& d, const float* u, float* wdot_rows, bool acc, cudaStream_t s,
                        int* launches, int variant = 0);
 

@@ -727,15 +727,18 @@ k_wgrad_small4(int S, const int32_t* __restrict__ seg_off, int chunk,
 }
 
 // dtheta of one layer from the per-item partial sums (splits per item): n < K_s: weight W[m][n]; n ==
-// bias_col: bias b[m].  CTA: 32 outputs, the parts dealt to 8 threads each, whose sums are added in order
-// (one thread per output, a chain of 300 loads, took 15 us for 1024 molecules' 32 x 129 layer).
-constexpr int kRedWays = 8;
-__global__ void __launch_bounds__(32 * kRedWays)
+// bias_col: bias b[m].  CTA: 256 / WAYS outputs, the parts dealt to WAYS threads each, whose sums are added
+// in order.  Narrow layers have many parts: with one thread per output, a chain of 300 loads, 1024
+// molecules' 32 x 129 layer took 15 us, with eight 7; wide ones few: 8.5 us with one, 27 with eight.
+template <int WAYS>
+__global__ void __launch_bounds__(256)
 k_wgrad_reduce(LayerArgs la, const int32_t* __restrict__ seg_off, int chunk, int splits, int Mvalid, int ldn,
                int bias_col, const float* __restrict__ part, float* __restrict__ dtheta)
 {
-    __shared__ float sums[kRedWays][32];
-    const int64_t idx = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    constexpr int OUT = 256 / WAYS;
+    __shared__ float sums[WAYS][OUT];
+    const int x = threadIdx.x % OUT, y = threadIdx.x / OUT;
+    const int64_t idx = (int64_t)blockIdx.x * OUT + x;
     const int s = (int)(idx / ((int64_t)Mvalid * ldn));
     const int m = (int)((idx / ldn) % Mvalid);
     const int n = (int)(idx % ldn);
@@ -745,13 +748,16 @@ k_wgrad_reduce(LayerArgs la, const int32_t* __restrict__ seg_off, int chunk, int
         int it = 0;
         for (int q = 0; q < s; ++q) it += (seg_off[q + 1] - seg_off[q] + chunk - 1) / chunk;
         const int end = (it + (seg_off[s + 1] - seg_off[s] + chunk - 1) / chunk) * splits;
-        for (it = it * splits + threadIdx.y; it < end; it += kRedWays) acc += part[((size_t)it * Mvalid + m) * ldn + n];
+        for (it = it * splits + y; it < end; it += WAYS) acc += part[((size_t)it * Mvalid + m) * ldn + n];
     }
-    sums[threadIdx.y][threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.y || !on) return;
+    if (WAYS > 1) {
+        sums[y][x] = acc;
+        __syncthreads();
+        if (y) return;
 #pragma unroll
-    for (int w = 1; w < kRedWays; ++w) acc += sums[w][threadIdx.x];
+        for (int w = 1; w < WAYS; ++w) acc += sums[w][x];
+    }
+    if (!on) return;
     if (n < la.K[s]) dtheta[la.w_off[s] + (int64_t)m * la.K[s] + n] = acc;
     else dtheta[la.b_off[s] + m] = acc;
 }
@@ -828,8 +834,12 @@ cudaError_t wgrad_layer(const MlpPlan& p, const MlpBuffers& b, int64_t N, float*
                                              nullptr, M, b.status, WgradArgs{A, Ad, K, w.chunk});
     }
     const int64_t n = (int64_t)p.S * M * w.ldn;
-    k_wgrad_reduce<<<(unsigned)((n + 31) / 32), dim3(32, kRedWays), 0, s>>>(la, b.seg_off, w.chunk, w.splits, M, w.ldn, K,
-                                                                           part, dtheta);
+    if (w.narrow)
+        k_wgrad_reduce<8><<<(unsigned)((n + 31) / 32), 256, 0, s>>>(la, b.seg_off, w.chunk, w.splits, M, w.ldn, K, part,
+                                                                    dtheta);
+    else
+        k_wgrad_reduce<1><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(la, b.seg_off, w.chunk, w.splits, M, w.ldn, K, part,
+                                                                      dtheta);
     *launches += 2;
     return cudaGetLastError();
 }
