@@ -1359,6 +1359,11 @@ cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows,
     return two ? run(k_adj_mma<false, 2, 0, false>) : run(k_adj_mma<false, 1, 0, false>);
 }
 
+int small_rows_variant(const Work& w, const DescDev& d)
+{
+    return w.N < kSplitAtoms && d.zeta >= 16.f && desc_mma_fits(w, d, false) ? 5 : 0;
+}
+
 // exponents as for the adjoint's fast form
 bool jvp_mma_fits(const Work& w, const DescDev& d)
 {

@@ -489,7 +489,8 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
             stage_mark(c, 1, s);
             const int fv = c->force_variant[KV_DESC];
             CU(launch_descriptor(L.w, c->d, rq.G_out, nullptr, c->ang_mode != 2, s, &nl,
-                                 fv >= 0 ? fv : (sys->n_atoms < kSplitAtoms ? 0 : 2)));
+                                 fv >= 0 ? fv : sys->n_atoms >= kSplitAtoms ? 2
+                                 : c->ang_mode != 2 ? small_rows_variant(L.w, c->d) : 0));
             if (c->profiling) cudaEventRecord(c->ev[kNumStages], s);
             return PANNA_OK;
         }

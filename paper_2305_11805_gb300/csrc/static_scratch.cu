@@ -146,7 +146,7 @@ extern "C" panna_status panna_descriptors_static(const panna_desc_params* p, con
     // the array keeps the previous call's contents: clear what must start at zero
     cudaError_t e = cudaMemsetAsync(w.status, 0, sizeof(DevStatus), s);
     if (e == cudaSuccess) e = build_neighbors(w, d, s, &launches);
-    if (e == cudaSuccess) e = launch_descriptor(w, d, G, nullptr, true, s, &launches);
+    if (e == cudaSuccess) e = launch_descriptor(w, d, G, nullptr, true, s, &launches, small_rows_variant(w, d));
     DevStatus h{};
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, w.status, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
