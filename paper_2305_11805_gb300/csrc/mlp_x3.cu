@@ -24,10 +24,9 @@
 // three stages (128-byte rows, 128-byte swizzle); warp 24 issues the MMAs (M = 128, K = 8 each); warps 0..7
 // add up the finished accumulators and write out finished tiles.  Every wait is bounded: on time-out the CTA sets
 // PANNA_ERR_TIMEOUT, waits for what it issued, frees its TMEM and returns.
-// Bound: the shared-memory data path, which carries 96 KB of operand reads and 64 KB of writes a step, and
-// the waits between the roles (a step takes about 1,700 cycles, its MMAs 768; one set of 16 warps for
-// splitting and adding took 3,000).  Registers: none of the adders' sums may spill, shared memory leaves
-// the L1 no room for them.
+// Bound: the waits between the roles (a step takes about 1,700 cycles, its MMAs 768, issue is 50 % busy; one
+// set of 16 warps for splitting and adding took 3,000).  Registers: none of the adders' sums may spill,
+// shared memory leaves the L1 no room for them.
 // Measured (17,396 rows, us; k_gemm -> here): K = 768, N = 128: 110 -> 50; K = 128, N = 32: 24 -> 16; input
 // gradient K = 128, N = 768: 121 -> 49; tangent K = 768 (before: a pass that split the operand, then TMA and
 // MMAs) 86 -> 52; weight gradient 768 x 128 (before: passes that transposed and split both operands) 163 -> 93.
