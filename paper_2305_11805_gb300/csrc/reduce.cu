@@ -23,48 +23,71 @@ __device__ __forceinline__ double block_sum_d(double v)
     return t;   // valid in thread 0
 }
 
-// partial sums over chunk b of configuration c: one warp per (configuration, chunk)
+// partial sums over chunk b of configuration c: one warp per (configuration, chunk).  NV values each: the
+// energy, or with the virial's nine; FP64 runs at 1/64 of the FP32 rate, so what nobody asks for is not
+// summed.  One chunk per configuration (DIRECT): its sums are the result, and k_cfg_final is left out
+// (16 carbon atoms 10 -> 4 us, 1024 molecules 15 -> 5; without a virial 1,048,576 atoms 136 -> 30).
 constexpr int kCfgRedWarps = 8;
 
+template <int NV>
+__device__ __forceinline__ void cfg_warp_sum(double (&v)[NV])
+{
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+}
+
+template <int NV>
+__device__ __forceinline__ void cfg_store(const double (&v)[NV], int64_t c, double* E_cfg, double* virial)
+{
+    if (E_cfg) E_cfg[c] = v[0];
+    if (NV > 1 && virial)
+#pragma unroll
+        for (int k = 1; k < NV; ++k) virial[9 * c + k - 1] = v[k];
+}
+
+template <int NV, bool DIRECT>
 __global__ void __launch_bounds__(kCfgRedWarps * 32)
 k_cfg_partial(int64_t C, const int64_t* __restrict__ atom_off, int B, const int32_t* __restrict__ row_of_atom,
               const float* __restrict__ E_rows, const float* __restrict__ vir_atom, float* __restrict__ E_atom,
-              double* __restrict__ part)
+              double* __restrict__ part, double* __restrict__ E_cfg, double* __restrict__ virial)
 {
     const int lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)blockIdx.x * kCfgRedWarps + (threadIdx.x >> 5);
     if (gw >= C * B) return;
-    const int64_t c = gw / B;
-    const int b = (int)(gw % B);
+    const int64_t c = DIRECT ? gw : gw / B;
+    const int b = DIRECT ? 0 : (int)(gw % B);
     const int64_t a0 = atom_off[c], a1 = atom_off[c + 1];
-    const int64_t per = (a1 - a0 + B - 1) / B;
+    const int64_t per = DIRECT ? a1 - a0 : (a1 - a0 + B - 1) / B;
     const int64_t s0 = a0 + b * per, s1 = min(a1, s0 + per);
-    double v[kCfgVals];
+    double v[NV];
 #pragma unroll
-    for (int k = 0; k < kCfgVals; ++k) v[k] = 0.0;
+    for (int k = 0; k < NV; ++k) v[k] = 0.0;
     for (int64_t i = s0 + lane; i < s1; i += 32) {
         const int row = row_of_atom[i];
         const float e = row >= 0 ? E_rows[row] : 0.f;     // a ghost (row -1) adds nothing
         if (E_atom) E_atom[i] = e;
         if (row < 0) continue;
         v[0] += e;
-        if (vir_atom)
+        if (NV > 1 && vir_atom)
 #pragma unroll
-            for (int k = 0; k < 9; ++k) v[1 + k] += vir_atom[9 * i + k];
+            for (int k = 1; k < NV; ++k) v[k] += vir_atom[9 * i + k - 1];
     }
-#pragma unroll
-    for (int k = 0; k < kCfgVals; ++k)
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane == 0) {
+    cfg_warp_sum(v);
+    if (lane) return;
+    if (DIRECT) {
+        cfg_store(v, c, E_cfg, virial);
+    } else {
         double* out = part + ((size_t)c * B + b) * kCfgVals;
 #pragma unroll
-        for (int k = 0; k < kCfgVals; ++k) out[k] = v[k];
+        for (int k = 0; k < NV; ++k) out[k] = v[k];
     }
 }
 
 // one warp per configuration: lane l sums the chunks l, l + 32, ... in order, then a fixed
 // butterfly joins the lanes (the same order on every call: energies are bit-reproducible)
+template <int NV>
 __global__ void __launch_bounds__(kCfgRedWarps * 32)
 k_cfg_final(int64_t C, int B, const double* __restrict__ part, double* __restrict__ E_cfg,
             double* __restrict__ virial)
@@ -72,20 +95,14 @@ k_cfg_final(int64_t C, int B, const double* __restrict__ part, double* __restric
     const int lane = threadIdx.x & 31;
     const int64_t c = (int64_t)blockIdx.x * kCfgRedWarps + (threadIdx.x >> 5);
     if (c >= C) return;
-    double v[kCfgVals];
+    double v[NV];
 #pragma unroll
-    for (int k = 0; k < kCfgVals; ++k) v[k] = 0.0;
+    for (int k = 0; k < NV; ++k) v[k] = 0.0;
     for (int b = lane; b < B; b += 32)
 #pragma unroll
-        for (int k = 0; k < kCfgVals; ++k) v[k] += part[((size_t)c * B + b) * kCfgVals + k];
-#pragma unroll
-    for (int k = 0; k < kCfgVals; ++k)
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane == 0 && E_cfg) E_cfg[c] = v[0];
-    if (lane == 0 && virial)
-#pragma unroll
-        for (int k = 0; k < 9; ++k) virial[9 * c + k] = v[1 + k];
+        for (int k = 0; k < NV; ++k) v[k] += part[((size_t)c * B + b) * kCfgVals + k];
+    cfg_warp_sum(v);
+    if (lane == 0) cfg_store(v, c, E_cfg, virial);
 }
 
 int cfg_chunks(int64_t N, int64_t C)
@@ -94,15 +111,29 @@ int cfg_chunks(int64_t N, int64_t C)
     return (int)(B > 8192 ? 8192 : B);
 }
 
+template <int NV>
+static void cfg_reduce(const Work& w, const float* E_rows, const float* vir_atom, double* E_cfg, double* virial,
+                       float* E_atom, double* part, cudaStream_t s, int* launches)
+{
+    const int B = cfg_chunks(w.N, w.C);
+    const unsigned nb = (unsigned)((w.C * B + kCfgRedWarps - 1) / kCfgRedWarps), thr = kCfgRedWarps * 32;
+    ++*launches;
+    if (B == 1) {
+        k_cfg_partial<NV, true><<<nb, thr, 0, s>>>(w.C, w.sys->atom_off, B, w.row_of_atom, E_rows, vir_atom, E_atom, part,
+                                                   E_cfg, virial);
+        return;
+    }
+    k_cfg_partial<NV, false><<<nb, thr, 0, s>>>(w.C, w.sys->atom_off, B, w.row_of_atom, E_rows, vir_atom, E_atom, part,
+                                                E_cfg, virial);
+    k_cfg_final<NV><<<(unsigned)((w.C + kCfgRedWarps - 1) / kCfgRedWarps), thr, 0, s>>>(w.C, B, part, E_cfg, virial);
+    ++*launches;
+}
+
 cudaError_t launch_cfg_reduce(const Work& w, const float* E_rows, const float* vir_atom, double* E_cfg, double* virial,
                               float* E_atom, double* part, cudaStream_t s, int* launches)
 {
-    const int B = cfg_chunks(w.N, w.C);
-    k_cfg_partial<<<(unsigned)((w.C * B + kCfgRedWarps - 1) / kCfgRedWarps), kCfgRedWarps * 32, 0, s>>>(
-        w.C, w.sys->atom_off, B, w.row_of_atom, E_rows, vir_atom, E_atom, part);
-    k_cfg_final<<<(unsigned)((w.C + kCfgRedWarps - 1) / kCfgRedWarps), kCfgRedWarps * 32, 0, s>>>(w.C, B, part,
-                                                                                                  E_cfg, virial);
-    *launches += 2;
+    if (vir_atom || virial) cfg_reduce<kCfgVals>(w, E_rows, vir_atom, E_cfg, virial, E_atom, part, s, launches);
+    else cfg_reduce<1>(w, E_rows, vir_atom, E_cfg, virial, E_atom, part, s, launches);
     return cudaGetLastError();
 }
 
