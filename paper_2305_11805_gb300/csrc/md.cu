@@ -44,7 +44,7 @@ __device__ __forceinline__ double gauss_component(uint64_t seed, int64_t a, int6
 
 // (B of the step before when pending) B A O A: v += dt/2 a F; x += dt/2 v; v = c1 v + c2 sigma g;
 // x += dt/2 v.  Four lanes per atom, one per component: the normals' FP64 logarithm, root and sine are
-// the kernel's time (one lane per atom took all three in turn: 10 -> 5 us).  With a reference (positions
+// the kernel's time (one lane per atom took all three in turn: 10 -> 8 us).  With a reference (positions
 // of the last neighbour build), an atom that has moved more than sqrt(lim2) since then raises *stale,
 // and the positions folded with the lattice offsets of that build (wrap) go to pos_hi / pos_lo for the
 // list's refresh, so the image shifts stored with the candidates stay valid while atoms move.

@@ -9,8 +9,10 @@
 // meet in one butterfly.  Backward, a warp owns 128 inputs and a slice of the units; the slices' sums
 // meet in shared memory in a fixed order.
 //
-// The weights cross from L2 once per CTA, so the time grows with N / R.  Measured (forward + energies +
-// input gradient, against the GEMM path): see launch rule in mlp_small_rows.
+// The weights cross from L2 once per CTA, so the time grows with N / R.  Measured (forward + energies + input
+// gradient, us, here / layer by layer with k_gemm_x3 just past the line of 2,048 rows): 64 rows of
+// 96-256-128-32-1 28; 768-128-32-1: 850 rows 47, 1,960 rows 82 / 2,200 rows 103; 256-256-128-1: 2,000 rows 78 /
+// 2,052 rows 107; 192-128-64-1: 2,048 rows 45 / 2,916 rows 78.
 #include <algorithm>
 
 #include "mlp.cuh"

@@ -322,12 +322,12 @@ k_tc_gemm_p(const __grid_constant__ TcMaps tm, TcArgs a, int n_nt)
 #pragma unroll
                     for (int kk = 0; kk < BKE / MMAK; ++kk) {
                         const uint64_t a1 = sw128_desc(a0 + kk * 32), b1 = sw128_desc(b0 + kk * 32);
-                        tc_mma<false>(d, a1, b1, idesc, (kc | kk) ? 1u : 0u);
+                        tc_mma(d, a1, b1, idesc, (kc | kk) ? 1u : 0u);
                         if (PARTS >= 2) {
                             const uint64_t a2 = sw128_desc(a0 + kTileA + kk * 32);
                             const uint64_t b2 = sw128_desc(b0 + Cfg::kTileB + kk * 32);
-                            tc_mma<false>(d, a1, b2, idesc, 1u);
-                            tc_mma<false>(d, a2, b1, idesc, 1u);
+                            tc_mma(d, a1, b2, idesc, 1u);
+                            tc_mma(d, a2, b1, idesc, 1u);
                         }
                     }
                     tc_commit(empty + st);
