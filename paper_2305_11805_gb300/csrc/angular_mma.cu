@@ -277,7 +277,8 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
     const int ncm = (d.n_theta + 7) / 8, ncn = (d.n_ang_r + 7) / 8;
     const int nbins = d.n_theta * d.n_ang_r;
     const float eta_rl = d.eta_rad * 1.4426950408889634f;   // exp(-eta x^2) = 2^(-eta_l x^2)
-    const bool even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0;   // bin pairs on 8-byte boundaries
+    // bin pairs on 8-byte boundaries; FP32 rows may be the caller's own, which start at any float
+    const bool even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0 && (Gh || (reinterpret_cast<uintptr_t>(out) & 7) == 0);
     auto put = [&](size_t idx, float v) {
         if (Gh) {
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
