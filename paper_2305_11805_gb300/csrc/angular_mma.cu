@@ -1227,7 +1227,7 @@ int sm_count()
 template <class Kern, class... Args>
 cudaError_t launch_resident(Kern kern, int64_t N, size_t smem, cudaStream_t s, Args... args)
 {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMW * 32, smem);
@@ -1244,7 +1244,7 @@ struct Team {
 template <class Kern, class... Args>
 cudaError_t launch_team(Kern kern, int64_t N, Team tm, size_t smem, cudaStream_t s, Args... args)
 {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;

@@ -368,7 +368,7 @@ cudaError_t launch_bp(const Work& w, const DescDev& d, const int32_t* row_map, c
     while (nc > 1 && (size_t)kBWarps * bp_warp_floats(w.cap, MODE, nc) * 4 > 40 * 1024) nc /= 2;
     const size_t smem = (size_t)kBWarps * bp_warp_floats(w.cap, MODE, nc) * 4;
     auto run = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         kern<<<(unsigned)((w.N + kBWarps - 1) / kBWarps), kBWarps * 32, smem, s>>>(d, w, row_map, in, out, F, vir_atom,
                                                                                   nc);

@@ -26,6 +26,24 @@ __device__ __forceinline__ void set_status(DevStatus* st, int32_t code, int32_t 
     if (atomicCAS(&st->code, 0, code) == 0) st->bad_index = idx;
 }
 
+// Lets a launch of `kern` take `bytes` of dynamic shared memory.  The limit belongs to the kernel on the
+// device, not to a context or a thread, so it is only ever raised, and to the device's whole size: with each
+// launch setting its own batch's size, a thread with a smaller batch lowered the limit between another
+// thread's setting and its launch.
+template <class... Args>
+cudaError_t allow_smem(void (*kern)(Args...), size_t bytes)
+{
+    const void* f = reinterpret_cast<const void*>(kern);
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, f);
+    if (e != cudaSuccess || bytes <= (size_t)at.maxDynamicSharedSizeBytes) return e;
+    int dev = 0, all = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    if (bytes + at.sharedSizeBytes > (size_t)all) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, all - (int)at.sharedSizeBytes);
+}
+
 // Descriptor parameters as the kernels read them (FP32 copies plus FP64 cutoff).  The
 // struct is passed by value, so the grids sit in the kernel-parameter constant bank.
 constexpr int kMaxRad = 256;

@@ -251,7 +251,7 @@ template <int R>
 cudaError_t run_rows(const NetDev& p, const float* theta, int64_t N, const int32_t* seg_off, const float* G,
                      float* E_rows, float* g, int keep, size_t smem, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_rows<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_mlp_rows<R>, smem);
     if (e != cudaSuccess) return e;
     k_mlp_rows<R><<<(unsigned)((N + R - 1) / R + p.S), kRowThreads, smem, s>>>(p, theta, seg_off, G, E_rows, g, keep);
     return cudaGetLastError();

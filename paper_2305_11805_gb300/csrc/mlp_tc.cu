@@ -523,7 +523,7 @@ cudaError_t launch_tc_p(const TcMaps& m, const TcArgs& ta, int64_t N, int nmax, 
     const int64_t items = ((N + kTcBM - 1) / kTcBM + ta.S) * n_nt;
     const unsigned grid = (unsigned)std::min<int64_t>(items, n_sm);
     const int smem = (int)TcCfg<PARTS>::kSmem;
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm_p<EPI, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k_tc_gemm_p<EPI, PARTS>, smem);
     if (e != cudaSuccess) return e;
     k_tc_gemm_p<EPI, PARTS><<<grid, kTcThreads, smem, s>>>(m, ta, n_nt);
     return cudaGetLastError();

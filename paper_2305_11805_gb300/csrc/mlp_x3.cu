@@ -550,7 +550,7 @@ cudaError_t launch_gemm_x3(dim3 grid, cudaStream_t s, const LayerArgs& la, const
     bool vec = aligned(A) && lda % 4 == 0 && (PRO == PRO_NONE || (aligned(Zp) && ldp % 4 == 0));
     for (int q = 0; q < la.S; ++q) vec = vec && la.K[q] % 4 == 0;
     auto kern = vec ? k_gemm_x3<B_TRANS, PRO, EPI, OP_ROWS, true> : k_gemm_x3<B_TRANS, PRO, EPI, OP_ROWS, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXSmem);
+    cudaError_t e = allow_smem(kern, kXSmem);
     if (e != cudaSuccess) return e;
     kern<<<grid, kXThreads, kXSmem, s>>>(la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc, C2, Ze, lde, status,
                                          WgradArgs{});
@@ -826,7 +826,7 @@ cudaError_t wgrad_layer(const MlpPlan& p, const MlpBuffers& b, int64_t N, float*
             k_wgrad_small<<<grid, 256, smem, s>>>(p.S, b.seg_off, w.chunk, w.splits, M, K, b.Zb, b.Zdb, A, Ad, part);
     } else {
         auto kern = k_gemm_x3<false, PRO_NONE, EPI_STORE, OP_WGRAD, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXSmem);
+        cudaError_t e = allow_smem(kern, kXSmem);
         if (e != cudaSuccess) return e;
         dim3 grid((unsigned)w.items, (unsigned)((K + 127) / 128), (unsigned)((M + 127) / 128));
         kern<<<grid, kXThreads, kXSmem, s>>>(la, nullptr, b.seg_off, nullptr, b.Zb, M, b.Zdb, M, part, w.ldn, nullptr,

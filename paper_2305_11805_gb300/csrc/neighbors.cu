@@ -989,7 +989,7 @@ cudaError_t build_neighbors(Work& w, const DescDev& d, cudaStream_t s, int* laun
     w.rows_ready = false;
     if (N > 0 && N <= kSmallAtoms && C <= kSmallCfgs && w.row_of_atom) {
         const size_t smem_c = cells_small_smem(N, C);
-        e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
+        e = allow_smem(k_cells_small, smem_c);
         if (e != cudaSuccess) return e;
         const unsigned per_cfg = (unsigned)((N + C * kBinThreads - 1) / (C * kBinThreads));
         k_cfg_bin<<<dim3((unsigned)C, per_cfg), kBinThreads, 0, s>>>(sys, w, d.S, d.rc_d);
@@ -1020,7 +1020,7 @@ cudaError_t build_neighbors(Work& w, const DescDev& d, cudaStream_t s, int* laun
         *launches += 2;
     }
     size_t smem = (size_t)kNbWarps * w.cap * (sizeof(float4) + sizeof(int2) + (w.nb_vlo ? sizeof(float4) : 0));
-    e = cudaFuncSetAttribute(k_neighbors, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(k_neighbors, smem);
     if (e != cudaSuccess) return e;
     unsigned nbW = (unsigned)((N + kNbWarps - 1) / kNbWarps);
     if (nbW == 0) nbW = 1;

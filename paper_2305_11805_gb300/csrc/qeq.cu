@@ -338,8 +338,7 @@ static cudaError_t qeq_launch(const QeqDev& qp, const Work& w, const float* out,
 {
     if (w.C == 0) return cudaSuccess;
     const int classes[3] = {0, 32, kQeqMax};
-    cudaError_t e = cudaFuncSetAttribute(k_qeq<TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)qeq_smem_bytes(kQeqMax));
+    cudaError_t e = allow_smem(k_qeq<TRAIN>, qeq_smem_bytes(kQeqMax));
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);

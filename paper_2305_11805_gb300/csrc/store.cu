@@ -267,7 +267,7 @@ cudaError_t launch_store_jacobian(const Work& w, const DescDev& d, const DescGri
     const int warps = jac_warps(w.cap);
     if (warps < 1) return cudaErrorInvalidValue;
     const size_t smem = (size_t)warps * kJacStage * w.cap * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_store_jacobian, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_store_jacobian, smem);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((w.N + warps - 1) / warps);
     k_store_jacobian<<<nb, warps * 32, smem, s>>>(d, g, *w.sys, w, v);
@@ -606,7 +606,7 @@ template <int NP>
 static cudaError_t store_tangent_np(const StoreView& v, const DescDev& d, const float* u, float* wd, cudaStream_t s)
 {
     const size_t smem = (size_t)kStoreWarps * ((d.D + 3) & ~3) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_store_tangent_b<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_store_tangent_b<NP>, smem);
     if (e != cudaSuccess) return e;
     const unsigned nb = balanced_blocks(k_store_tangent_b<NP>, smem, v.N);
     k_store_tangent_b<NP><<<nb, kStoreWarps * 32, smem, s>>>(v, d, u, wd);
@@ -708,7 +708,7 @@ cudaError_t launch_store_tangent(const StoreView& v, const DescDev& d, const flo
     warps = warps > kStoreWarps ? kStoreWarps : warps;
     if (warps < 1) return cudaErrorInvalidValue;
     const size_t smem = (size_t)warps * row;
-    cudaError_t e = cudaFuncSetAttribute(k_store_tangent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_store_tangent, smem);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((v.N + warps - 1) / warps);
     k_store_tangent<<<nb, warps * 32, smem, s>>>(v, d, u, wdot_rows);
