@@ -652,7 +652,7 @@ k_jvp_mma(DescDev d, Work w, const float* __restrict__ u, float* __restrict__ ou
     const int ncm = (d.n_theta + 7) / 8, ncn = (d.n_ang_r + 7) / 8;
     const int nbins = d.n_theta * d.n_ang_r;
     const float r_c = d.rs_ang[d.n_ang_r / 2], s_eta = sqrtf(d.eta_ang * 1.4426950408889634f);
-    const float c_x = -2.f * d.eta_ang / s_eta, eta_rl = d.eta_rad * 1.4426950408889634f;
+    const float c_x = d.eta_ang > 0.f ? -2.f * d.eta_ang / s_eta : 0.f, eta_rl = d.eta_rad * 1.4426950408889634f;
     const bool even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0;
     for (int64_t i = (int64_t)blockIdx.x * kMW + warp; i < w.N; i += (int64_t)gridDim.x * kMW) {
         const int64_t row = w.row_of_atom[i];
@@ -899,7 +899,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
         }
     }
     // dT/dr = s1 Fp S1 + ...: x e in the units of nR0
-    const float s1 = FAST ? -2.f * d.eta_ang / s_eta : -2.f * d.eta_ang;
+    const float s1 = FAST && d.eta_ang > 0.f ? -2.f * d.eta_ang / s_eta : -2.f * d.eta_ang;
     const bool gvec = (d.D & 3) == 0 && (reinterpret_cast<uintptr_t>(g_rows) & 15) == 0;
 
     for (int64_t i = TEAM ? blockIdx.x / ctas : (int64_t)blockIdx.x * kMW + warp; i < w.N;
