@@ -468,7 +468,8 @@ panna_status run_once(panna_ctx* c, const panna_system* sys, const Request& rq, 
     if (!acc) L.w.nb_vlo = nullptr;   // the plain and compensated kernels read no low parts
     for (int k = 0; k < kNumStages; ++k) c->stage_seen[k] = false;
     c->n_marked = 0;
-    CU(cudaMemsetAsync(L.w.status, 0, sizeof(DevStatus), s));
+    // dynamics clears the word itself: it still holds what a rebuild of the list reported
+    if (!rq.cand) CU(cudaMemsetAsync(L.w.status, 0, sizeof(DevStatus), s));
     const StoreView* sv = rq.store;
     bool g16_ready = false;   // BF16 networks: the descriptor kernel wrote their operand rows
     if (sv) {
@@ -872,10 +873,20 @@ panna_status panna_md_run(panna_ctx* c, const panna_system* sys, double* vel, co
         ++builds;
         break;
     }
-    // Each step: integrate, read the status word (the step before's errors, this step's stale flag),
-    // forces.  With a skin the forces are enqueued before the status is waited for, so that the host's
-    // wait and launches overlap the GPU's work; a stale list (rare) is rebuilt and the forces redone.
+    // Each step: integrate, read the status word (the step before's errors, those of its rebuild among
+    // them, and this step's stale flag), forces.  With a skin the forces are enqueued before the status is
+    // waited for, so that the host's wait and launches overlap the GPU's work; a stale list (rare) is
+    // rebuilt and the forces redone, with the word cleared of what the stale list's forces reported.
     // The closing half kick of a step runs in the next step's integration kernel.
+    auto step_error = [&](const DevStatus& d, int64_t t) {
+        if (d.code == PANNA_ERR_NEIGHBOR_OVERFLOW && d.need_cap > c->cap_c)
+            return fail(PANNA_ERR_NEIGHBOR_OVERFLOW, "step %lld: atom %d has %d neighbours within the cutoff and the skin, "
+                        "capacity %d (raise the neighbour capacity and restart)", (long long)t, d.bad_index, d.need_cap,
+                        c->cap_c);
+        status_error(c, d);
+        return fail((panna_status)d.code, "step %lld: %s (raise the neighbour capacity and restart)", (long long)t,
+                    panna_last_error());
+    };
     for (int64_t t = 0; t < n_steps; ++t) {
         CU(launch_md_baoa(L.w, ms, pos, vel, F, p->dt, c1, c2, thermostat, p->seed, p->step0 + t, t > 0, L.pos_ref,
                           lim2, s));
@@ -887,11 +898,10 @@ panna_status panna_md_run(panna_ctx* c, const panna_system* sys, double* vel, co
         const DevStatus now = *c->h_status;
         if (now.code != PANNA_OK) {
             CU(cudaStreamSynchronize(s));
-            status_error(c, now);
-            return fail((panna_status)now.code, "step %lld: %s (raise the neighbour capacity and restart)", (long long)t,
-                        panna_last_error());
+            return step_error(now, t);
         }
         if (now.stale || !ahead) {
+            CU(cudaMemsetAsync(L.w.status, 0, sizeof(DevStatus), s));
             ST(md_build(c, sys, L, wc, p->skin, s));
             ++builds;
             ST(run_once(c, sys, rq, L, s));
@@ -902,7 +912,8 @@ panna_status panna_md_run(panna_ctx* c, const panna_system* sys, double* vel, co
     }
     if (n_steps > 0) CU(launch_md_b(N, sys->species, ms, vel, F, p->dt, s));
     if (n_builds) *n_builds = builds;
-    return collect(c, L, s, &need);
+    const panna_status st = md_status(c, L, s, &stale, &need);
+    return st != PANNA_OK && st == c->h_status->code ? step_error(*c->h_status, n_steps) : st;
 }
 
 panna_status panna_set_loss_options(panna_ctx* c, const panna_loss_options* o)
