@@ -153,7 +153,7 @@ __device__ __forceinline__ float pow_low(float zeta, int n, float t)
     return fmaf(p, zeta * rel, p);
 }
 
-// y^zeta = 2^(zeta log2 |y|) (FAST): y >= -eps/2, so its powers vanish to rounding below 0
+// y^zeta = 2^(zeta log2 |y|) (FAST): where no_clamp lets it stand for max(y, 0)^zeta
 __device__ __forceinline__ float2 pow2_y(float zeta, float2 y)
 {
     const float2 z = __fmul2_rn(make_float2(lg2f(fabsf(y.x)), lg2f(fabsf(y.y))), dup(zeta));
@@ -1264,10 +1264,13 @@ constexpr size_t kMaxSmem = 200 * 1024;
 
 }  // namespace
 
-// FAST needs exponents for which the splits' truncation (descriptor) and |y|^(zeta - 1) in place of
-// the clamp at y = 0 (adjoint) stay below the hardware log2's error
-static bool desc_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 16.f; }
-static bool adj_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 2.f; }
+// |y|^e in place of max(y, 0)^e: y is at least -(R - 1)/2, so below 0 this is at most ((R - 1)/2)^e, which
+// has to stay below the hardware log2's error of the powers near 1 (zeta = 2: up to eps = 1.9e-6, zeta = 4: 0.03)
+static bool no_clamp(const DescDev& d, float e) { return powf(d.r_half, e) <= 4.77e-7f; }
+// FAST needs exponents for which the splits' truncation (descriptor) and |y|^e in place of the clamp at
+// y = 0 (descriptor e = zeta, adjoint and tangent zeta - 1) stay below the hardware log2's error
+static bool desc_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 16.f && no_clamp(d, d.zeta); }
+static bool adj_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 2.f && no_clamp(d, d.zeta - 1.f); }
 
 static size_t desc_smem(const Work& w, const DescDev& d, bool fast)
 {
@@ -1368,7 +1371,7 @@ int small_rows_variant(const Work& w, const DescDev& d)
 // exponents as for the adjoint's fast form
 bool jvp_mma_fits(const Work& w, const DescDev& d)
 {
-    return d.ang_kind == 0 && d.zeta >= 2.f && kMW * jvp_mma_bytes(w.cap) <= kMaxSmem;
+    return d.ang_kind == 0 && adj_fast(d, true) && kMW * jvp_mma_bytes(w.cap) <= kMaxSmem;
 }
 
 cudaError_t launch_jvp_mma(const Work& w, const DescDev& d, const float* u, float* wdot_rows, cudaStream_t s)

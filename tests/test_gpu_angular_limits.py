@@ -1,7 +1,10 @@
 """The angular kernels at the ends of what the descriptor's parameters may be, through the default choice of
-kernels and against the oracle: shells without width (eta = 0).  Bounds as everywhere; the fast forms (angular
+kernels and against the oracle: shells without width (eta = 0), large eps_theta, where y_m passes below 0 and
+above 1 (below 0 for sectors outside [0, pi] only).  Bounds as everywhere; the fast forms (angular
 precision 2) carry about zeta 2^-22 per term, 1.2e-5 at zeta = 50, and a force sums terms up to 30 times its
 size: 5e-4 of RMS."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -20,7 +23,8 @@ def repeat(system, k):
 
 
 # (zeta, eta, eps, sectors, shells)
-LIMITS = [(4.0, 0.0, 1e-6, 8, 8), (50.0, 0.0, 1e-6, 16, 5)]
+LIMITS = [(4.0, 0.0, 1e-6, 8, 8), (50.0, 0.0, 1e-6, 16, 5), (2.0, 12.0, 0.5, 8, 8), (2.0, 12.0, 0.5, 9, 8),
+          (3.0, 12.0, 0.5, 8, 5)]
 
 
 @pytest.mark.parametrize("copies", [1, 51])       # below and above the limit of the teams of warps
@@ -33,6 +37,8 @@ def test_parameter_limits(limits, copies):
     one = H.triclinic_system()
     n = one.n_atoms
     desc = W.descriptor_params(2, 5.0, 8, n_theta, n_r, zeta=zeta, eta_ang=eta, eps_theta=eps)
+    if eps > 0.1 and (n_theta, n_r) != (8, 8):
+        desc = dataclasses.replace(desc, theta_s=np.linspace(-1.0, np.pi + 1.0, n_theta))
     archs = [W._mlp(desc.D, (32, 16)) for _ in range(2)]
     rng = np.random.default_rng(2)
     theta = W.init_weights(rng, desc, archs, 0.3, 0.1).astype(np.float32)
