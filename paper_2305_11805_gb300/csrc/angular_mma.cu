@@ -1271,6 +1271,14 @@ static bool no_clamp(const DescDev& d, float e) { return powf(d.r_half, e) <= 4.
 // y = 0 (descriptor e = zeta, adjoint and tangent zeta - 1) stay below the hardware log2's error
 static bool desc_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 16.f && no_clamp(d, d.zeta); }
 static bool adj_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 2.f && no_clamp(d, d.zeta - 1.f); }
+// Terms of the logarithm's series for (1 - t)^e, 0 for pow_low.  For t > 0 see the file comment; t is at least
+// -(R - 1)/2, where dropping the terms from t^(k+1) on moves the power by e |t|^(k+1)/(k+1) of itself: 8 terms
+// serve zeta = 50 up to eps = 0.4, at eps = 3 they were off by 1e-2
+static int log_terms(const DescDev& d, float e)
+{
+    auto holds = [&](int k) { return e * powf(d.r_half, (float)(k + 1)) / (float)(k + 1) <= 1e-8f; };
+    return e >= 32.f && holds(8) ? 8 : e >= 16.f && holds(13) ? 13 : 0;
+}
 
 static size_t desc_smem(const Work& w, const DescDev& d, bool fast)
 {
@@ -1319,19 +1327,20 @@ cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_
     if (!desc_mma_fits(w, d, fast)) return cudaErrorNotSupported;
     if (w.N == 0) return cudaSuccess;
     const bool two = ((d.n_theta + 7) / 8) % 2 == 0;
+    const int pw = log_terms(d, d.zeta);
     const Team tm = team_of(w, desc_fast(d, fast));
     if (tm.warps > 1) {
         const size_t smem = desc_mma_atom_bytes<false>(w.cap) + tm.warps * desc_mma_warp_bytes<false>(two ? 2 : 1);
         auto run = [&](auto kern) { return launch_team(kern, w.N, tm, smem, s, d, w, row_map, G_rows, Gh, Gl); };
-        if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8, true>) : run(k_desc_mma<false, 1, 8, true>);
-        if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13, true>) : run(k_desc_mma<false, 1, 13, true>);
+        if (pw == 8) return two ? run(k_desc_mma<false, 2, 8, true>) : run(k_desc_mma<false, 1, 8, true>);
+        if (pw == 13) return two ? run(k_desc_mma<false, 2, 13, true>) : run(k_desc_mma<false, 1, 13, true>);
         return two ? run(k_desc_mma<false, 2, 0, true>) : run(k_desc_mma<false, 1, 0, true>);
     }
     const size_t smem = desc_smem(w, d, fast);
     auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, row_map, G_rows, Gh, Gl); };
     if (desc_fast(d, fast)) return two ? run(k_desc_mma<true, 2, 0, false>) : run(k_desc_mma<true, 1, 0, false>);
-    if (d.zeta >= 32.f) return two ? run(k_desc_mma<false, 2, 8, false>) : run(k_desc_mma<false, 1, 8, false>);
-    if (d.zeta >= 16.f) return two ? run(k_desc_mma<false, 2, 13, false>) : run(k_desc_mma<false, 1, 13, false>);
+    if (pw == 8) return two ? run(k_desc_mma<false, 2, 8, false>) : run(k_desc_mma<false, 1, 8, false>);
+    if (pw == 13) return two ? run(k_desc_mma<false, 2, 13, false>) : run(k_desc_mma<false, 1, 13, false>);
     return two ? run(k_desc_mma<false, 2, 0, false>) : run(k_desc_mma<false, 1, 0, false>);
 }
 
@@ -1341,6 +1350,7 @@ cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows,
     if (!adj_mma_fits(w, d, fast)) return cudaErrorNotSupported;
     if (w.N == 0) return cudaSuccess;
     const bool two = d.n_theta > 8;
+    const int pw = log_terms(d, d.zeta - 1.f);
     int nc = adj_copies(w, d, fast);
     Team tm = team_of(w, adj_fast(d, fast));
     if (tm.warps > 1) {
@@ -1349,8 +1359,8 @@ cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows,
         while (tm.warps > 2 && bytes() > kMaxSmem) tm.warps /= 2;
         const size_t smem = bytes();
         auto run = [&](auto kern) { return launch_team(kern, w.N, tm, smem, s, d, w, g_rows, F, vir_atom, nc); };
-        if (d.zeta >= 33.f) return two ? run(k_adj_mma<false, 2, 8, true>) : run(k_adj_mma<false, 1, 8, true>);
-        if (d.zeta >= 17.f) return two ? run(k_adj_mma<false, 2, 13, true>) : run(k_adj_mma<false, 1, 13, true>);
+        if (pw == 8) return two ? run(k_adj_mma<false, 2, 8, true>) : run(k_adj_mma<false, 1, 8, true>);
+        if (pw == 13) return two ? run(k_adj_mma<false, 2, 13, true>) : run(k_adj_mma<false, 1, 13, true>);
         return two ? run(k_adj_mma<false, 2, 0, true>) : run(k_adj_mma<false, 1, 0, true>);
     }
     const size_t smem = (size_t)adj_mma_smem(d, w.cap, nc, adj_fast(d, fast)).total(1) * kMW;
@@ -1358,8 +1368,8 @@ cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows,
         return launch_resident(kern, w.N, smem, s, d, w, g_rows, F, vir_atom, nc);
     };
     if (adj_fast(d, fast)) return two ? run(k_adj_mma<true, 2, 0, false>) : run(k_adj_mma<true, 1, 0, false>);
-    if (d.zeta >= 33.f) return two ? run(k_adj_mma<false, 2, 8, false>) : run(k_adj_mma<false, 1, 8, false>);
-    if (d.zeta >= 17.f) return two ? run(k_adj_mma<false, 2, 13, false>) : run(k_adj_mma<false, 1, 13, false>);
+    if (pw == 8) return two ? run(k_adj_mma<false, 2, 8, false>) : run(k_adj_mma<false, 1, 8, false>);
+    if (pw == 13) return two ? run(k_adj_mma<false, 2, 13, false>) : run(k_adj_mma<false, 1, 13, false>);
     return two ? run(k_adj_mma<false, 2, 0, false>) : run(k_adj_mma<false, 1, 0, false>);
 }
 

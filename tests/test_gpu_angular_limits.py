@@ -58,3 +58,18 @@ def test_parameter_limits(limits, copies):
         print("mode %d: F %.3g (rms %.3g), gradient %.3g" % (mode, ferr, rms, gerr))
         assert ferr <= tol_f
         assert gerr <= H.TOL_DTHETA
+
+
+@pytest.mark.parametrize("zeta", [20.0, 50.0])
+def test_rows_with_large_eps(zeta):
+    """eps = 3: y_m from -1/2 to 3/2."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    system = H.triclinic_system()
+    desc = W.descriptor_params(2, 5.0, 8, 8, 8, zeta=zeta, eps_theta=3.0)
+    archs = [W._mlp(desc.D, (16,)) for _ in range(2)]
+    G0 = O.batch(system, desc, archs, np.zeros(2 * archs[0].n_params), want_G=True)["G"]
+    pot = P.Potential(desc, archs)
+    err = H.descriptor_error(pot.descriptors(P.DeviceSystem(system)).cpu().numpy().astype(np.float64), G0, desc)
+    assert err <= H.TOL_G
