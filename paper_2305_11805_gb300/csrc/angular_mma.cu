@@ -44,7 +44,7 @@
 // small t, and dropping the terms from t^(d+1) on moves y^zeta by at most
 // zeta t^(d+1)/(d+1) (1-t)^zeta <= 1.5e-9 (d = 8, zeta >= 32), 1.1e-9 (d = 13, zeta >= 16) of its
 // maximum; all terms have one sign, so for t near 1 the sum still underflows as y^zeta does.  Below
-// zeta = 16 the power comes from the float pair 1 - t.
+// zeta = 16, and where eps makes the series too short, the power comes from the float pair 1 - t.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -136,21 +136,15 @@ __device__ __forceinline__ float2 log_series(const float* zl, float2 t)
     return __fmul2_rn(p, t);
 }
 
-// (1 - t)^zeta below zeta = 16, from the float pair yh + yl = 1 - t: repeated squaring for whole
-// exponents (n > 0), the hardware log2 otherwise
-__device__ __forceinline__ float pow_low(float zeta, int n, float t)
+// (1 - t)^zeta below zeta = 16, from the float pair yh + yl = 1 - t.  The library's logarithm: the hardware's,
+// off by up to 2^-22, made rows of zeta = 15.5 2.4 times as far off as the blocked kernel's, and repeated
+// squaring for whole exponents took 1 to 10 us more of 155 (4,096 atoms, 47 neighbours)
+__device__ __forceinline__ float pow_low(float zeta, float t)
 {
     const float yh = 1.f - t;
     const float yl = (1.f - yh) - t;
     if (!(yh > 0.f)) return 0.f;
-    const float rel = yl * rcpf(yh);
-    if (n <= 0) return ex2f(zeta * fmaf(rel, 1.4426950408889634f, lg2f(yh)));
-    float p = 1.f, b = yh;
-    for (int k = n; k; k >>= 1) {
-        if (k & 1) p *= b;
-        b *= b;
-    }
-    return fmaf(p, zeta * rel, p);
+    return exp2f(zeta * fmaf(yl * rcpf(yh), 1.4426950408889634f, log2f(yh)));
 }
 
 // y^zeta = 2^(zeta log2 |y|) (FAST): where no_clamp lets it stand for max(y, 0)^zeta
@@ -162,9 +156,9 @@ __device__ __forceinline__ float2 pow2_y(float zeta, float2 y)
 
 // (1 - t)^zeta, zeta the exponent of the coefficients zl
 template <int PW>
-__device__ __forceinline__ float2 pow2_t(const float* zl, float zeta, int zeta_int, float2 t)
+__device__ __forceinline__ float2 pow2_t(const float* zl, float zeta, float2 t)
 {
-    if (PW == 0) return make_float2(pow_low(zeta, zeta_int, t.x), pow_low(zeta, zeta_int, t.y));
+    if (PW == 0) return make_float2(pow_low(zeta, t.x), pow_low(zeta, t.y));
     const float2 z = log_series<PW ? PW : 1>(zl, t);
     return make_float2(ex2f(z.x), ex2f(z.y));
 }
@@ -541,14 +535,18 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
                                     const float2 cc = __ffma2_rn(ch, chm[mc], __fmul2_rn(sh, shm[mc]));
                                     const float2 dt = __fadd2_rn(make_float2(hd.x, hd.y), tan_m[mc]);
                                     ee = __fadd2_rn(ee, __ffma2_rn(dt, cc, dw));
-                                    const float2 A = pow2_t<PW>(d.zlog, d.zeta, d.zeta_int, __ffma2_rn(ee, ee, nk0));
+                                    const float2 A = pow2_t<PW>(d.zlog, d.zeta, __ffma2_rn(ee, ee, nk0));
                                     float2 Ah, Al;
                                     tf_split<true>(A, Ah, Al);
-                                    // the tensor cores truncate their sums: two groups deep here
-                                    if (k & 1) mma8(q2[mc], Ah.x, Al.x, Ah.y, Al.y, el.x, el.y);
+                                    // the tensor cores truncate their sums: two groups deep here, one where
+                                    // a small exponent makes the terms of a block alike in size, so that what
+                                    // is lost does not average out (zeta <= 8: 1.03 to 1.06 times the blocked
+                                    // kernel's error with two, 0.93 to 1.01 with one, the same time)
+                                    constexpr int deep = PW ? 2 : 1;
+                                    if (k % deep) mma8(q2[mc], Ah.x, Al.x, Ah.y, Al.y, el.x, el.y);
                                     else mma8z(q2[mc], Ah.x, Al.x, Ah.y, Al.y, el.x, el.y);
                                     mma8(q2[mc], Ah.x, Al.x, Ah.y, Al.y, eh.x, eh.y);
-                                    if ((k & 1) || 8 * (k + 1) >= left) {
+                                    if (k % deep == deep - 1 || 8 * (k + 1) >= left) {
 #pragma unroll
                                         for (int j = 0; j < 4; ++j) c[mc][j] += q2[mc][j];
                                     }
@@ -1095,7 +1093,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
                                     const float2 tt = __ffma2_rn(ee, ee, dup(-d.r_half));
                                     y = __fadd2_rn(dup(1.f), make_float2(-tt.x, -tt.y));
                                     ef = __fmul2_rn(ee, __ffma2_rn(ch2, chm[mc], __fmul2_rn(sh2, shm[mc])));
-                                    p1 = pow2_t<PW>(d.zlog1, d.zeta - 1.f, d.zeta_int - 1, tt);
+                                    p1 = pow2_t<PW>(d.zlog1, d.zeta - 1.f, tt);
                                 }
                                 const float2 U = __fmul2_rn(p1, y), Q = __fmul2_rn(p1, ef);
                                 const float2 Cp = P ? make_float2(C[2], C[3]) : make_float2(C[0], C[1]);
@@ -1375,7 +1373,7 @@ cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows,
 
 int small_rows_variant(const Work& w, const DescDev& d)
 {
-    return w.N < kSplitAtoms && d.zeta >= 16.f && desc_mma_fits(w, d, false) ? 5 : 0;
+    return w.N < kSplitAtoms && desc_mma_fits(w, d, false) ? 5 : 0;
 }
 
 // exponents as for the adjoint's fast form

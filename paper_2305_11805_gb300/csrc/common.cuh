@@ -195,9 +195,9 @@ cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_
 cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows, float* F, float* vir_atom,
                            bool fast, cudaStream_t s);
 // The kernel of FP32 descriptor rows that are asked for by themselves, in small batches (below kSplitAtoms
-// atoms; larger ones take the compensated kernel): the matrix form with several warps per atom, from zeta =
-// 16 on, with 0.85 to 1.0 times the blocked kernel's error (16 carbon atoms 35 -> 16 us, 850 atoms in 50
-// molecules 43 -> 23, 1,000 of water 184 -> 109); below, its powers are 1.25 times as far off.
+// atoms; larger ones take the compensated kernel): the matrix form with several warps per atom, with 0.85 to
+// 1.01 times the blocked kernel's error at every exponent (16 carbon atoms 35 -> 16 us, 850 atoms in 50
+// molecules 43 -> 23, 1,000 of water 184 -> 109).
 int small_rows_variant(const Work& w, const DescDev& d);
 bool jvp_mma_fits(const Work& w, const DescDev& d);
 cudaError_t launch_jvp_mma(const Work& w, const DescDev& d, const float* u, float* wdot_rows, cudaStream_t s);
