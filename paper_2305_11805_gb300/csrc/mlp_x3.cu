@@ -92,10 +92,10 @@ __device__ __forceinline__ void split(float x, float& hi, float& lo)
     lo = low_clear(x - hi);
 }
 
-// the same where rounding would overflow, for infinities and NaN
+// the same where rounding would overflow, for infinities and NaN (x + x: a NaN that TF32 keeps as one)
 __device__ __noinline__ float2 split_special(float x)
 {
-    if (!(fabsf(x) < __int_as_float(0x7f800000))) return make_float2(x, 0.f);
+    if (!(fabsf(x) < __int_as_float(0x7f800000))) return make_float2(x + x, 0.f);
     const float h = low_clear(x);
     return make_float2(h, low_clear(x - h));
 }
@@ -429,13 +429,26 @@ k_gemm_x3(LayerArgs la, const float* __restrict__ theta, const int32_t* __restri
         const int q = warp & 3, c0 = (warp >> 2) * 64;
         const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
         float acc[64];
-        auto add = [&](uint32_t col, float lost) {
+        auto add = [&](uint32_t col) {
 #pragma unroll
             for (int x = 0; x < 2; ++x) {
                 float v[32];
                 tc_ld32(lanes + col + 32 * x, v);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) acc[32 * x + j] += fmaf(lost, acc[32 * x + j], v[j]);
+                for (int j = 0; j < 32; ++j) acc[32 * x + j] += v[j];
+            }
+        };
+        // an infinite operand leaves its products in the sum of hi hi, and 0 times infinity in the cross terms
+        auto add_cross = [&](uint32_t col, float lost) {
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                float v[32];
+                tc_ld32(lanes + col + 32 * x, v);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float a = acc[32 * x + j];
+                    if (fabsf(a) < __int_as_float(0x7f800000)) acc[32 * x + j] = a + fmaf(lost, a, v[j]);
+                }
             }
         };
         const float* bias = WG ? nullptr : theta + la.b_off[s];
@@ -509,8 +522,8 @@ k_gemm_x3(LayerArgs la, const float* __restrict__ theta, const int32_t* __restri
                 }
                 const bool used = c0 < tile_bn(dt);
                 // the last step may be too short for its second part
-                if (used && (SUB == 1 || dc * KS * 8 < K)) add((uint32_t)b * 128, 0.f);
-                if (dc == nk * SUB - 1 && used) add(kXAcc * 128, kXLost / SUB);
+                if (used && (SUB == 1 || dc * KS * 8 < K)) add((uint32_t)b * 128);
+                if (dc == nk * SUB - 1 && used) add_cross(kXAcc * 128, kXLost / SUB);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acce + b);
