@@ -136,30 +136,35 @@ __device__ __forceinline__ float2 log_series(const float* zl, float2 t)
     return __fmul2_rn(p, t);
 }
 
-// (1 - t)^zeta below zeta = 16, from the float pair yh + yl = 1 - t.  The library's logarithm: the hardware's,
-// off by up to 2^-22, made rows of zeta = 15.5 2.4 times as far off as the blocked kernel's, and repeated
-// squaring for whole exponents took 1 to 10 us more of 155 (4,096 atoms, 47 neighbours)
-__device__ __forceinline__ float pow_low(float zeta, float t)
+// (1 - t)^e below e = 16, from the float pair yh + yl = 1 - t.  LIB: the library's logarithm; the hardware's,
+// off by up to 2^-22, made descriptor rows of zeta = 15.5 2.4 times as far off as the blocked kernel's, and
+// repeated squaring for whole exponents took 1 to 10 us more of 155 (4,096 atoms, 47 neighbours).  The adjoint's
+// forces are bound by the angle in single floats, as those of its other kernels, which take the hardware's too
+// (0.95 to 1.03 times the diagonal-order kernel's error with either; 191 us with the library's or with a loop of
+// squarings, 125 so).
+template <bool LIB>
+__device__ __forceinline__ float pow_low(float e, float t)
 {
     const float yh = 1.f - t;
     const float yl = (1.f - yh) - t;
     if (!(yh > 0.f)) return 0.f;
-    return exp2f(zeta * fmaf(yl * rcpf(yh), 1.4426950408889634f, log2f(yh)));
+    const float z = e * fmaf(yl * rcpf(yh), 1.4426950408889634f, LIB ? log2f(yh) : lg2f(yh));
+    return LIB ? exp2f(z) : ex2f(z);
+}
+
+// (1 - t)^zeta, zeta the exponent of the coefficients zl
+template <int PW, bool LIB>
+__device__ __forceinline__ float2 pow2_t(const float* zl, float zeta, float2 t)
+{
+    if (PW == 0) return make_float2(pow_low<LIB>(zeta, t.x), pow_low<LIB>(zeta, t.y));
+    const float2 z = log_series<PW ? PW : 1>(zl, t);
+    return make_float2(ex2f(z.x), ex2f(z.y));
 }
 
 // y^zeta = 2^(zeta log2 |y|) (FAST): where no_clamp lets it stand for max(y, 0)^zeta
 __device__ __forceinline__ float2 pow2_y(float zeta, float2 y)
 {
     const float2 z = __fmul2_rn(make_float2(lg2f(fabsf(y.x)), lg2f(fabsf(y.y))), dup(zeta));
-    return make_float2(ex2f(z.x), ex2f(z.y));
-}
-
-// (1 - t)^zeta, zeta the exponent of the coefficients zl
-template <int PW>
-__device__ __forceinline__ float2 pow2_t(const float* zl, float zeta, float2 t)
-{
-    if (PW == 0) return make_float2(pow_low(zeta, t.x), pow_low(zeta, t.y));
-    const float2 z = log_series<PW ? PW : 1>(zl, t);
     return make_float2(ex2f(z.x), ex2f(z.y));
 }
 
@@ -535,7 +540,7 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
                                     const float2 cc = __ffma2_rn(ch, chm[mc], __fmul2_rn(sh, shm[mc]));
                                     const float2 dt = __fadd2_rn(make_float2(hd.x, hd.y), tan_m[mc]);
                                     ee = __fadd2_rn(ee, __ffma2_rn(dt, cc, dw));
-                                    const float2 A = pow2_t<PW>(d.zlog, d.zeta, __ffma2_rn(ee, ee, nk0));
+                                    const float2 A = pow2_t<PW, true>(d.zlog, d.zeta, __ffma2_rn(ee, ee, nk0));
                                     float2 Ah, Al;
                                     tf_split<true>(A, Ah, Al);
                                     // the tensor cores truncate their sums: two groups deep here, one where
@@ -1093,7 +1098,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
                                     const float2 tt = __ffma2_rn(ee, ee, dup(-d.r_half));
                                     y = __fadd2_rn(dup(1.f), make_float2(-tt.x, -tt.y));
                                     ef = __fmul2_rn(ee, __ffma2_rn(ch2, chm[mc], __fmul2_rn(sh2, shm[mc])));
-                                    p1 = pow2_t<PW>(d.zlog1, d.zeta - 1.f, tt);
+                                    p1 = pow2_t<PW, false>(d.zlog1, d.zeta - 1.f, tt);
                                 }
                                 const float2 U = __fmul2_rn(p1, y), Q = __fmul2_rn(p1, ef);
                                 const float2 Cp = P ? make_float2(C[2], C[3]) : make_float2(C[0], C[1]);
