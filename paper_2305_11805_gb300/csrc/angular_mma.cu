@@ -1274,6 +1274,7 @@ static bool no_clamp(const DescDev& d, float e) { return powf(d.r_half, e) <= 4.
 // y = 0 (descriptor e = zeta, adjoint and tangent zeta - 1) stay below the hardware log2's error
 static bool desc_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 16.f && no_clamp(d, d.zeta); }
 static bool adj_fast(const DescDev& d, bool fast) { return fast && d.zeta >= 2.f && no_clamp(d, d.zeta - 1.f); }
+bool mma_fast(const DescDev& d, bool adjoint) { return adjoint ? adj_fast(d, true) : desc_fast(d, true); }
 // Terms of the logarithm's series for (1 - t)^e, 0 for pow_low.  For t > 0 see the file comment; t is at least
 // -(R - 1)/2, where dropping the terms from t^(k+1) on moves the power by e |t|^(k+1)/(k+1) of itself: 8 terms
 // serve zeta = 50 up to eps = 0.4, at eps = 3 they were off by 1e-2

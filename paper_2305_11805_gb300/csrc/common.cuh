@@ -190,6 +190,8 @@ cudaError_t launch_descriptor_bf16(const Work& w, const DescDev& d, __nv_bfloat1
 // fast: the forms of the BF16 networks; otherwise those of the FP32 ones.
 bool desc_mma_fits(const Work& w, const DescDev& d, bool fast);
 bool adj_mma_fits(const Work& w, const DescDev& d, bool fast);
+// whether `fast` gets the fast arithmetic for this descriptor (else the FP32 networks' form)
+bool mma_fast(const DescDev& d, bool adjoint);
 cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_map, float* G_rows,
                             __nv_bfloat16* Gh, __nv_bfloat16* Gl, bool fast, cudaStream_t s);
 cudaError_t launch_adj_mma(const Work& w, const DescDev& d, const float* g_rows, float* F, float* vir_atom,
