@@ -388,6 +388,7 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
 // with several warps per atom (descriptor + adjoint: 16 carbon atoms 93 -> 28 us, 64 diamond atoms 42 ->
 // 20 us, 850 atoms in 50 molecules 60 -> 38 us); with BF16 networks, whose rows are those of large
 // batches, the old kernels spread an atom over several warps and are tuned against them.
+constexpr int kMmaSpecies = 4;
 int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
 {
     if (c->d.ang_kind != 0) return 0;   // the standard BP term has one kernel
@@ -398,7 +399,11 @@ int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
     // 4,096 atoms, zeta = 6: 47 neighbours 65 against 156 us, 87 neighbours 166 against 420).
     if (!acc && !mma_fast(c->d, kind == KV_ADJ)) return -1;
     if (kind == KV_DESC && desc_mma_fits(w, c->d, !acc)) return 5;
-    if (kind == KV_ADJ && adj_mma_fits(w, c->d, !acc)) return 6;
+    // A species block takes whole rounds of 32 pairs: with many species and few neighbours most of a round is
+    // empty.  Adjoint, 4,096 atoms, FP32, against variant 5 (us): four species, 18 neighbours 45 and 49; six
+    // 119 and 55, with 87 neighbours 414 and 457; eight, 18 neighbours 257 and 72.  From five species on the
+    // two are measured (the descriptor's form stays the fastest: eight species, 18 neighbours 63 against 206).
+    if (kind == KV_ADJ && c->d.S <= kMmaSpecies && adj_mma_fits(w, c->d, !acc)) return 6;
     return -1;
 }
 
@@ -430,18 +435,20 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
             t = &q;
     }
     if (t && t->variant[kind] >= 0) return t->variant[kind];
-    const int fallback = (sys->n_atoms < kSplitAtoms || ext) ? 0 : (kind == KV_ADJ ? 5 : 2);
-    if (!c->autotune || c->async || sys->n_atoms == 0) return fallback;
-    float ms[kNumVariants] = {};
     const bool mma = kind == KV_DESC ? desc_mma_fits(w, c->d, !acc)
                      : kind == KV_ADJ ? adj_mma_fits(w, c->d, !acc) : !acc && jvp_mma_fits(w, c->d);
+    // the adjoint's matrix form where mma_variant leaves it open: one of the two was the fastest everywhere
+    const bool two = kind == KV_ADJ && mma && (acc || w.N >= kSplitAtoms) && mma_fast(c->d, true);
+    const int fallback = sys->n_atoms < kSplitAtoms ? (two ? 6 : 0) : ext ? 0 : kind == KV_ADJ ? 5 : 2;
+    if (!c->autotune || c->async || sys->n_atoms == 0) return fallback;
+    float ms[kNumVariants] = {};
     auto candidate = [&](int v) {
         if (v == kMmaVariant[kind]) return mma;
-        return !ext || v < 2;
+        return two ? v == 5 : !ext || v < 2;
     };
     for (int v = 0; v < kKindVariants[kind]; ++v)
         if (candidate(v)) launch(v);   // first launches load and configure the kernels
-    int best = 0;
+    int best = -1;
     // three back-to-back launches per variant: the host's launch work then overlaps the kernels
     // instead of showing up as idle device time in a single short measurement
     for (int v = 0; v < kKindVariants[kind]; ++v) {
@@ -451,7 +458,7 @@ int tuned_variant_(panna_ctx* c, const panna_system* sys, const Work& w, int pre
         cudaEventRecord(c->tev[1], s);
         cudaEventSynchronize(c->tev[1]);
         cudaEventElapsedTime(&ms[v], c->tev[0], c->tev[1]);
-        if (ms[v] < ms[best]) best = v;
+        if (best < 0 || ms[v] < ms[best]) best = v;
     }
     if (!t) {
         t = &c->tuned[c->n_tuned < 16 ? c->n_tuned++ : 15];

@@ -32,3 +32,33 @@ def test_bf16_networks_below_the_fast_powers(zeta, matrix):
     assert (choice == 5) == matrix, choice
     err, _ = H.force_error(F[:one.n_atoms].cpu().numpy().astype(np.float64), ref["F"])
     assert err <= H.TOL_F_BF16
+
+
+def clusters_of(n_species, copies, seed=7):
+    """Boxes of 216 atoms on a jittered grid, about 18 neighbours within 3.2 A: with eight species 36 species
+    blocks of four or five pairs each."""
+    rng = np.random.default_rng(seed)
+    g = np.stack(np.meshgrid(*[np.arange(6)] * 3, indexing="ij"), -1).reshape(-1, 3) * 2.0
+    pos = g + rng.uniform(-0.35, 0.35, g.shape)
+    one = W.System(np.array([0, 216], np.int64), pos, rng.integers(0, n_species, 216).astype(np.int32),
+                   (np.eye(3) * 12.0).reshape(1, 9), np.ones((1, 3), np.uint8), n_species)
+    return one, repeat(one, copies)
+
+
+@pytest.mark.parametrize("copies", [1, 19])        # 216 and 4,104 atoms
+@pytest.mark.parametrize("autotune", [1, 0])
+@pytest.mark.parametrize("n_species", [5, 8])
+def test_adjoint_of_many_species(n_species, autotune, copies):
+    one, system = clusters_of(n_species, copies)
+    desc = W.descriptor_params(n_species, 3.2, 8, 8, 8)
+    torch, archs, theta, th, pot, sysd = setup(system, desc)
+    P.panna_set_tuning(pot.ctx, "autotune", autotune)
+    ref = O.batch(one, desc, archs, theta.astype(np.float64))
+    for prec, tol in ((P.PANNA_MLP_FP32, H.TOL_F_FP32), (P.PANNA_MLP_BF16, H.TOL_F_BF16)):
+        F = pot.energy_forces(sysd, th, prec)[2]
+        choice = P.panna_tuning_choice(pot.ctx, "adjoint")
+        if n_species == 8 and copies == 19:
+            assert choice == 5, (prec, choice)      # 72 us against 257
+        err, _ = H.force_error(F[:216].cpu().numpy().astype(np.float64), ref["F"])
+        print("%d species, %d atoms, precision %d: variant %d, %.3g" % (n_species, 216 * copies, prec, choice, err))
+        assert err <= tol
