@@ -392,7 +392,16 @@ constexpr int kMmaSpecies = 4;
 int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
 {
     if (c->d.ang_kind != 0) return 0;   // the standard BP term has one kernel
-    if (kind == KV_JVP) return !acc && jvp_mma_fits(w, c->d) ? 5 : -1;
+    if (kind == KV_JVP) {
+        if (acc || !jvp_mma_fits(w, c->d)) return -1;
+        // One warp per atom: with less than an atom per warp scheduler an atom's chain of rounds is the time, and
+        // a round of variant 2 is the shorter one.  512 atoms of one species, variants 5 and 2 (us): 18 neighbours
+        // 12.3 and 12.3, 30: 18.4 and 16.4, 51: 37 and 31, 87: 84 and 68; 1,000 atoms, 87: 92 and 90; 4,096 atoms,
+        // 51: 84 and 103.  Four species: 18 neighbours 14 and 21, 87: 88 and 74.  The neighbours are not known
+        // here; a capacity past the initial one tells of more than 64.
+        if (w.N < kSplitAtoms / 2 && w.cap > 64) return 2;
+        return 5;
+    }
     if (w.N < kSplitAtoms && !acc) return -1;
     // The fast arithmetic takes zeta >= 16 (descriptor) and 2 (adjoint): below, BF16 networks' kernels are
     // measured, since the float-pair form is slower than the compensated kernels' own fast one (descriptor,

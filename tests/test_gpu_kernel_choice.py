@@ -62,3 +62,18 @@ def test_adjoint_of_many_species(n_species, autotune, copies):
         err, _ = H.force_error(F[:216].cpu().numpy().astype(np.float64), ref["F"])
         print("%d species, %d atoms, precision %d: variant %d, %.3g" % (n_species, 216 * copies, prec, choice, err))
         assert err <= tol
+
+
+@pytest.mark.parametrize("rc,copies,variant", [(3.2, 1, 5), (5.6, 1, 2), (5.6, 3, 5)])
+def test_tangent_of_small_dense_batches(rc, copies, variant):
+    """216 atoms with 18 and 87 neighbours, and 648 with 87."""
+    one, system = clusters_of(2, copies)
+    desc = W.descriptor_params(2, rc, 8, 8, 8)
+    torch, archs, theta, th, pot, sysd = setup(system, desc)
+    f_ref = np.random.default_rng(3).normal(size=(216, 3)).astype(np.float32)
+    ref = O.batch(one, desc, archs, theta.astype(np.float64), e_ref=np.zeros(1), f_ref=f_ref.astype(np.float64),
+                  w_force=1.0, param_grad=True)
+    g = pot.loss_grad(sysd, th, torch.zeros(copies, dtype=torch.float64, device="cuda"),
+                      torch.as_tensor(np.tile(f_ref, (copies, 1)), device="cuda"), 1.0)[1]
+    assert P.panna_tuning_choice(pot.ctx, "jvp") == variant
+    assert max(H.layer_errors(archs, g.cpu().numpy().astype(np.float64), ref["dtheta"])) <= H.TOL_DTHETA
