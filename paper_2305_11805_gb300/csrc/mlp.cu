@@ -435,7 +435,7 @@ constexpr int kX3MinK = 128;
 template <bool B_TRANS, int PRO, int EPI>
 static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStream_t s, const LayerArgs& la,
                                const float* theta, const MlpBuffers& b, const float* A, int lda, const float* Zp,
-                               int ldp, float* C, int ldc, float* C2, const float* Ze, int lde)
+                               int ldp, float* C, int ldc, float* C2, const float* Ze, int lde, int* launches)
 {
     const int32_t *seg_off = b.seg_off, *tile_start = b.tile_start;
     dim3 g = gemm_grid(p, N, n_max);
@@ -448,7 +448,9 @@ static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStrea
             cudaError_t e = launch_gemm_x3<B_TRANS, PRO, EPI>(g, s, la, theta, seg_off, tile_start, Zp, lda, nullptr, 0, C2,
                                                               ldc, nullptr, nullptr, 0, b.status);
             if (e != cudaSuccess) return e;
+            ++*launches;
         }
+        ++*launches;
         return launch_gemm_x3<B_TRANS, PRO, EPI>(g, s, la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc, C2, Ze,
                                                  lde, b.status);
     }
@@ -463,6 +465,7 @@ static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStrea
         k_gemm<B_TRANS, PRO, EPI, 128><<<g, 256, 0, s>>>(la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc,
                                                          C2, Ze, lde);
     }
+    ++*launches;
     return cudaGetLastError();
 }
 
@@ -481,9 +484,9 @@ cudaError_t mlp_forward(const MlpPlan& p, const MlpBuffers& b, const float* thet
         const float* Ain = l == 0 ? b.G : b.A[l];
         const int lda = p.ld[l];
         cudaError_t e = launch_gemm<true, PRO_NONE, EPI_FWD>(p, N, p.ld[l + 1], s, la, theta, b, Ain, lda,
-                                             nullptr, 0, b.Z[l + 1], p.ld[l + 1], b.A[l + 1], nullptr, 0);
+                                             nullptr, 0, b.Z[l + 1], p.ld[l + 1], b.A[l + 1], nullptr, 0,
+                                             launches);
         if (e != cudaSuccess) return e;
-        ++*launches;
     }
     return cudaGetLastError();
 }
@@ -504,9 +507,9 @@ cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         float* out = l == 0 ? g : nxt;
         const int ldo = p.ld[l];
         cudaError_t e = launch_gemm<false, PRO_DACT, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, cur,
-                                                p.ld[l + 1], b.Z[l + 1], p.ld[l + 1], out, ldo, nullptr, nullptr, 0);
+                                                p.ld[l + 1], b.Z[l + 1], p.ld[l + 1], out, ldo, nullptr, nullptr, 0,
+                                                launches);
         if (e != cudaSuccess) return e;
-        ++*launches;
         float* t = cur; cur = out; nxt = t;
     }
     if (ab1) *ab1 = cur;
@@ -523,9 +526,8 @@ cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         const float* Ain = l == 0 ? wdot : b.Ad[l];
         cudaError_t e = launch_gemm<true, PRO_NONE, EPI_TAN>(p, N, p.ld[l + 1], s, la, theta, b, Ain,
                                              p.ld[l], nullptr, 0, b.Zd[l + 1], p.ld[l + 1], b.Ad[l + 1], b.Z[l + 1],
-                                             p.ld[l + 1]);
+                                             p.ld[l + 1], launches);
         if (e != cudaSuccess) return e;
-        ++*launches;
     }
     if (part == MLP_GRAD_TANGENT) return cudaGetLastError();
     // reverse pass: seeds abar_L = alpha, adotbar_L = -1 (unless given)
@@ -556,9 +558,8 @@ cudaError_t mlp_param_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
             // abar_{l} = Zb W_{l+1}, adotbar_{l} = Zdb W_{l+1}
             LayerArgs la = layer_args(p, l, true);
             cudaError_t e = launch_gemm<false, PRO_NONE, EPI_STORE>(p, N, p.ld[l], s, la, theta, b, b.Zb, ldl, b.Zdb, ldl,
-                                                                    b.Ab, p.ld[l], b.Adb, nullptr, 0);
+                                                                    b.Ab, p.ld[l], b.Adb, nullptr, 0, launches);
             if (e != cudaSuccess) return e;
-            ++*launches;
         }
     }
     if (!wgrad_part) {
