@@ -1219,13 +1219,6 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
     if (TEAM) sync();   // the other CTAs' shared memory is read until here
 }
 
-int sm_count()
-{
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 152;
-    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 152;
-}
-
 // resident CTAs walking the atoms: as many as fit on the GPU at once, no more than the atoms need
 template <class Kern, class... Args>
 cudaError_t launch_resident(Kern kern, int64_t N, size_t smem, cudaStream_t s, Args... args)

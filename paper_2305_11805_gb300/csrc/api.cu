@@ -1142,7 +1142,7 @@ panna_status panna_qeq_energy_forces(panna_ctx* c, const panna_system* sys, cons
         CU(launch_qeq(c->qeq, L.w, L.mb.A[c->plan.L], ldL, total_charge, L.E_rows, charges, F, L.mb.Ab, ldL, s,
                       &nl));
         stage_mark(c, 3, s);
-        CU(mlp_input_grad(c->plan, L.mb, theta, N, L.g, s, &nl, nullptr, true));
+        CU(mlp_input_grad(c->plan, L.mb, theta, N, L.g, s, &nl, true));
         const int va = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_ADJ, s, [&](int vv) {
             launch_adjoint(L.w, c->d, L.g, L.F_tune, nullptr, acc, vv, s, &dummy);
         }, acc);
@@ -1214,7 +1214,7 @@ panna_status panna_qeq_loss_grad(panna_ctx* c, const panna_system* sys, const fl
         CU(launch_qeq(c->qeq, L.w, L.mb.A[c->plan.L], ldL, total_charge, L.E_rows, L.qbuf, Fo, L.mb.Ab, ldL, s,
                       &nl));
         stage_mark(c, 3, s);
-        CU(mlp_input_grad(c->plan, L.mb, theta, N, L.g, s, &nl, nullptr, true));
+        CU(mlp_input_grad(c->plan, L.mb, theta, N, L.g, s, &nl, true));
         const int va = tuned_variant(c, sys, L.w, PANNA_MLP_FP32, KV_ADJ, s, [&](int vv) {
             launch_adjoint(L.w, c->d, L.g, L.F_tune, nullptr, acc, vv, s, &dummy);
         }, acc);

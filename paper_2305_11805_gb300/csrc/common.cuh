@@ -44,6 +44,14 @@ cudaError_t allow_smem(void (*kern)(Args...), size_t bytes)
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, all - (int)at.sharedSizeBytes);
 }
 
+// SMs of the current device
+inline int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0 ? n : 152;
+}
+
 // Descriptor parameters as the kernels read them (FP32 copies plus FP64 cutoff).  The
 // struct is passed by value, so the grids sit in the kernel-parameter constant bank.
 constexpr int kMaxRad = 256;

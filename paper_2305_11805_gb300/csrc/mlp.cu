@@ -409,20 +409,6 @@ static dim3 gemm_grid(const MlpPlan& p, int64_t N, int n_max)
     return dim3((unsigned)((N + kGM - 1) / kGM + p.S), (unsigned)((n_max + kGN - 1) / kGN), 1);
 }
 
-static int device_sms()
-{
-    static int n_sm = 0;
-    if (n_sm == 0) {
-        int dev = 0, v = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0)
-            n_sm = v;
-        else
-            return 1;
-    }
-    return n_sm;
-}
-
 // One layer's product.  From 128 summands on the tensor cores' form (k_gemm_x3) is the faster and the more
 // accurate one (17,396 rows, K = 128, N = 32: 24 -> 16 us, error 2.0e-7 -> 1.1e-7; 300 rows: both 14.6 us);
 // with fewer, the split of its operands costs as much accuracy as the short sums do here (K = 65, input
@@ -443,7 +429,7 @@ static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStrea
     for (int q = 1; q < la.S; ++q) kmin = std::min(kmin, la.K[q]);
     if (p.x3 && kmin >= kX3MinK) {
         // a CTA takes a row tile's column tiles in turn once the row tiles fill the SMs
-        g.y = std::min<unsigned>(g.y, std::max(1u, (unsigned)device_sms() / g.x));
+        g.y = std::min<unsigned>(g.y, std::max(1u, (unsigned)sm_count() / g.x));
         if (PRO == PRO_NONE && EPI == EPI_STORE) {
             cudaError_t e = launch_gemm_x3<B_TRANS, PRO, EPI>(g, s, la, theta, seg_off, tile_start, Zp, lda, nullptr, 0, C2,
                                                               ldc, nullptr, nullptr, 0, b.status);
@@ -457,7 +443,7 @@ static cudaError_t launch_gemm(const MlpPlan& p, int64_t N, int n_max, cudaStrea
     int kmax = 0;
     for (int q = 0; q < la.S; ++q) kmax = std::max(kmax, la.K[q]);
     if (PRO == PRO_NONE && EPI == EPI_STORE) g.z = 2;   // only used for pairs of products
-    if ((int64_t)g.x * g.y * g.z < 2 * (int64_t)device_sms() && kmax <= 256) {
+    if ((int64_t)g.x * g.y * g.z < 2 * (int64_t)sm_count() && kmax <= 256) {
         g.x *= 2;
         k_gemm<B_TRANS, PRO, EPI, 64><<<g, 256, 0, s>>>(la, theta, seg_off, tile_start, A, lda, Zp, ldp, C, ldc,
                                                         C2, Ze, lde);
@@ -492,7 +478,7 @@ cudaError_t mlp_forward(const MlpPlan& p, const MlpBuffers& b, const float* thet
 }
 
 cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, float* g,
-                           cudaStream_t s, int* launches, float** ab1, bool seeded)
+                           cudaStream_t s, int* launches, bool seeded)
 {
     // seed dE/da_L = 1 (unless given), then a_{l-1}bar = (a_l bar * act'(z_l)) W_l
     if (!seeded) {
@@ -501,8 +487,7 @@ cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
     }
     float* cur = b.Ab;
     float* nxt = b.Ab2;
-    const int lstop = ab1 ? 1 : 0;
-    for (int l = p.L - 1; l >= lstop; --l) {
+    for (int l = p.L - 1; l >= 0; --l) {
         LayerArgs la = layer_args(p, l, true);
         float* out = l == 0 ? g : nxt;
         const int ldo = p.ld[l];
@@ -512,7 +497,6 @@ cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* t
         if (e != cudaSuccess) return e;
         float* t = cur; cur = out; nxt = t;
     }
-    if (ab1) *ab1 = cur;
     return cudaGetLastError();
 }
 

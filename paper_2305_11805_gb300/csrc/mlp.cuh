@@ -74,10 +74,9 @@ cudaError_t launch_gemm_x3(dim3 grid, cudaStream_t s, const LayerArgs& la, const
 cudaError_t mlp_tiles(const MlpPlan& p, const int32_t* seg_off, int32_t* tile_start, cudaStream_t s, int* launches);
 cudaError_t mlp_forward(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, cudaStream_t s, int* launches);
 cudaError_t mlp_energy_rows(const MlpPlan& p, const MlpBuffers& b, int64_t N, float* E_rows, cudaStream_t s, int* launches);
-// g = dE/dG; with ab1 != nullptr the chain stops at dE/dA_1 (row stride ld[1]), returned in *ab1;
-// seeded: b.Ab already holds the output seeds (rows, stride ld[L]) instead of dE/da_L = 1
+// g = dE/dG; seeded: b.Ab already holds the output seeds (rows, stride ld[L]) instead of dE/da_L = 1
 cudaError_t mlp_input_grad(const MlpPlan& p, const MlpBuffers& b, const float* theta, int64_t N, float* g,
-                           cudaStream_t s, int* launches, float** ab1 = nullptr, bool seeded = false);
+                           cudaStream_t s, int* launches, bool seeded = false);
 // Small batches (at most kSmallBatch rows, one output): forward pass, energies and, with g, the input
 // gradient in one launch (mlp_small.cu); keep: Z and A of every layer are written as mlp_forward does.
 // cudaErrorNotSupported for other batches and for networks too wide for its shared memory.

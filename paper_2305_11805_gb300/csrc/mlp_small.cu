@@ -33,25 +33,6 @@ struct NetDev {
     float* A[kMaxLayers + 1];
 };
 
-__device__ __forceinline__ float act_value(int t, float z)
-{
-    switch (t) {
-    case PANNA_ACT_GAUSSIAN: return __expf(-z * z);
-    case PANNA_ACT_RELU: return z > 0.f ? z : 0.f;
-    case PANNA_ACT_TANH: return tanhf(z);
-    default: return z;
-    }
-}
-__device__ __forceinline__ float act_slope(int t, float z)
-{
-    switch (t) {
-    case PANNA_ACT_GAUSSIAN: return -2.f * z * __expf(-z * z);
-    case PANNA_ACT_RELU: return z > 0.f ? 1.f : 0.f;
-    case PANNA_ACT_TANH: { const float h = tanhf(z); return 1.f - h * h; }
-    default: return 1.f;
-    }
-}
-
 // four consecutive values of a row of length n from index k on (0 past its end)
 __device__ __forceinline__ float4 load4(const float* __restrict__ p, int k, int n, bool vec)
 {
@@ -167,7 +148,7 @@ k_mlp_rows(NetDev p, const float* __restrict__ theta, const int32_t* __restrict_
             constexpr int share = 32 / (4 * R);
             const int e = lane / share, n = n0 + e / R, r = e % R;
             if (lane % share == 0 && n < N) {
-                const float zv = v + bias[n], av = act_value(at, zv);
+                const float zv = v + bias[n], av = act_f(at, zv);
                 z[r * ldz + n] = zv;
                 out[r * ldw + n] = av;
                 if (r < nr) {
@@ -193,7 +174,7 @@ k_mlp_rows(NetDev p, const float* __restrict__ theta, const int32_t* __restrict_
         const float* z = zs + zoff[p.L];
         const int ldz = pad4(p.ld[p.L]);
         for (int idx = tid; idx < N * R; idx += kRowThreads)
-            zb[idx] = idx / R == 0 ? act_slope(at, z[(idx % R) * ldz + idx / R]) : 0.f;
+            zb[idx] = idx / R == 0 ? act_d1(at, z[(idx % R) * ldz + idx / R]) : 0.f;
     }
     __syncthreads();
     for (int l = p.L - 1; l >= 0; --l) {
@@ -239,7 +220,7 @@ k_mlp_rows(NetDev p, const float* __restrict__ theta, const int32_t* __restrict_
                 if (kk >= K) continue;
                 float v = 0.f;
                 for (int q = 0; q < ns && q * nb < kRowWarps; ++q) v += slice[(size_t)((q * nb + b) * R + r) * 128 + c];
-                if (l > 0) zb[kk * R + r] = v * act_slope(at, z[r * ldz + kk]);
+                if (l > 0) zb[kk * R + r] = v * act_d1(at, z[r * ldz + kk]);
                 else if (r < nr) g[(size_t)(r0 + r) * p.ld[0] + kk] = v;
             }
             __syncthreads();

@@ -774,16 +774,6 @@ k_wgrad_reduce(LayerArgs la, const int32_t* __restrict__ seg_off, int chunk, int
     else dtheta[la.b_off[s] + m] = acc;
 }
 
-int sm_count()
-{
-    static int n = 0;
-    int dev = 0;
-    if (n == 0 && (cudaGetDevice(&dev) != cudaSuccess ||
-                   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
-        n = 152;
-    return n;
-}
-
 // How a layer's weight gradient is summed: on the CUDA cores when it is narrow (rows of its inputs and
 // adjoints in 48 KB of shared memory), else by k_gemm_x3 with as many items as fill the SMs once, no
 // shorter than 256 atoms (each leaves a part to add up).
