@@ -397,9 +397,10 @@ int mma_variant(const panna_ctx* c, const Work& w, int kind, bool acc)
         // One warp per atom: with less than an atom per warp scheduler an atom's chain of rounds is the time, and
         // a round of variant 2 is the shorter one.  512 atoms of one species, variants 5 and 2 (us): 18 neighbours
         // 12.3 and 12.3, 30: 18.4 and 16.4, 51: 37 and 31, 87: 84 and 68; 1,000 atoms, 87: 92 and 90; 4,096 atoms,
-        // 51: 84 and 103.  Four species: 18 neighbours 14 and 21, 87: 88 and 74.  The neighbours are not known
-        // here; a capacity past the initial one tells of more than 64.
-        if (w.N < kSplitAtoms / 2 && w.cap > 64) return 2;
+        // 51: 84 and 103.  Four species: 18 neighbours 14 and 21, 87: 88 and 74.  With an even number of chunks of
+        // eight sectors the matrix form's round serves two (512 atoms, 87 neighbours, 16 sectors 96 and 145, 24:
+        // 236 and 211).  The neighbours are not known here; a capacity past the initial one tells of more than 64.
+        if (w.N < kSplitAtoms / 2 && w.cap > 64 && (c->d.n_theta + 7) / 8 % 2 == 1) return 2;
         return 5;
     }
     if (w.N < kSplitAtoms && !acc) return -1;

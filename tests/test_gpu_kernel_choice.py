@@ -64,11 +64,11 @@ def test_adjoint_of_many_species(n_species, autotune, copies):
         assert err <= tol
 
 
-@pytest.mark.parametrize("rc,copies,variant", [(3.2, 1, 5), (5.6, 1, 2), (5.6, 3, 5)])
-def test_tangent_of_small_dense_batches(rc, copies, variant):
-    """216 atoms with 18 and 87 neighbours, and 648 with 87."""
+@pytest.mark.parametrize("rc,copies,n_theta,variant", [(3.2, 1, 8, 5), (5.6, 1, 8, 2), (5.6, 1, 16, 5), (5.6, 3, 8, 5)])
+def test_tangent_of_small_dense_batches(rc, copies, n_theta, variant):
+    """216 atoms with 18 and 87 neighbours, one and two chunks of sectors, and 648 with 87."""
     one, system = clusters_of(2, copies)
-    desc = W.descriptor_params(2, rc, 8, 8, 8)
+    desc = W.descriptor_params(2, rc, 8, n_theta, 8)
     torch, archs, theta, th, pot, sysd = setup(system, desc)
     f_ref = np.random.default_rng(3).normal(size=(216, 3)).astype(np.float32)
     ref = O.batch(one, desc, archs, theta.astype(np.float64), e_ref=np.zeros(1), f_ref=f_ref.astype(np.float64),
