@@ -232,11 +232,15 @@ panna_status panna_set_angular_precision(panna_ctx* ctx, int32_t mode);
  * Matrix forms: descriptor 5 (any descriptor of the modified term) and adjoint 6 (at most 16 sectors
  * and 8 shells): one warp per atom (below 1216 atoms with FP32 networks: 2 to 64 warps of a cluster),
  * the products over sectors and shells on the tensor cores from operands split into TF32 parts; sums in
- * a fixed order.  Where they apply, batches of at least 1216 atoms and all batches with FP32 networks
- * take them without measuring.  JVP 5: likewise (zeta >= 2, plain arithmetic), for batches of every size.  With FP32 networks (extended angular terms) the descriptor's
- * candidates are variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that
- * the matrix forms do not take use variant 2 (adjoint: 5; the descriptor with FP32 networks: 0) and
- * smaller ones variant 0 (several warps per atom).  knob "mlp_fp32" (PANNA_MLP_FP32 networks):
+ * a fixed order.  Batches of at least 1216 atoms and all batches with FP32 networks take them without
+ * measuring, except where they are not the fastest: the descriptor with BF16 networks and zeta < 16, the
+ * adjoint of five or more species (variants 5 and 6 are measured against each other).  JVP 5 (zeta >= 2 and
+ * ((sqrt(1 + eps_theta) - 1) / 2)^(zeta - 1) <= 2^-21, plain arithmetic): likewise, for batches of every size
+ * but those below 608 atoms with a neighbour capacity above 64 and an odd number of groups of 8 sectors,
+ * which take variant 2.  With FP32 networks (extended angular terms) the descriptor's candidates are
+ * variants 0, 1 and 5 only.  Without autotuning, batches of at least 1216 atoms that the matrix forms do not
+ * take use variant 2 (adjoint: 5; the descriptor with FP32 networks: 0) and smaller ones variant 0 (several
+ * warps per atom; the adjoint of FP32 networks with five or more species 6).  knob "mlp_fp32" (PANNA_MLP_FP32 networks):
  * a bit mask of the products that run on the tensor cores, from FP32 operands split into TF32 parts with
  * partial sums rounded to nearest in FP32 (more accurate than an FP32 dot product of the same length): 1 or
  * 4 = the layers' products of at least 128 summands (forward, input gradient, tangents; batches past the

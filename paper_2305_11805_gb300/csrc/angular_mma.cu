@@ -16,7 +16,7 @@
 // What bounds it (ncu, water box of 16,384 atoms): instruction issue, two-wide FP32 instructions taking
 // two dispatch cycles each, next to the shared-memory data path.  A round of 32 pairs takes about 214
 // warp instructions (fast descriptor) against 400 in the lane-per-pair kernel; mma.m16n8k8 with TF32
-// operands issues every 8 cycles per scheduler and stays below 20 % busy.  Pair buffers hold what a
+// operands issues every 8 cycles per scheduler and is 20 % busy.  Pair buffers hold what a
 // lane reads as 4-byte words because a load returns at most 128 bytes a cycle to the warp, also when
 // its lanes share addresses.
 //
@@ -28,6 +28,8 @@
 //   water box (16,384 atoms)           0.67 -> 0.59  1.26 -> 0.94   1.89 -> 1.16  1.57 -> 1.26
 //   FCC box (131,072 atoms)            1.66 -> 1.07  2.56 -> 1.66   4.47 -> 2.3   3.13 -> 2.14
 //   1024 molecules (17,396 atoms)      0.14 -> 0.07  0.125 -> 0.117 0.23 -> 0.10  0.145 -> 0.133
+// Below zeta = 16 (FP32 networks, 4,096 atoms, 47 neighbours): descriptor 172 (230 with fractional exponents) ->
+// 155 us, adjoint 150 -> 125.  The 16-sector descriptors of FP32 networks spill 32 and 40 bytes.
 //
 // FP32 accuracy on TF32 operands: every operand is split into hi + lo TF32 parts (hi its leading 11
 // bits, lo the exact rest), so products carry about 22 bits; the descriptor puts A_hi in rows 0..7

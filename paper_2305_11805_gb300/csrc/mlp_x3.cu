@@ -25,11 +25,11 @@
 // add up the finished accumulators and write out finished tiles.  Every wait is bounded: on time-out the CTA sets
 // PANNA_ERR_TIMEOUT, waits for what it issued, frees its TMEM and returns.
 // Bound: the waits between the roles (a step takes about 1,700 cycles, its MMAs 768, issue is 50 % busy; one
-// set of 16 warps for splitting and adding took 3,000).  Registers: none of the adders' sums may spill,
-// shared memory leaves the L1 no room for them.
-// Measured (17,396 rows, us; k_gemm -> here): K = 768, N = 128: 110 -> 50; K = 128, N = 32: 24 -> 16; input
-// gradient K = 128, N = 768: 121 -> 49; tangent K = 768 (before: a pass that split the operand, then TMA and
-// MMAs) 86 -> 52; weight gradient 768 x 128 (before: passes that transposed and split both operands) 163 -> 93.
+// set of 16 warps for splitting and adding took 3,000).  Registers: the adders' sums must not spill, shared
+// memory leaves the L1 no room for them (the forward product without 16-byte loads spills 12 bytes).
+// Measured (17,396 rows, us; k_gemm -> here): K = 768, N = 128: 110 -> 48; K = 128, N = 32: 24 -> 16; input
+// gradient K = 128, N = 768: 121 -> 48; tangent K = 768 (before: a pass that split the operand, then TMA and
+// MMAs) 86 -> 51; weight gradient 768 x 128 (before: passes that transposed and split both operands) 163 -> 91.
 #include <stdint.h>
 
 #include <algorithm>
