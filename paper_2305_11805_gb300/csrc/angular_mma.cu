@@ -233,7 +233,7 @@ template <bool FAST, int CM, int PW, bool TEAM>
 __global__ void __launch_bounds__((TEAM ? kTeamMax : kMW) * 32,
                                   TEAM ? 2 : FAST ? (CM == 1 ? 8 : 7) : (CM == 1 ? 6 : 5))
 k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __restrict__ out,
-           __nv_bfloat16* __restrict__ Gh, __nv_bfloat16* __restrict__ Gl)
+           __nv_bfloat16* __restrict__ Gh, __nv_bfloat16* __restrict__ Gl, int even)
 {
     extern __shared__ float4 sm4[];
     __shared__ int s_seg[TEAM ? kTeamMax : kMW][kMaxSpecies + 1];
@@ -278,8 +278,6 @@ k_desc_mma(DescDev d, Work w, const int32_t* __restrict__ row_map, float* __rest
     const int ncm = (d.n_theta + 7) / 8, ncn = (d.n_ang_r + 7) / 8;
     const int nbins = d.n_theta * d.n_ang_r;
     const float eta_rl = d.eta_rad * 1.4426950408889634f;   // exp(-eta x^2) = 2^(-eta_l x^2)
-    // bin pairs on 8-byte boundaries; FP32 rows may be the caller's own, which start at any float
-    const bool even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0 && (Gh || (reinterpret_cast<uintptr_t>(out) & 7) == 0);
     auto put = [&](size_t idx, float v) {
         if (Gh) {
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
@@ -657,7 +655,7 @@ k_jvp_mma(DescDev d, Work w, const float* __restrict__ u, float* __restrict__ ou
     const int ncm = (d.n_theta + 7) / 8, ncn = (d.n_ang_r + 7) / 8;
     const int nbins = d.n_theta * d.n_ang_r;
     const float r_c = d.rs_ang[d.n_ang_r / 2], s_eta = sqrtf(d.eta_ang * 1.4426950408889634f);
-    const float c_x = d.eta_ang > 0.f ? -2.f * d.eta_ang / s_eta : 0.f, eta_rl = d.eta_rad * 1.4426950408889634f;
+    const float c_x = -1.3862943611f * s_eta, eta_rl = d.eta_rad * 1.4426950408889634f;
     const bool even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0;
     for (int64_t i = (int64_t)blockIdx.x * kMW + warp; i < w.N; i += (int64_t)gridDim.x * kMW) {
         const int64_t row = w.row_of_atom[i];
@@ -904,7 +902,7 @@ k_adj_mma(DescDev d, Work w, const float* __restrict__ g_rows, float* __restrict
         }
     }
     // dT/dr = s1 Fp S1 + ...: x e in the units of nR0
-    const float s1 = FAST && d.eta_ang > 0.f ? -2.f * d.eta_ang / s_eta : -2.f * d.eta_ang;
+    const float s1 = FAST ? -1.3862943611f * s_eta : -2.f * d.eta_ang;   // -2 eta / s_eta, s_eta^2 = eta log2(e)
     const bool gvec = (d.D & 3) == 0 && (reinterpret_cast<uintptr_t>(g_rows) & 15) == 0;
 
     for (int64_t i = TEAM ? blockIdx.x / ctas : (int64_t)blockIdx.x * kMW + warp; i < w.N;
@@ -1327,16 +1325,18 @@ cudaError_t launch_desc_mma(const Work& w, const DescDev& d, const int32_t* row_
     if (w.N == 0) return cudaSuccess;
     const bool two = ((d.n_theta + 7) / 8) % 2 == 0;
     const int pw = log_terms(d, d.zeta);
+    // pairs of bins on 8-byte boundaries; FP32 rows may be the caller's own, which start at any float
+    const int even = ((d.D | d.rad_cols | d.n_ang_r) & 1) == 0 && (Gh || (reinterpret_cast<uintptr_t>(G_rows) & 7) == 0);
     const Team tm = team_of(w, desc_fast(d, fast));
     if (tm.warps > 1) {
         const size_t smem = desc_mma_atom_bytes<false>(w.cap) + tm.warps * desc_mma_warp_bytes<false>(two ? 2 : 1);
-        auto run = [&](auto kern) { return launch_team(kern, w.N, tm, smem, s, d, w, row_map, G_rows, Gh, Gl); };
+        auto run = [&](auto kern) { return launch_team(kern, w.N, tm, smem, s, d, w, row_map, G_rows, Gh, Gl, even); };
         if (pw == 8) return two ? run(k_desc_mma<false, 2, 8, true>) : run(k_desc_mma<false, 1, 8, true>);
         if (pw == 13) return two ? run(k_desc_mma<false, 2, 13, true>) : run(k_desc_mma<false, 1, 13, true>);
         return two ? run(k_desc_mma<false, 2, 0, true>) : run(k_desc_mma<false, 1, 0, true>);
     }
     const size_t smem = desc_smem(w, d, fast);
-    auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, row_map, G_rows, Gh, Gl); };
+    auto run = [&](auto kern) { return launch_resident(kern, w.N, smem, s, d, w, row_map, G_rows, Gh, Gl, even); };
     if (desc_fast(d, fast)) return two ? run(k_desc_mma<true, 2, 0, false>) : run(k_desc_mma<true, 1, 0, false>);
     if (pw == 8) return two ? run(k_desc_mma<false, 2, 8, false>) : run(k_desc_mma<false, 1, 8, false>);
     if (pw == 13) return two ? run(k_desc_mma<false, 2, 13, false>) : run(k_desc_mma<false, 1, 13, false>);
